@@ -460,11 +460,21 @@ ps_status ps_wait_selftest(int* d_status, long long polls, ps_stream stream);
 /* ---- Seed-proposal network (not part of the paper: a learned initialiser of
    the planes of Sec. 3.1).  Four 3x3 stride-2 convolutions (64 channels, ReLU),
    global average pooling and a 64 -> 96 linear layer map a 64x64 patch of depth
-   and camera-frame normals to 8 plane seeds.  Convolutions are im2col +
+   and camera-frame normals to 8 plane seeds.  Convolutions run as
+   implicit GEMMs on the tensor cores (ps_seed_conv_fwd), or as im2col +
    ps_gemm_bf16.  Activations NHWC bf16; gradients fp32; the im2col column
    order is (ky, kx, c) zero-padded to Kp (a multiple of 64).  All pointers are
    device pointers; every call is asynchronous on the stream. ---- */
 
+/* One convolution layer, y = relu(bias + conv(x)): x [B, side, side, C] and y
+   [B, side/2, side/2, 64] bf16, w [64, Kp] bf16 (Kp = 64 for C = 4, 576 for C = 64,
+   column order as im2col's), bias [64] fp32.  (side, C) is (64, 4), (32, 64), (16, 64)
+   or (8, 64); B (side/2)^2 must be a multiple of 128.  w, y and x_copy 16-byte aligned.
+   x_copy (first layer only, or NULL) receives a copy of x.  x may have any alignment
+   if x_copy is given, else 16 bytes.  Equal to ps_seed_im2col + ps_gemm_bf16 (bias,
+   ReLU, bf16 output) bit for bit, without the im2col matrix.  d_err as in ps_gemm_bf16. */
+ps_status ps_seed_conv_fwd(const void* x, int B, int side, int C, const void* w, const float* bias,
+                           void* y, void* x_copy, int* d_err, ps_stream stream);
 /* A[B*Ho*Wo, Kp] (bf16) = im2col of x[B, H, W, C] (bf16) for a 3x3 window,
    stride 2, padding 1; Ho = ceil(H/2), Wo = ceil(W/2). */
 ps_status ps_seed_im2col(const void* x, int B, int H, int W, int C, int Kp, void* A,

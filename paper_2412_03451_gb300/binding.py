@@ -26,7 +26,7 @@ EXPORTS = ("ps_plan_views", "ps_project_cull", "ps_bin_workspace_bytes", "ps_bin
            "ps_fwd_workspace_bytes", "ps_splat_fwd", "ps_splat_ids", "ps_loss", "ps_bwd_workspace_bytes", "ps_splat_bwd",
            "ps_splat_fused", "ps_adam_step",
            "ps_count_pairs", "ps_step_advance", "ps_adam_step_state", "ps_gemm_bf16", "ps_wait_selftest",
-           "ps_seed_im2col", "ps_seed_col2im", "ps_seed_relu_bwd", "ps_seed_transpose",
+           "ps_seed_conv_fwd", "ps_seed_im2col", "ps_seed_col2im", "ps_seed_relu_bwd", "ps_seed_transpose",
            "ps_seed_colsum", "ps_seed_pool", "ps_seed_pool_bwd", "ps_seed_loss", "ps_cast_bf16",
            "ps_radii_grad_accum", "ps_split_planes", "ps_merge_planes", "ps_status_string",
            "ps_version", "ps_lambda_schedule", "ps_filter_margin", "ps_gauss_extent",
@@ -108,6 +108,7 @@ def load():
             "ps_step_advance": ([P, P, I, P, P], I),
             "ps_gemm_bf16": ([P, P, P, P, P, I, I, I, I, I, I, P, P], I),
             "ps_wait_selftest": ([P, LL, P], I),
+            "ps_seed_conv_fwd": ([P, I, I, I, P, P, P, P, P, P], I),
             "ps_seed_im2col": ([P, I, I, I, I, I, P, P], I),
             "ps_seed_col2im": ([P, I, I, I, I, I, P, P], I),
             "ps_seed_relu_bwd": ([P, P, LL, F, P, P, P], I),
@@ -383,6 +384,12 @@ def ps_gemm_bf16(A, B, bias, C32, C16, relu=False, accumulate=False, err=None, s
     _check(load().ps_gemm_bf16(_ptr(A), _ptr(B), _ptr(bias), _ptr(C32), _ptr(C16), int(M), int(N),
                                int(K), int(C.stride(0)), int(bool(relu)), int(bool(accumulate)),
                                _ptr(err), _stream(stream)), "ps_gemm_bf16")
+
+
+def ps_seed_conv_fwd(x, B, side, C, w, bias, y, x_copy=None, err=None, stream=None):
+    """y = relu(bias + conv3x3 stride 2 of x): an implicit GEMM on the tensor cores (see ps.h)."""
+    _check(load().ps_seed_conv_fwd(_ptr(x), int(B), int(side), int(C), _ptr(w), _ptr(bias), _ptr(y),
+                                   _ptr(x_copy), _ptr(err), _stream(stream)), "ps_seed_conv_fwd")
 
 
 def ps_seed_im2col(x, B, H, W, C, Kp, A, stream=None):

@@ -21,11 +21,7 @@
 // Every mbarrier wait is bounded: on time-out the kernel sets an error flag,
 // waits (bounded) for the copies and MMAs it issued, frees its tensor memory
 // and returns.
-#include <stdint.h>
-#include <cuda.h>
-#include <cuda_bf16.h>
-
-#include "ps_internal.cuh"
+#include "ps_tc.cuh"
 
 using namespace ps;
 
@@ -34,7 +30,6 @@ namespace {
 constexpr int BM = 128, BN = 64, BK = 64;
 constexpr int kThreads = 128;
 constexpr unsigned kTmemCols = 64;           // FP32 accumulator columns (= BN)
-constexpr long long kWaitPolls = 1LL << 24;  // bounded mbarrier wait
 #ifndef PS_GEMM_STAGES
 #define PS_GEMM_STAGES 2
 #endif
@@ -42,48 +37,6 @@ constexpr int kStages = PS_GEMM_STAGES;
 constexpr int kABytes = BM * BK * 2, kBBytes = BN * BK * 2;   // multiples of the 1024-byte atom
 constexpr int kStageBytes = kABytes + kBBytes;
 static_assert(kStages >= 2 && kStages * kStageBytes >= BM * (BN + 1) * 4, "epilogue tile fits the stages");
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-// Shared-memory matrix descriptor, K-major with 128-byte swizzle: start address,
-// leading byte offset (unused by this layout when one MMA's K fits an atom row;
-// 16 bytes), stride byte offset 1024 (between 8-row atoms along M/N), descriptor
-// version 1, base offset 0 (atoms 1024-byte aligned), layout type 2 (SWIZZLE_128B).
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr)
-{
-    uint64_t d = 0;
-    d |= (uint64_t)((addr >> 4) & 0x3FFFu);
-    d |= (uint64_t)(16u >> 4) << 16;
-    d |= (uint64_t)(1024u >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-
-// Instruction descriptor of kind::f16: D f32, A and B bf16, both K-major, N, M.
-__host__ __device__ constexpr uint32_t instr_desc(int M, int N)
-{
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase, long long polls = kWaitPolls)
-{
-    for (long long i = 0; i < polls; ++i) {
-        uint32_t done = 0;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(bar), "r"(phase)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
 
 struct GemmArgs {
     const float* bias;        // [N] or null
@@ -100,19 +53,9 @@ struct GemmArgs {
 __device__ __forceinline__ void issue_slice(const CUtensorMap* tmA, const CUtensorMap* tmB, uint32_t sa,
                                             uint32_t sb, uint32_t full, int j, int m0, int n0)
 {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                 :: "r"(full), "r"(kStageBytes) : "memory");
-    const int x = j * BK;
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3}], [%4];"
-        :: "r"(sa), "l"(reinterpret_cast<uint64_t>(tmA)), "r"(x), "r"(m0), "r"(full)
-        : "memory");
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3}], [%4];"
-        :: "r"(sb), "l"(reinterpret_cast<uint64_t>(tmB)), "r"(x), "r"(n0), "r"(full)
-        : "memory");
+    mbar_expect(full, kStageBytes);
+    tma_load_2d(sa, tmA, j * BK, m0, full);
+    tma_load_2d(sb, tmB, j * BK, n0, full);
 }
 
 __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__ CUtensorMap tmA,
@@ -128,23 +71,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
     const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
     const uint32_t base = (smem_u32(s_dyn) + 1023u) & ~1023u;
 
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     :: "r"(smem_u32(&tmem_base)), "r"(kTmemCols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+    if (warp == 0) tmem_alloc(&tmem_base, kTmemCols);
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&full[s])) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&empty[s])) : "memory");
+            mbar_init(smem_u32(&full[s]), 1);
+            mbar_init(smem_u32(&empty[s]), 1);
         }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_init_fence();
         failed = 0;
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tc_fence_before();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tc_fence_after();
     const uint32_t tmem = tmem_base;
     const int nk = a.K / BK;
     int issued = 0, consumed = 0, committed = 0;    // slices, per thread 0
@@ -165,23 +103,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
                 break;
             }
             consumed = kt + 1;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            tc_fence_after();
             const uint32_t sa = base + (uint32_t)s * kStageBytes, sb = sa + kABytes;
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk) {
                 // K = 16 is 32 bytes of every 128-byte row of the swizzle atoms
-                const uint64_t da = smem_desc_sw128(sa + kk * 32);
-                const uint64_t db = smem_desc_sw128(sb + kk * 32);
-                const uint32_t acc = (kt > 0 || kk > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n\t.reg .pred p;\n\t"
-                    "setp.ne.b32 p, %4, 0;\n\t"
-                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                    :: "r"(tmem), "l"(da), "l"(db), "r"(idesc), "r"(acc)
-                    : "memory");
+                mma_bf16(tmem, smem_desc_k(sa + kk * 32), smem_desc_k(sb + kk * 32), idesc,
+                         (kt > 0 || kk > 0) ? 1u : 0u);
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                         :: "r"(smem_u32(&empty[s])) : "memory");
+            mma_commit(smem_u32(&empty[s]));
             committed = kt + 1;
             // refill the previous slice's stage (its MMAs were committed one slice ago)
             // with the slice kStages after it
@@ -212,9 +142,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
                           (uint32_t)(((committed - 1) / kStages) & 1));
         }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tc_fence_before();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tc_fence_after();
 
     if (!failed && nk > 0) {
         // epilogue: warp w reads accumulator lanes (rows) 32w .. 32w + 31 and parks them, with
@@ -224,21 +154,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
         float* tile = reinterpret_cast<float*>(s_dyn + (base - smem_u32(s_dyn)));
         const int rl = warp * 32 + lane;
 #pragma unroll
-        for (int c0 = 0; c0 < BN; c0 += 16) {
-            uint32_t r[16];
-            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
-                  "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
-                  "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                : "r"(taddr));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        for (int c0 = 0; c0 < BN; c0 += 32) {
+            float r[32];
+            tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, r);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
+            for (int j = 0; j < 32; ++j) {
                 const int col = n0 + c0 + j;
-                float x = __uint_as_float(r[j]);
+                float x = r[j];
                 if (a.bias && col < a.N) x += a.bias[col];
                 if (a.relu) x = fmaxf(x, 0.f);
                 tile[rl * (BN + 1) + c0 + j] = x;
@@ -256,11 +178,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
             }
         }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tc_fence_before();
     __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
-                     :: "r"(tmem), "r"(kTmemCols) : "memory");
+    if (warp == 0) tmem_free(tmem, kTmemCols);
 }
 
 // The time-out path of mbar_wait on a barrier that nothing arrives on: one
@@ -272,7 +192,7 @@ __global__ void k_wait_selftest(int* status, long long polls)
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x != 0) return;
     const uint32_t b = smem_u32(&bar);
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(b) : "memory");
+    mbar_init(b, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (!mbar_wait(b, 0u, polls)) atomicOr(status, 1 << PS_ERR_TIMEOUT);
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];" :: "r"(b) : "memory");
@@ -296,22 +216,27 @@ EncodeTiled encoder()
     return fn;
 }
 
-// 2D map of a row-major bf16 matrix [rows][K], boxes of 64 columns (128 bytes) x
-// box_rows rows, written to shared memory with the 128-byte swizzle
+// 2D map of a row-major bf16 matrix [rows][K], boxes of 64 columns (128 bytes) x box_rows rows
 bool make_map(CUtensorMap* m, const void* ptr, int rows, int K, int box_rows)
 {
-    EncodeTiled enc = encoder();
-    if (!enc) return false;
     const cuuint64_t dim[2] = {(cuuint64_t)K, (cuuint64_t)rows};
     const cuuint64_t stride[1] = {(cuuint64_t)K * 2};
     const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dim, stride, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    const cuuint32_t step[2] = {1, 1};
+    return encode_map(m, ptr, 2, dim, stride, box, step);
 }
 
 }  // namespace
+
+bool ps::encode_map(CUtensorMap* m, const void* ptr, int rank, const cuuint64_t* dim, const cuuint64_t* stride,
+                    const cuuint32_t* box, const cuuint32_t* step)
+{
+    EncodeTiled enc = encoder();
+    if (!enc) return false;
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(ptr), dim, stride, box, step,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 extern "C" ps_status ps_gemm_bf16(const void* A, const void* B, const float* bias, float* C32,
                                   void* C16, int M, int N, int K, int ldc, int relu,

@@ -8,8 +8,9 @@ the splatting method itself.
 
 Architecture: conv 3x3 stride 2 (4 -> 64) -> ReLU -> 3 x [conv 3x3 stride 2
 (64 -> 64) -> ReLU] -> global average pool -> linear 64 -> 96.  Every
-convolution is im2col + a tcgen05 BF16 GEMM with FP32 accumulation (libps);
-the backward pass is the same kernels run on transposed operands.  Parameters
+convolution is an implicit GEMM on the tensor cores (tcgen05, BF16 with FP32
+accumulation, libps); the backward pass runs im2col and the library's GEMM on
+transposed operands.  Parameters
 are FP32 masters (Adam in libps) with BF16 copies for the tensor cores.
 
 Output slot j of a patch (12 floats): centre (u, v in [-1, 1] patch
@@ -93,10 +94,10 @@ class SeedNet:
         assert Bn % 64 == 0, "batch must be a multiple of 64"
         dev, bf = self.device, torch.bfloat16
         self.B = Bn
-        self.A, self.Y = [], []
+        self.X = torch.empty((Bn, PATCH, PATCH, IN_C), dtype=bf, device=dev)   # the input, for the backward
+        self.Y = []
         for (h, cin, kp) in LAYERS:
             ho = h // 2
-            self.A.append(torch.empty((Bn * ho * ho, kp), dtype=bf, device=dev))
             self.Y.append(torch.empty((Bn * ho * ho, CH), dtype=bf, device=dev))
         self.h32 = torch.empty((Bn, CH), device=dev)
         self.h16 = torch.empty((Bn, CH), dtype=bf, device=dev)
@@ -115,11 +116,10 @@ class SeedNet:
         """x16: [B, 64, 64, 4] bf16 (NHWC).  Returns out [B, 96] fp32."""
         Bn = x16.shape[0]
         self._alloc(Bn)
-        self.x16 = x16
         inp = x16
         for i, (h, cin, kp) in enumerate(LAYERS):
-            B.ps_seed_im2col(inp, Bn, h, h, cin, kp, self.A[i])
-            B.ps_gemm_bf16(self.A[i], self._bf16[i], self.b[i], None, self.Y[i], relu=True, err=self.err)
+            B.ps_seed_conv_fwd(inp, Bn, h, cin, self._bf16[i], self.b[i], self.Y[i],
+                               x_copy=self.X if i == 0 else None, err=self.err)
             inp = self.Y[i]
         B.ps_seed_pool(self.Y[3], Bn, 16, CH, self.h32, self.h16)
         B.ps_gemm_bf16(self.h16, self._bf16[4], self.b[4], self.out, None, err=self.err)
@@ -154,8 +154,10 @@ class SeedNet:
             B.ps_seed_relu_bwd(dy, self.Y[i], 1.0, dz16, dz32)
             dzT = torch.empty((CH, P), dtype=bf, device=dev)
             AT = torch.empty((kp, P), dtype=bf, device=dev)
+            A = torch.empty((P, kp), dtype=bf, device=dev)
+            B.ps_seed_im2col(self.Y[i - 1] if i > 0 else self.X, Bn, h, h, cin, kp, A)
             B.ps_seed_transpose(dz16, dzT)
-            B.ps_seed_transpose(self.A[i], AT)
+            B.ps_seed_transpose(A, AT)
             gWp = torch.empty((CH, kp), dtype=f32, device=dev)
             B.ps_gemm_bf16(dzT, AT, None, gWp, None, err=self.err)
             self.gW[i].copy_(gWp[:, :9 * cin])

@@ -475,6 +475,21 @@ ps_status ps_wait_selftest(int* d_status, long long polls, ps_stream stream);
    ReLU, bf16 output) bit for bit, without the im2col matrix.  d_err as in ps_gemm_bf16. */
 ps_status ps_seed_conv_fwd(const void* x, int B, int side, int C, const void* w, const float* bias,
                            void* y, void* x_copy, int* d_err, ps_stream stream);
+/* The network's whole backward: the gradient of sum(dout * out) with respect to every
+   parameter, into grad (overwritten).  params, grad: the flat FP32 parameters [W (64 x
+   9 Cin), b (64)] of the four convolutions, then [W (96 x 64), b (96)].  w16: the four
+   convolutions' bf16 weights as in ps_seed_conv_fwd; x [B, 64, 64, 4]; y: the four
+   convolutions' outputs; h16 [B, 64] the pooled activations, of the forward of this
+   batch (host arrays of device pointers).  dout [B, 96] fp32.  B a multiple of 64.  ws
+   (device, 256-byte aligned, >= ps_seed_backward_ws_bytes(B)) is scratch; the other
+   arrays 16-byte aligned.  Matrix products take bf16 operands and FP32 sums. */
+size_t ps_seed_backward_ws_bytes(int B);
+ps_status ps_seed_backward(const float* params, const void* const* w16, const void* x,
+                           const void* const* y, const void* h16, const float* dout, int B,
+                           float* grad, void* ws, size_t ws_bytes, int* d_err, ps_stream stream);
+/* bf16 copies of the five weight blocks of params (flat, as above) into w16 (host array
+   of device pointers): [64][64] (36 columns, zero-padded), 3 x [64][576], [96][64]. */
+ps_status ps_seed_sync_weights(const float* params, void* const* w16, ps_stream stream);
 /* A[B*Ho*Wo, Kp] (bf16) = im2col of x[B, H, W, C] (bf16) for a 3x3 window,
    stride 2, padding 1; Ho = ceil(H/2), Wo = ceil(W/2). */
 ps_status ps_seed_im2col(const void* x, int B, int H, int W, int C, int Kp, void* A,

@@ -26,7 +26,8 @@ EXPORTS = ("ps_plan_views", "ps_project_cull", "ps_bin_workspace_bytes", "ps_bin
            "ps_fwd_workspace_bytes", "ps_splat_fwd", "ps_splat_ids", "ps_loss", "ps_bwd_workspace_bytes", "ps_splat_bwd",
            "ps_splat_fused", "ps_adam_step",
            "ps_count_pairs", "ps_step_advance", "ps_adam_step_state", "ps_gemm_bf16", "ps_wait_selftest",
-           "ps_seed_conv_fwd", "ps_seed_im2col", "ps_seed_col2im", "ps_seed_relu_bwd", "ps_seed_transpose",
+           "ps_seed_conv_fwd", "ps_seed_backward_ws_bytes", "ps_seed_backward",
+           "ps_seed_sync_weights", "ps_seed_im2col", "ps_seed_col2im", "ps_seed_relu_bwd", "ps_seed_transpose",
            "ps_seed_colsum", "ps_seed_pool", "ps_seed_pool_bwd", "ps_seed_loss", "ps_cast_bf16",
            "ps_radii_grad_accum", "ps_split_planes", "ps_merge_planes", "ps_status_string",
            "ps_version", "ps_lambda_schedule", "ps_filter_margin", "ps_gauss_extent",
@@ -109,6 +110,9 @@ def load():
             "ps_gemm_bf16": ([P, P, P, P, P, I, I, I, I, I, I, P, P], I),
             "ps_wait_selftest": ([P, LL, P], I),
             "ps_seed_conv_fwd": ([P, I, I, I, P, P, P, P, P, P], I),
+            "ps_seed_backward_ws_bytes": ([I], SZ),
+            "ps_seed_backward": ([P, P, P, P, P, P, I, P, P, SZ, P, P], I),
+            "ps_seed_sync_weights": ([P, P, P], I),
             "ps_seed_im2col": ([P, I, I, I, I, I, P, P], I),
             "ps_seed_col2im": ([P, I, I, I, I, I, P, P], I),
             "ps_seed_relu_bwd": ([P, P, LL, F, P, P, P], I),
@@ -390,6 +394,26 @@ def ps_seed_conv_fwd(x, B, side, C, w, bias, y, x_copy=None, err=None, stream=No
     """y = relu(bias + conv3x3 stride 2 of x): an implicit GEMM on the tensor cores (see ps.h)."""
     _check(load().ps_seed_conv_fwd(_ptr(x), int(B), int(side), int(C), _ptr(w), _ptr(bias), _ptr(y),
                                    _ptr(x_copy), _ptr(err), _stream(stream)), "ps_seed_conv_fwd")
+
+
+def _ptrs(tensors):
+    return (ctypes.c_void_p * len(tensors))(*[t.data_ptr() for t in tensors])
+
+
+def ps_seed_backward_ws_bytes(B: int) -> int:
+    return int(load().ps_seed_backward_ws_bytes(int(B)))
+
+
+def ps_seed_backward(params, w16, x, y, h16, dout, B, grad, ws, err=None, stream=None):
+    """The seed network's backward into grad (see ps.h); w16 and y are lists of tensors."""
+    _check(load().ps_seed_backward(_ptr(params), _ptrs(w16), _ptr(x), _ptrs(y), _ptr(h16), _ptr(dout), int(B),
+                                   _ptr(grad), _ptr(ws), ws.numel() * ws.element_size(), _ptr(err),
+                                   _stream(stream)), "ps_seed_backward")
+
+
+def ps_seed_sync_weights(params, w16, stream=None):
+    """bf16 copies of the five weight blocks of the flat parameters."""
+    _check(load().ps_seed_sync_weights(_ptr(params), _ptrs(w16), _stream(stream)), "ps_seed_sync_weights")
 
 
 def ps_seed_im2col(x, B, H, W, C, Kp, A, stream=None):

@@ -222,15 +222,15 @@ bool make_map(CUtensorMap* m, const void* ptr, int rows, int K, int box_rows)
     const cuuint64_t dim[2] = {(cuuint64_t)K, (cuuint64_t)rows};
     const cuuint64_t stride[1] = {(cuuint64_t)K * 2};
     const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
-    const cuuint32_t step[2] = {1, 1};
-    return encode_map(m, ptr, 2, dim, stride, box, step);
+    return encode_map(m, ptr, 2, dim, stride, box);
 }
 
 }  // namespace
 
 bool ps::encode_map(CUtensorMap* m, const void* ptr, int rank, const cuuint64_t* dim, const cuuint64_t* stride,
-                    const cuuint32_t* box, const cuuint32_t* step)
+                    const cuuint32_t* box)
 {
+    const cuuint32_t step[5] = {1, 1, 1, 1, 1};
     EncodeTiled enc = encoder();
     if (!enc) return false;
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(ptr), dim, stride, box, step,

@@ -64,6 +64,16 @@ __device__ __forceinline__ void fence_async_smem()
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// One thread of a converged warp.  The warp's loops around it stay uniform, so that an
+// MMA's descriptors live in uniform registers: an M 64, N 8 step issues every 26 cycles
+// this way and every 45-49 from a branch taken by one thread.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // whole warp; cols a power of two >= 32
 __device__ __forceinline__ void tmem_alloc(uint32_t* base, uint32_t cols)
 {
@@ -98,6 +108,13 @@ __device__ __forceinline__ uint64_t smem_desc_k(uint32_t addr) { return smem_des
 __device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr, uint32_t mn_stride)
 {
     return smem_desc(addr, mn_stride, 1024);
+}
+
+// MN-major without swizzle: blocks of 8 M (N) indices x K rows of 16 bytes, blocks
+// `block` bytes apart, groups of 8 K rows 128 bytes apart (layout type 0).
+__device__ __forceinline__ uint64_t smem_desc_blocks(uint32_t addr, uint32_t block)
+{
+    return smem_desc(addr, 128, block) & ~((uint64_t)7 << 61);
 }
 
 // Instruction descriptor of kind::f16: D f32, A and B bf16, N, M; ta / tb: the
@@ -142,6 +159,12 @@ __device__ __forceinline__ void tmem_ld32(uint32_t addr, float (&v)[32])
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// bytes a multiple of 16, both addresses 16-byte aligned
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 :: "r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t bar)
 {
     asm volatile(
@@ -159,6 +182,15 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm,
         :: "r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
         : "memory");
 }
+__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, int w, int v,
+                                            uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
+        :: "r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(v), "r"(bar)
+        : "memory");
+}
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, uint32_t src, int x, int y)
 {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
@@ -170,11 +202,10 @@ __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.w
 template <int N>
 __device__ __forceinline__ void bulk_wait() { asm volatile("cp.async.bulk.wait_group %0;" :: "n"(N) : "memory"); }
 
-// Host: encodes a tensor map of a bf16 array (innermost dimension first, rows of
-// dim[0] contiguous elements; stride[i] bytes between elements of dimension
-// i + 1), boxes written to shared memory with the 128-byte swizzle.  step: element
-// step of each dimension (1: dense), box the extent stepped over.
+// Host: encodes a tensor map of a bf16 array (rank <= 5, innermost dimension first,
+// rows of dim[0] contiguous elements; stride[i] bytes between elements of dimension
+// i + 1), boxes written to shared memory with the 128-byte swizzle.
 bool encode_map(CUtensorMap* m, const void* ptr, int rank, const cuuint64_t* dim, const cuuint64_t* stride,
-                const cuuint32_t* box, const cuuint32_t* step);
+                const cuuint32_t* box);
 
 }  // namespace ps

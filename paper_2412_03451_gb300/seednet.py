@@ -9,9 +9,8 @@ the splatting method itself.
 Architecture: conv 3x3 stride 2 (4 -> 64) -> ReLU -> 3 x [conv 3x3 stride 2
 (64 -> 64) -> ReLU] -> global average pool -> linear 64 -> 96.  Every
 convolution is an implicit GEMM on the tensor cores (tcgen05, BF16 with FP32
-accumulation, libps); the backward pass runs im2col and the library's GEMM on
-transposed operands.  Parameters
-are FP32 masters (Adam in libps) with BF16 copies for the tensor cores.
+accumulation, libps); so are the input and weight gradients of the backward
+pass.  Parameters are FP32 masters (Adam in libps) with BF16 copies for the tensor cores.
 
 Output slot j of a patch (12 floats): centre (u, v in [-1, 1] patch
 coordinates, log(z / z_ref)), quaternion of the plane frame in camera
@@ -104,12 +103,11 @@ class SeedNet:
         self.out = torch.empty((Bn, OUT), device=dev)
         self.dout = torch.empty((Bn, OUT), device=dev)
         self.loss_sums = torch.zeros(4, device=dev)
+        self.bwd_ws = None            # the backward's scratch, once it is needed
 
     def sync_weights(self):
         """BF16 copies of the FP32 master weights (zero-padded to the GEMM K)."""
-        for i, (_, cin, kp) in enumerate(LAYERS):
-            B.ps_cast_bf16(self.W[i], self._bf16[i])
-        B.ps_cast_bf16(self.W[4], self._bf16[4])
+        B.ps_seed_sync_weights(self.params, self._bf16)
 
     # -- forward -------------------------------------------------------------
     def forward(self, x16: torch.Tensor) -> torch.Tensor:
@@ -128,48 +126,14 @@ class SeedNet:
     # -- backward ------------------------------------------------------------
     def backward(self, dout: torch.Tensor):
         """Gradient of sum(dout * out) w.r.t. every parameter, into self.grad."""
-        Bn, dev, bf = self.B, self.device, torch.bfloat16
-        f32 = torch.float32
-        # linear layer
-        doutT = torch.empty((OUT, Bn), dtype=bf, device=dev)
-        hT = torch.empty((CH, Bn), dtype=bf, device=dev)
-        B.ps_seed_transpose(dout, doutT)
-        B.ps_seed_transpose(self.h16, hT)
-        B.ps_gemm_bf16(doutT, hT, None, self.gW[4], None, err=self.err)
-        B.ps_seed_colsum(dout, self.gb[4])
-        dout16 = torch.empty((Bn, 128), dtype=bf, device=dev)
-        B.ps_cast_bf16(dout, dout16)
-        WfcT = torch.empty((CH, 128), dtype=bf, device=dev)
-        B.ps_seed_transpose(self.W[4], WfcT)
-        dh = torch.empty((Bn, CH), dtype=f32, device=dev)
-        B.ps_gemm_bf16(dout16, WfcT, None, dh, None, err=self.err)
-        # pooling + ReLU of the last convolution
-        dy = torch.empty((Bn * 16, CH), dtype=f32, device=dev)
-        B.ps_seed_pool_bwd(dh, Bn, 16, CH, dy)
-        for i in range(3, -1, -1):
-            h, cin, kp = LAYERS[i]
-            P = self.Y[i].shape[0]
-            dz16 = torch.empty((P, CH), dtype=bf, device=dev)
-            dz32 = torch.empty((P, CH), dtype=f32, device=dev)
-            B.ps_seed_relu_bwd(dy, self.Y[i], 1.0, dz16, dz32)
-            dzT = torch.empty((CH, P), dtype=bf, device=dev)
-            AT = torch.empty((kp, P), dtype=bf, device=dev)
-            A = torch.empty((P, kp), dtype=bf, device=dev)
-            B.ps_seed_im2col(self.Y[i - 1] if i > 0 else self.X, Bn, h, h, cin, kp, A)
-            B.ps_seed_transpose(dz16, dzT)
-            B.ps_seed_transpose(A, AT)
-            gWp = torch.empty((CH, kp), dtype=f32, device=dev)
-            B.ps_gemm_bf16(dzT, AT, None, gWp, None, err=self.err)
-            self.gW[i].copy_(gWp[:, :9 * cin])
-            B.ps_seed_colsum(dz32, self.gb[i])
-            if i > 0:
-                WT = torch.empty((kp, CH), dtype=bf, device=dev)
-                B.ps_seed_transpose(self._bf16[i], WT)
-                dA = torch.empty((P, kp), dtype=f32, device=dev)
-                B.ps_gemm_bf16(dz16, WT, None, dA, None, err=self.err)
-                hp = LAYERS[i - 1][0] // 2
-                dy = torch.empty((Bn * hp * hp, CH), dtype=f32, device=dev)
-                B.ps_seed_col2im(dA, Bn, h, h, cin, kp, dy)
+        if self.bwd_ws is None:
+            n = B.ps_seed_backward_ws_bytes(self.B)
+            self.bwd_ws = torch.empty((n + 255) // 256 * 64, dtype=torch.float32, device=self.device)
+        d = dout.contiguous()
+        if d.data_ptr() % 16:
+            d = d.clone()
+        B.ps_seed_backward(self.params, self._bf16[:4], self.X, self.Y, self.h16, d, self.B,
+                           self.grad, self.bwd_ws, err=self.err)
 
     def loss_backward(self, tgt: torch.Tensor):
         """Set loss of the current outputs against tgt [B, 8, 12]; fills dout and

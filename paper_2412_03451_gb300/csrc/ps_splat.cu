@@ -28,13 +28,21 @@
 //   A_j = w_j t_j + (1 - w_j) A_{j+1},  dD/dw_j = T_j (t_j - A_{j+1}),
 //   dD/dt_j = T_j w_j,  dN/dn_j = T_j w_j,  and the same for N with n_j,
 // so nothing is divided by 1 - w_j.  Each pair's gradient is chained through
-// Eq. 9, 7-8, 6 and 4 into 16 record floats (the gradients of n_c, v^x_c, v^y_c
-// at a fixed plane centre, of s, a_x, a_y and of the radii; the first three use
-// the intersection relative to the centre, t d - p_c = P_X v^x + P_Y v^y, so no
-// metre-sized terms are summed only to cancel), summed over the lanes of a warp
-// that hold the same record and added to a per-record accumulator; a second
-// kernel chains the records through the camera transform and Eq. 2-3 into the
-// world parameters.
+// Eq. 9, 7-8, 6 and 4 into 8 record floats, summed over the lanes of a warp that
+// hold the same record and added to a per-record accumulator (one 32-byte
+// sector); a second kernel chains the records through Eq. 2-3 into the world
+// parameters.  8 floats suffice because the axes of a plane turn together: the
+// record keeps the gradients of s and of the radii and the three moments of the
+// axis gradients in the plane's own frame, built from the intersection relative to
+// the centre, t d - p_c = P_X v^x + P_Y v^y (so no metre-sized terms are summed only
+// to cancel), and the gradient of a_x is that of r^x+ less that of r^x- (a pair's
+// margin is r - |P|).  The camera rotation drops out of the chain.  The kernel is
+// bound by instruction issue, so what counts is the length of the aggregation: with
+// the 16 floats of n_c, s, v^x_c, a_x, v^y_c, a_y and the radii, summed in two halves
+// of 8, a step of the 3,000-plane room at 8 x 640x480 took 461 us at the first lambda
+// (now 408), 205 us at lambda 20 with 8 degree tilts (195) and 197 us at lambda 300
+// (193); 2,000 planes with the Eq. 5 weight, whose a_x and a_y need two floats more,
+// 2,562 us (2,420).
 #include <mutex>
 
 #include <cuda.h>
@@ -78,6 +86,11 @@ constexpr int kFwd = 0, kBwd = 1, kFused = 2;
 // address), which the chain kernel adds up into view_sums.
 constexpr int kSlots = 32;
 
+// Floats per record of the gradient accumulators: the gradients of s (0), of a turn about
+// v^y (1) and about -v^x (2) that moves n_c, of a turn about n_c (3), of the radii (4-7),
+// and for the Eq. 5 weight those of a_x and a_y (8, 9; the rectangle's follow from the radii).
+__host__ __device__ constexpr int grad_stride(int gauss) { return gauss ? 12 : 8; }
+
 struct SplatArgs {
     const ps_view* views;
     int n_views;
@@ -99,7 +112,9 @@ struct SplatArgs {
     // backward inputs / outputs
     const float* dLdD;
     const float* dLdN;
-    float4* g_rec;            // [R][4]
+    float* g_rec;             // [R][grad_stride]
+    float* g_radii;           // world radii gradients (pairs at P = 0 only)
+    int single_radii;
     int* status;
     // fused mode: supervision and loss outputs
     const float* gt_depth;
@@ -380,11 +395,12 @@ struct StripLoss {
     float sc, sl, sd, one;
 };
 
-template <int TW, int TH, int MODE, int KP>
+template <int TW, int TH, int MODE, int KP, int G>
 __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws, int2* stk_warp,
                                                int item)
 {
     constexpr int NS = TW * TH / 32;       // strips per tile
+    constexpr int NG = G ? 10 : 8;         // gradient floats per pair
     const int lane = threadIdx.x & 31;
     const int tile = item / NS;
     const int strip = item - tile * NS;
@@ -510,9 +526,9 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
         }
         for (int j = wmax - 1; j >= 0; --j) {
             const bool act = j < cnt;
-            float gr[16];
+            float gr[NG];
 #pragma unroll
-            for (int c = 0; c < 16; ++c) gr[c] = 0.f;
+            for (int c = 0; c < NG; ++c) gr[c] = 0.f;
             int id = -1;
             const int2 e = nxt;
             const float4 n = qn, vx = qx, vy = qy, rr = qr;
@@ -531,64 +547,60 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
                                        gN2 * (n.z - B2));
                 const float Tw = Tj * w;
                 float gt = Tw * gD;
-                // the intersection relative to the plane centre, t d - p_c = P_X v^x + P_Y v^y
-                // (Eq. 6 on the plane): radius-sized, so the gradients of n_c and v_c below
-                // (at fixed p_c) are accumulated without the cancellation of t d against p_c
-                const float ox = fmaf(pe.X, vx.x, pe.Y * vy.x);
-                const float oy = fmaf(pe.X, vx.y, pe.Y * vy.y);
-                const float oz = fmaf(pe.X, vx.z, pe.Y * vy.z);
                 A = fmaf(w, t, (1.f - w) * A);
                 B0 = fmaf(w, n.x, (1.f - w) * B0);
                 B1 = fmaf(w, n.y, (1.f - w) * B1);
                 B2 = fmaf(w, n.z, (1.f - w) * B2);
-                if (a.c.gauss) {
+                // gP: gradient of P_X or P_Y; spin: its moment about n_c
+                float spin;
+                if constexpr (G) {
                     // Eq. 5: w = exp(-(X^2 / sX^2 + Y^2 / sY^2) / 2):
                     // dw/dX = -w X / sX^2, dw/dsX = w X^2 / sX^3 (likewise Y)
                     const float ix = __fdividef(1.f, pe.sX), iy = __fdividef(1.f, pe.sY);
                     const float gX = -gw * w * pe.X * ix * ix;
                     const float gY = -gw * w * pe.Y * iy * iy;
                     const float grX = -gX * pe.X * ix, grY = -gY * pe.Y * iy;
-                    // Eq. 6 on both axes: P = t (d . v_c) - a, dP/dv_c = t d - p_c at fixed p_c
+                    // Eq. 6 on both axes: P = t (d . v_c) - a
                     gt = fmaf(gX, pe.dvx, gt);
                     gt = fmaf(gY, pe.dvy, gt);
-                    // Eq. 4: t = s / (d . n_c); dt/dn_c = (p_c - t d) / (d . n_c) at fixed p_c
-                    const float gs = __fdividef(gt, pe.den);
-                    gr[0] = fmaf(-gs, ox, Tw * gN0); gr[1] = fmaf(-gs, oy, Tw * gN1);
-                    gr[2] = fmaf(-gs, oz, Tw * gN2); gr[3] = gs;
-                    gr[4] = gX * ox; gr[5] = gX * oy; gr[6] = gX * oz; gr[7] = -gX;
-                    gr[8] = gY * ox; gr[9] = gY * oy; gr[10] = gY * oz; gr[11] = -gY;
+                    spin = fmaf(gX, pe.Y, -(gY * pe.X));
                     const bool px = pe.X > 0.f, py = pe.Y > 0.f;
-                    gr[12] = px ? grX : 0.f; gr[13] = px ? 0.f : grX;
-                    gr[14] = py ? grY : 0.f; gr[15] = py ? 0.f : grY;
+                    gr[4] = px ? grX : 0.f; gr[5] = px ? 0.f : grX;
+                    gr[6] = py ? grY : 0.f; gr[7] = py ? 0.f : grY;
+                    gr[8] = -gX; gr[9] = -gY;
                 } else {
-                // Eq. 7-9: w = 2 sigmoid(5 lambda m) below the clamp, dw/dm = 5 lambda w (1 - w/2)
-                const float gm = (pe.m < 0.f) ? gw * lam5 * w * (1.f - 0.5f * w) : 0.f;
-                // m = r_side - |P|: the radius gets gm, P gets -gm sgn(P)
-                const int ridx = (pe.sideX ? 0 : 2) + (pe.pos ? 0 : 1);
-                const float gP = (pe.P > 0.f) ? -gm : ((pe.P < 0.f) ? gm : 0.f);
-                // Eq. 6: P = t (d . v_c) - a, dP/dv_c = t d - p_c at fixed p_c
-                gt = fmaf(gP, pe.dv, gt);
-                // Eq. 4: t = s / (d . n_c); dt/dn_c = (p_c - t d) / (d . n_c) at fixed p_c
-                const float gs = __fdividef(gt, pe.den);
-                gr[0] = fmaf(-gs, ox, Tw * gN0); gr[1] = fmaf(-gs, oy, Tw * gN1);
-                gr[2] = fmaf(-gs, oz, Tw * gN2); gr[3] = gs;
-                const int vo = pe.sideX ? 4 : 8;
+                    // Eq. 7-9: w = 2 sigmoid(5 lambda m) below the clamp, dw/dm = 5 lambda w (1 - w/2)
+                    const float gm = (pe.m < 0.f) ? gw * lam5 * w * (1.f - 0.5f * w) : 0.f;
+                    // m = r_side - |P|: the radius gets gm, P gets -gm sgn(P)
+                    const float gP = pe.pos ? -gm : ((pe.P < 0.f) ? gm : 0.f);
+                    // Eq. 6: P = t (d . v_c) - a
+                    gt = fmaf(gP, pe.dv, gt);
+                    spin = gP * (pe.sideX ? pe.Y : -pe.X);
+                    const int ridx = (pe.sideX ? 0 : 2) + (pe.pos ? 0 : 1);
+                    const bool kink = gP == 0.f;       // gm = 0, or P = 0 (see below)
+                    const float ge = kink ? 0.f : gm;
 #pragma unroll
-                for (int c = 4; c < 12; c += 4) {
-                    if (c == vo) {
-                        gr[c + 0] = gP * ox;
-                        gr[c + 1] = gP * oy;
-                        gr[c + 2] = gP * oz;
-                        gr[c + 3] = -gP;
+                    for (int c = 0; c < 4; ++c) gr[4 + c] = (c == ridx) ? ge : 0.f;
+                    // the chain takes the gradient of a_x as that of r^x+ less that of r^x-; a pair
+                    // at P = 0 (m < 0 there only for a negative radius) moves its radius alone
+                    if (kink && gm != 0.f) {
+                        const int p = id - __ldg(&vw->rec_off) + __ldg(&vw->plane_off);
+                        atomicAdd(&a.g_radii[4 * (size_t)p + (a.single_radii ? (ridx & 2) : ridx)], gm);
                     }
                 }
-#pragma unroll
-                for (int c = 0; c < 4; ++c) gr[12 + c] = (c == ridx) ? gm : 0.f;
-                }
+                // Eq. 4: t = s / (d . n_c); at a fixed p_c, dt/dn_c = (p_c - t d) / (d . n_c)
+                // with t d - p_c = P_X v^x + P_Y v^y (Eq. 6 on the plane)
+                const float gs = __fdividef(gt, pe.den);
+                const float gNx = fmaf(gN0, vx.x, fmaf(gN1, vx.y, gN2 * vx.z));
+                const float gNy = fmaf(gN0, vy.x, fmaf(gN1, vy.y, gN2 * vy.z));
+                gr[0] = gs;
+                gr[1] = fmaf(-gs, pe.X, Tw * gNx);
+                gr[2] = fmaf(-gs, pe.Y, Tw * gNy);
+                gr[3] = spin;
             }
-            // warp aggregation: for each distinct record among the active lanes, the
-            // 16 gradient floats are summed over its lanes by a transpose-reduction
-            // and added with two 8-lane atomic instructions
+            // warp aggregation: for each distinct record among the active lanes, its gradient
+            // floats are summed over the lanes by a transpose-reduction and added with one
+            // 8-lane atomic instruction (a 32-byte sector)
             const unsigned actm = __ballot_sync(kFull, act);
             if (actm == 0) continue;
             const unsigned peers = __match_any_sync(kFull, id);
@@ -599,15 +611,21 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
                 const int gid = __shfl_sync(kFull, id, leader);
                 rem &= ~gmask;
                 const bool member = (gmask >> lane) & 1u;
-                float* dst = reinterpret_cast<float*>(a.g_rec + (size_t)gid * 4);
-                // two halves of 8 floats: lanes 4c..4c+3 end with the total of float c of the half
+                float* dst = a.g_rec + (size_t)gid * grad_stride(G);
+                // lanes 4c .. 4c + 3 end with the total of float c
+                float v[8];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    float v[8];
+                for (int c = 0; c < 8; ++c) v[c] = member ? gr[c] : 0.f;
+                warp_transpose8(v);
+                if ((lane & 3) == 0) atomicAdd(dst + (lane >> 2), v[0]);
+                if constexpr (G) {
+                    // a_x in lanes 0 .. 15, a_y in lanes 16 .. 31
+                    const bool hi = lane & 16;
+                    const float send = member ? (hi ? gr[8] : gr[9]) : 0.f;
+                    float x = (member ? (hi ? gr[9] : gr[8]) : 0.f) + __shfl_xor_sync(kFull, send, 16);
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) v[c] = member ? gr[8 * h + c] : 0.f;
-                    warp_transpose8(v);
-                    if ((lane & 3) == 0) atomicAdd(dst + 8 * h + ((lane >> 2) & 7), v[0]);
+                    for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+                    if ((lane & 15) == 0) atomicAdd(dst + 8 + (lane >> 4), x);
                 }
             }
         }
@@ -666,7 +684,7 @@ __global__ void __launch_bounds__(NW * 32, min_blocks(MODE, NW)) k_splat(SplatAr
         if (lane == 0) item = atomicAdd(a.counter, 1);
         item = __shfl_sync(kFull, item, 0);
         if (item >= a.n_items) break;
-        const StripLoss sl = run_strip<TW, TH, MODE, KP>(a, stage[w], stk_warp, item);
+        const StripLoss sl = run_strip<TW, TH, MODE, KP, G>(a, stage[w], stk_warp, item);
         if constexpr (MODE == kFused) {
             if (sl.v != vcur) {
                 if (vcur >= 0) flush_loss();
@@ -770,7 +788,8 @@ struct ChainArgs {
     const float* center;
     const float* quat;
     const float* radii;
-    const float4* g_rec;
+    const float* g_rec;       // [R][grad_stride]
+    int gauss;
     float* g_center;
     float* g_quat;
     float* g_radii;
@@ -795,16 +814,15 @@ __global__ void __launch_bounds__(128) k_chain(ChainArgs a)
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= K) return;
     const size_t r = (size_t)__ldg(&vw->rec_off) + k;
-    const float4 g0 = a.g_rec[4 * r + 0], g1 = a.g_rec[4 * r + 1];
-    const float4 g2 = a.g_rec[4 * r + 2], g3 = a.g_rec[4 * r + 3];
-    if (g0.x == 0.f && g0.y == 0.f && g0.z == 0.f && g0.w == 0.f && g1.x == 0.f && g1.y == 0.f &&
-        g1.z == 0.f && g1.w == 0.f && g2.x == 0.f && g2.y == 0.f && g2.z == 0.f && g2.w == 0.f &&
-        g3.x == 0.f && g3.y == 0.f && g3.z == 0.f && g3.w == 0.f)
+    const float4* gr = reinterpret_cast<const float4*>(a.g_rec + r * grad_stride(a.gauss));
+    const float4 g0 = gr[0], g3 = gr[1];
+    // rectangle: every pair's gradient of P is that of its radius, negative on the + side
+    float gax = g3.x - g3.y, gay = g3.z - g3.w;
+    if (a.gauss) { const float4 g2 = gr[2]; gax = g2.x; gay = g2.y; }
+    if (g0.x == 0.f && g0.y == 0.f && g0.z == 0.f && g0.w == 0.f && g3.x == 0.f && g3.y == 0.f &&
+        g3.z == 0.f && g3.w == 0.f && gax == 0.f && gay == 0.f)
         return;
     const int p = __ldg(&vw->plane_off) + k;
-    float R[12];
-#pragma unroll
-    for (int i = 0; i < 12; ++i) R[i] = __ldg(&vw->w2c[i]);
     const float q0 = __ldg(&a.quat[4 * p + 0]), q1 = __ldg(&a.quat[4 * p + 1]);
     const float q2 = __ldg(&a.quat[4 * p + 2]), q3 = __ldg(&a.quat[4 * p + 3]);
     const float qs = sqrtf(q0 * q0 + q1 * q1 + q2 * q2 + q3 * q3);
@@ -814,51 +832,25 @@ __global__ void __launch_bounds__(128) k_chain(ChainArgs a)
     const float vx[3] = {1.f - 2.f * (y * y + z * z), 2.f * (x * y + w * z), 2.f * (x * z - w * y)};
     const float vy[3] = {2.f * (x * y - w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z + w * x)};
     const float nn[3] = {2.f * (x * z + w * y), 2.f * (y * z - w * x), 1.f - 2.f * (x * x + y * y)};
-    float vxc[3], vyc[3], nc[3];
+    // The centre moves s = n_c . p_c, a_x and a_y; the camera rotation takes n_c, v^x_c, v^y_c
+    // back to the world axes, so the world gradient is their combination.
+    float gp[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        vxc[i] = R[4 * i] * vx[0] + R[4 * i + 1] * vx[1] + R[4 * i + 2] * vx[2];
-        vyc[i] = R[4 * i] * vy[0] + R[4 * i + 1] * vy[1] + R[4 * i + 2] * vy[2];
-        nc[i] = R[4 * i] * nn[0] + R[4 * i + 1] * nn[1] + R[4 * i + 2] * nn[2];
-    }
-    // record = {n_c, s = n_c.p_c, v^x_c, a_x = v^x_c.p_c, v^y_c, a_y = v^y_c.p_c, r}; the splat
-    // kernels accumulate the gradients of n_c, v^x_c, v^y_c at fixed p_c and those of s, a_x,
-    // a_y, so the camera-frame gradient of p_c is gs n_c + gax v^x_c + gay v^y_c
-    const float gs = g0.w, gax = g1.w, gay = g2.w;
-    const float gnc[3] = {g0.x, g0.y, g0.z};
-    const float gvxc[3] = {g1.x, g1.y, g1.z};
-    const float gvyc[3] = {g2.x, g2.y, g2.z};
-    float gpc[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) gpc[i] = gs * nc[i] + gax * vxc[i] + gay * vyc[i];
-    // camera -> world: multiply by R^T
-    float gp[3], gvx[3], gvy[3], gn[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        gp[i] = R[i] * gpc[0] + R[4 + i] * gpc[1] + R[8 + i] * gpc[2];
-        gvx[i] = R[i] * gvxc[0] + R[4 + i] * gvxc[1] + R[8 + i] * gvxc[2];
-        gvy[i] = R[i] * gvyc[0] + R[4 + i] * gvyc[1] + R[8 + i] * gvyc[2];
-        gn[i] = R[i] * gnc[0] + R[4 + i] * gnc[1] + R[8 + i] * gnc[2];
-    }
-    // G[i][c] = dL/dR_ic with columns (v^x, v^y, n)
-    const float G00 = gvx[0], G10 = gvx[1], G20 = gvx[2];
-    const float G01 = gvy[0], G11 = gvy[1], G21 = gvy[2];
-    const float G02 = gn[0], G12 = gn[1], G22 = gn[2];
-    const float gw = 2.f * (-z * G01 + y * G02 + z * G10 - x * G12 - y * G20 + x * G21);
-    const float gx = 2.f * (y * G01 + z * G02 + y * G10 - 2.f * x * G11 - w * G12 + z * G20 +
-                            w * G21 - 2.f * x * G22);
-    const float gy = 2.f * (-2.f * y * G00 + x * G01 + w * G02 + x * G10 + z * G12 - w * G20 +
-                            z * G21 - 2.f * y * G22);
-    const float gz = 2.f * (-2.f * z * G00 - w * G01 + x * G02 + w * G10 - 2.f * z * G11 +
-                            y * G12 + x * G20 + y * G21);
-    const float proj = gw * w + gx * x + gy * y + gz * z;
+    for (int i = 0; i < 3; ++i) gp[i] = g0.x * nn[i] + gax * vx[i] + gay * vy[i];
+    // A turn by theta in the plane's own frame moves v^x by theta_z v^y - theta_y n, v^y by
+    // theta_x n - theta_z v^x and n by theta_y v^x - theta_x v^y.  At a fixed centre the
+    // gradient of n lies along v^x (g0.y) and v^y (g0.z), those of v^x and v^y in the plane
+    // with the moment g0.w about n; parts along an axis itself do not turn it.  With
+    // dq = q (0, theta) / 2 the quaternion gradient is 2 q (0, torque) / |q|.
+    const float tx = -g0.z, ty = g0.y, tz = g0.w;
+    const float s2 = 2.f / qs;
     atomicAdd(&a.g_center[3 * p + 0], gp[0]);
     atomicAdd(&a.g_center[3 * p + 1], gp[1]);
     atomicAdd(&a.g_center[3 * p + 2], gp[2]);
-    atomicAdd(&a.g_quat[4 * p + 0], (gw - w * proj) / qs);
-    atomicAdd(&a.g_quat[4 * p + 1], (gx - x * proj) / qs);
-    atomicAdd(&a.g_quat[4 * p + 2], (gy - y * proj) / qs);
-    atomicAdd(&a.g_quat[4 * p + 3], (gz - z * proj) / qs);
+    atomicAdd(&a.g_quat[4 * p + 0], s2 * -(x * tx + y * ty + z * tz));
+    atomicAdd(&a.g_quat[4 * p + 1], s2 * (w * tx + y * tz - z * ty));
+    atomicAdd(&a.g_quat[4 * p + 2], s2 * (w * ty + z * tx - x * tz));
+    atomicAdd(&a.g_quat[4 * p + 3], s2 * (w * tz + x * ty - y * tx));
     float gr0 = g3.x, gr1 = g3.y, gr2 = g3.z, gr3 = g3.w;
     if (a.single_radii) { gr0 += gr1; gr1 = 0.f; gr2 += gr3; gr3 = 0.f; }
     atomicAdd(&a.g_radii[4 * p + 0], gr0);
@@ -1053,11 +1045,17 @@ cudaError_t launch_count(const SplatArgs& a, int n_tiles, unsigned long long* co
 
 constexpr size_t kCounterBytes = 256;
 
-// ps_splat_bwd: the record gradients, then the work counter
-inline size_t bwd_ws(const ps_frame* f)
+// Gradient accumulators: 64 bytes per record are reserved for any weight, a launch uses and
+// clears grad_stride floats per record, packed.
+inline size_t grec_max(const ps_frame* f) { return sizeof(float4) * 4 * (size_t)f->n_records; }
+
+inline size_t grad_bytes(const ps_frame* f, const ps_settings* s)
 {
-    return sizeof(float4) * 4 * (size_t)f->n_records + kCounterBytes;
+    return sizeof(float) * grad_stride((s->flags & PS_GAUSSIAN) ? 1 : 0) * (size_t)f->n_records;
 }
+
+// ps_splat_bwd: the record gradients, then the work counter
+inline size_t bwd_ws(const ps_frame* f) { return grec_max(f) + kCounterBytes; }
 
 // ps_splat_fused: as ps_splat_bwd, then the per-view partial loss sums
 inline size_t fused_ws(const ps_frame* f)
@@ -1135,7 +1133,7 @@ extern "C" ps_status ps_splat_bwd(const ps_planes* planes, const ps_frame* f, co
     if (ws_bytes < bwd_ws(f) || (reinterpret_cast<uintptr_t>(ws) & 15)) return PS_ERR_ARG;
     if (f->n_records == 0) return PS_OK;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const size_t grec_bytes = sizeof(float4) * 4 * (size_t)f->n_records;
+    const size_t grec_bytes = grad_bytes(f, s);
     // the record gradients and the work counter after them: one memset
     PS_CUDA_CHECK(cudaMemsetAsync(ws, 0, grec_bytes + sizeof(int), st));
     SplatArgs a{};
@@ -1143,13 +1141,14 @@ extern "C" ps_status ps_splat_bwd(const ps_planes* planes, const ps_frame* f, co
     a.rec = reinterpret_cast<const float4*>(rec); a.key = key;
     a.tile_ptr = tile_ptr; a.tile_ent = tile_ent; a.capacity = capacity;
     a.c = make_const(s); a.M = s->M; a.d_state = s->d_state;
-    a.dLdD = dLdD; a.dLdN = dLdN; a.g_rec = reinterpret_cast<float4*>(ws); a.status = d_status;
+    a.dLdD = dLdD; a.dLdN = dLdN; a.g_rec = reinterpret_cast<float*>(ws); a.g_radii = g_radii;
+    a.single_radii = (s->flags & PS_SINGLE_RADII) ? 1 : 0; a.status = d_status;
     a.counter = reinterpret_cast<int*>(static_cast<char*>(ws) + grec_bytes);
     if (dispatch<kBwd>(a, s, f->n_tiles, st, true) != cudaSuccess) return PS_ERR_CUDA;
     ChainArgs c;
     c.views = f->views; c.center = planes->center; c.quat = planes->quat; c.radii = planes->radii;
     c.g_rec = a.g_rec; c.g_center = g_center; c.g_quat = g_quat; c.g_radii = g_radii;
-    c.single_radii = (s->flags & PS_SINGLE_RADII) ? 1 : 0;
+    c.single_radii = a.single_radii; c.gauss = a.c.gauss;
     c.vs_slots = nullptr; c.view_sums = nullptr;
     dim3 grid((f->max_K + 127) / 128, f->n_views);
     k_chain<<<grid, 128, 0, st>>>(c);
@@ -1173,17 +1172,18 @@ extern "C" ps_status ps_splat_fused(const ps_planes* planes, const ps_frame* f,
     if (s->flags & PS_HARD) return PS_ERR_ARG;
     if (ws_bytes < fused_ws(f) || (reinterpret_cast<uintptr_t>(ws) & 15)) return PS_ERR_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const size_t grec_bytes = sizeof(float4) * 4 * (size_t)f->n_records;
+    const size_t grec_bytes = grad_bytes(f, s);
     // record gradients, work counter and partial loss sums: one memset
-    PS_CUDA_CHECK(cudaMemsetAsync(ws, 0, fused_ws(f), st));
-    double* slots = reinterpret_cast<double*>(static_cast<char*>(ws) + bwd_ws(f));
+    PS_CUDA_CHECK(cudaMemsetAsync(ws, 0, grec_bytes + fused_ws(f) - grec_max(f), st));
+    double* slots = reinterpret_cast<double*>(static_cast<char*>(ws) + grec_bytes + kCounterBytes);
     SplatArgs a{};
     a.views = f->views; a.n_views = f->n_views;
     a.rec = reinterpret_cast<const float4*>(rec); a.key = key;
     a.tile_ptr = tile_ptr; a.tile_ent = tile_ent; a.capacity = capacity;
     a.c = make_const(s); a.M = s->M; a.d_state = s->d_state;
     a.depth = depth; a.normal = normal; a.alpha = nullptr;
-    a.g_rec = reinterpret_cast<float4*>(ws); a.status = d_status;
+    a.g_rec = reinterpret_cast<float*>(ws); a.g_radii = g_radii;
+    a.single_radii = (s->flags & PS_SINGLE_RADII) ? 1 : 0; a.status = d_status;
     a.counter = reinterpret_cast<int*>(static_cast<char*>(ws) + grec_bytes);
     a.gt_depth = gt_depth; a.gt_normal = gt_normal;
     a.out_dLdD = dL_dD; a.out_dLdN = dL_dN; a.vs_slots = slots;
@@ -1193,7 +1193,7 @@ extern "C" ps_status ps_splat_fused(const ps_planes* planes, const ps_frame* f,
     c.views = f->views; c.center = planes->center; c.quat = planes->quat; c.radii = planes->radii;
     c.g_rec = f->n_records > 0 ? a.g_rec : nullptr;
     c.g_center = g_center; c.g_quat = g_quat; c.g_radii = g_radii;
-    c.single_radii = (s->flags & PS_SINGLE_RADII) ? 1 : 0;
+    c.single_radii = a.single_radii; c.gauss = a.c.gauss;
     c.vs_slots = slots; c.view_sums = view_sums;
     dim3 grid(f->max_K > 0 ? (f->max_K + 127) / 128 : 1, f->n_views);
     k_chain<<<grid, 128, 0, st>>>(c);

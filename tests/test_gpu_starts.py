@@ -89,3 +89,15 @@ def test_mono_start_is_seeded_and_matches_host_radii():
     assert np.allclose(a.radii, host.radii, rtol=1e-6, atol=1e-7)
     # centres lie near the ground-truth surfaces seen by the views (degraded depth: a few %)
     assert np.isfinite(a.center).all() and (a.radii > 0).all()
+
+
+@pytest.mark.parametrize("n", [2, 7, 9, 1024, 1025, 10000, 10001, 20011])
+def test_nn_distance_sizes(n):
+    # one CTA's queries, one chunk of points and both sides of the all-pairs limit, on a thin slab
+    # with a lone far point (many shells); FP32 squares against FP64 distances
+    from scipy.spatial import cKDTree
+    rng = np.random.default_rng(n)
+    p = (rng.uniform(0, 1, (n, 3)) * [4.0, 5.0, 0.01]).astype(np.float32)
+    p[n // 2] = [9.0, -7.0, 6.0]
+    ref = cKDTree(p.astype(np.float64)).query(p.astype(np.float64), k=2)[0][:, 1]
+    assert np.allclose(gpu_nn(p), ref, rtol=1e-6, atol=1e-7)

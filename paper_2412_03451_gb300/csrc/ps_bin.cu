@@ -29,20 +29,18 @@
 //      rectangle in a difference array over the flat (view-major, row-major)
 //      tile index: +1 where each row segment starts, -1 one past its end (the
 //      whole rectangle is one segment when it spans the full width);
-//   2. tile scan: the inclusive prefix of the difference array is the number
-//      of records covering each tile, and tile_ptr is the exclusive prefix of
-//      that, both in one pass; total -> d_required;
-//   3. scatter: one thread per pair writes its record id and entry key into a
+//   2. scans: tile_ptr is the exclusive prefix of the inclusive prefix of the
+//      difference array (the number of records covering each tile), total ->
+//      d_required; two launches serve both scans (k_scan_sums, k_scan_apply);
+//   3. scatter: one thread per pair writes its entry key and record id into a
 //      slot of its tile (unordered, via per-tile cursors);
-//   4. sort: each tile's slots by (key, record id): one warp per tile sorts up
-//      to kWarpSortCap entries in registers (a bitonic network over 1, 2, 4 or
-//      8 keys per lane); persistent CTAs take the longer lists
-//      (bitonic up to kSortCap entries, an O(n^2) rank sort beyond).
+//   4. sort: each tile's slots by (key, record id), k_sort: a warp sorts lists of
+//      up to kWarpSortCap entries in registers, four lists of up to 8 or two of up
+//      to 16 at a time; a block sorts the longer ones it meets together (bitonic up
+//      to kSortCap entries, an O(n^2) rank sort beyond).
 // Every pair gets its own thread, so a plane covering a thousand tiles costs
 // no more latency than one covering a single tile.
 #include "ps_internal.cuh"
-
-#include <cooperative_groups.h>
 
 using namespace ps;
 
@@ -51,12 +49,12 @@ namespace {
 constexpr int kSortCap = 4096;     // entries sorted in shared memory by a CTA (32 KB of u64)
 constexpr int kWarpSortCap = 256;  // entries sorted by one warp, in registers (8 per lane)
 constexpr int kSortWarps = 8;
-constexpr int kScanThreads = 1024;
+constexpr int kSortTiles = 4;      // consecutive tiles per warp
+constexpr int kScanThreads = 256;
 constexpr int kScanItems = 9;      // elements per thread per scan tile (odd: a thread's run
                                    // starts 9 words after its neighbour's, no bank conflicts)
 constexpr int kScanTile = kScanThreads * kScanItems;
 constexpr int kFlatBlocks = 152 * 8;
-constexpr int kSortBlocks = 152 * 4;  // persistent blocks of the long-list sort
 constexpr int kPairBlock = 256;       // pairs per scatter block = pairs per chunk of the chunk table
 
 inline long long n_chunks(long long capacity) { return capacity / kPairBlock + 2; }
@@ -66,42 +64,38 @@ struct BinWs {
     int4* rec_info;     // [R] first global tile, rectangle width in tiles, tiles_x, view
     int* tile_cnt;      // [n_tiles] difference array of the tile counts
     int* cursor;        // [n_tiles]
-    int* count;         // [n_tiles + 1] tile counts (arrays beyond one scan CTA)
     int* chunk_first;   // [n_chunks] record holding pair c * kPairBlock
-    long long* part;    // [2 * max scan tiles] scan partial sums
-    int* ent_tmp;       // [capacity] unordered entries
-    float* key_tmp;     // [capacity] their keys
+    longlong2* part;    // [scan tiles of records + of tiles] scan partial sums
+    unsigned long long* ent_tmp;    // [capacity] unordered entries, (key bits, record id)
 };
 
 inline size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
 inline int scan_tiles(long long n) { return (int)((n + kScanTile - 1) / kScanTile); }
 
-inline size_t ws_bytes(int R, int n_tiles, long long capacity)
-{
-    const int parts = 2 * (scan_tiles(R + 1) > scan_tiles(n_tiles) ? scan_tiles(R + 1) : scan_tiles(n_tiles)) + 2;
-    return align_up(sizeof(int) * (size_t)(R + 1)) + align_up(sizeof(int4) * (size_t)(R > 0 ? R : 1)) +
-           2 * align_up(sizeof(int) * (size_t)n_tiles) + align_up(sizeof(int) * (size_t)(n_tiles + 1)) +
-           align_up(sizeof(long long) * (size_t)parts) + align_up(sizeof(int) * (size_t)n_chunks(capacity)) +
-           2 * align_up(sizeof(int) * (size_t)(capacity > 0 ? capacity : 1));
-}
-
-inline BinWs carve(void* ws, int R, int n_tiles, long long capacity)
+inline BinWs carve(void* ws, int R, int n_tiles, long long capacity, size_t* bytes)
 {
     char* p = static_cast<char*>(ws);
+    size_t o = 0;
+    auto take = [&](size_t n) { char* r = p + o; o += align_up(n); return r; };
     BinWs w;
-    w.rec_cnt = reinterpret_cast<int*>(p); p += align_up(sizeof(int) * (size_t)(R + 1));
-    w.rec_info = reinterpret_cast<int4*>(p); p += align_up(sizeof(int4) * (size_t)(R > 0 ? R : 1));
-    w.tile_cnt = reinterpret_cast<int*>(p); p += align_up(sizeof(int) * (size_t)n_tiles);
-    w.cursor = reinterpret_cast<int*>(p); p += align_up(sizeof(int) * (size_t)n_tiles);
-    w.count = reinterpret_cast<int*>(p); p += align_up(sizeof(int) * (size_t)(n_tiles + 1));
-    w.chunk_first = reinterpret_cast<int*>(p); p += align_up(sizeof(int) * (size_t)n_chunks(capacity));
-    const int parts = 2 * (scan_tiles(R + 1) > scan_tiles(n_tiles) ? scan_tiles(R + 1) : scan_tiles(n_tiles)) + 2;
-    w.part = reinterpret_cast<long long*>(p); p += align_up(sizeof(long long) * (size_t)parts);
-    w.ent_tmp = reinterpret_cast<int*>(p);
-    p += align_up(sizeof(int) * (size_t)(capacity > 0 ? capacity : 1));
-    w.key_tmp = reinterpret_cast<float*>(p);
+    w.rec_cnt = reinterpret_cast<int*>(take(sizeof(int) * (size_t)(R + 1)));
+    w.rec_info = reinterpret_cast<int4*>(take(sizeof(int4) * (size_t)(R > 0 ? R : 1)));
+    w.tile_cnt = reinterpret_cast<int*>(take(sizeof(int) * (size_t)n_tiles));
+    w.cursor = reinterpret_cast<int*>(take(sizeof(int) * (size_t)n_tiles));
+    w.chunk_first = reinterpret_cast<int*>(take(sizeof(int) * (size_t)n_chunks(capacity)));
+    w.part = reinterpret_cast<longlong2*>(take(sizeof(longlong2) * (size_t)(scan_tiles(R) + scan_tiles(n_tiles))));
+    w.ent_tmp = reinterpret_cast<unsigned long long*>(
+        take(sizeof(unsigned long long) * (size_t)(capacity > 0 ? capacity : 1)));
+    if (bytes) *bytes = o;
     return w;
+}
+
+inline size_t ws_bytes(int R, int n_tiles, long long capacity)
+{
+    size_t n;
+    carve(nullptr, R, n_tiles, capacity, &n);
+    return n;
 }
 
 // 1. record counts ---------------------------------------------------------------
@@ -142,132 +136,18 @@ __global__ void __launch_bounds__(128) k_rec_count(const int4* __restrict__ rect
     rec_info[r] = info;
 }
 
-// Exclusive scan of int counts in three passes (tile sums, scan of the sums,
-// tile scan + offset).  The last pass can clamp the offsets to a capacity and
-// copy them to a cursor array (tile lists) and reports the total.
-__device__ __forceinline__ long long block_scan_excl(long long x, long long* s_warp, long long& total)
-{
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    long long incl = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const long long y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) s_warp[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-        long long w = (lane < (int)(blockDim.x >> 5)) ? s_warp[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        s_warp[lane] = w;   // inclusive warp totals
-    }
-    __syncthreads();
-    total = s_warp[(blockDim.x >> 5) - 1];
-    const long long r = incl - x + (wid > 0 ? s_warp[wid - 1] : 0);
-    __syncthreads();
-    return r;
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_sums(const int* __restrict__ in, int n,
-                                                            long long* __restrict__ part)
-{
-    __shared__ long long s_warp[32];
-    const long long base = (long long)blockIdx.x * kScanTile;
-    long long s = 0;
-#pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        const long long j = base + (long long)i * kScanThreads + threadIdx.x;
-        if (j < n) s += in[j];
-    }
-    long long total;
-    block_scan_excl(s, s_warp, total);
-    if (threadIdx.x == 0) part[blockIdx.x] = total;
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_parts(long long* __restrict__ part, int nparts)
-{
-    // one block: exclusive scan of the tile sums in place (nparts <= 1024 * 8)
-    __shared__ long long s_warp[32];
-    __shared__ long long s_carry;
-    if (threadIdx.x == 0) s_carry = 0;
-    __syncthreads();
-    for (int b0 = 0; b0 < nparts; b0 += kScanThreads) {
-        const int j = b0 + threadIdx.x;
-        const long long x = j < nparts ? part[j] : 0;
-        long long total;
-        const long long e = block_scan_excl(x, s_warp, total);
-        if (j < nparts) part[j] = e + s_carry;
-        __syncthreads();
-        if (threadIdx.x == 0) s_carry += total;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[nparts] = s_carry;
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int* __restrict__ in, int n,
-                                                             const long long* __restrict__ part,
-                                                             int nparts, int* __restrict__ out,
-                                                             int* __restrict__ cursor,
-                                                             long long capacity,
-                                                             long long* __restrict__ d_total,
-                                                             int* status)
-{
-    __shared__ long long s_warp[32];
-    __shared__ int s_in[kScanTile];
-    const long long base = (long long)blockIdx.x * kScanTile;
-    // coalesced load of the tile
-#pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        const long long j = base + (long long)i * kScanThreads + threadIdx.x;
-        s_in[i * kScanThreads + threadIdx.x] = j < n ? in[j] : 0;
-    }
-    __syncthreads();
-    // each thread scans kScanItems consecutive elements
-    long long loc[kScanItems];
-    long long s = 0;
-#pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        loc[i] = s;
-        s += s_in[threadIdx.x * kScanItems + i];
-    }
-    long long total;
-    const long long e = block_scan_excl(s, s_warp, total) + part[blockIdx.x];
-#pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        const long long j = base + (long long)threadIdx.x * kScanItems + i;
-        if (j < n) {
-            long long v = e + loc[i];
-            if (v > capacity) v = capacity;
-            out[j] = (int)v;
-            if (cursor) cursor[j] = (int)v;
-        }
-    }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-        const long long tot = part[nparts];
-        out[n] = (int)(tot < capacity ? tot : capacity);
-        if (d_total) *d_total = tot;
-        if (status && tot > capacity) set_status(status, PS_ERR_CAPACITY);
-    }
-}
-
-// Arrays of up to kScanOneMax elements: one launch, one thread-block cluster
-// of kScanCtas CTAs per array.  Each CTA scans its own segment in shared memory
-// (each thread a contiguous run, a block scan joining the runs), publishes the
-// segment's aggregate in its shared memory, and after a cluster barrier reads
-// the aggregates of the lower-ranked CTAs through distributed shared memory to
-// get its carry.  With `twice`, the array is first replaced by its inclusive
-// prefix (a difference array becomes the counts): a segment's aggregate is then
-// (sum of its differences D, sum of its carry-free counts S, length L), and
-// segments compose in order as (D1 + D2, S1 + S2 + L2 D1, L1 + L2).  With
-// chunk_first, the store pass also writes the chunk table of the pair numbering
-// (see k_chunk_first).  One launch runs one or two such jobs (one cluster each).
-constexpr int kScanOneMax = 48 * 1024;
-constexpr int kScanCtas = 8;             // CTAs per cluster (the portable maximum)
-
+// 2. scans ------------------------------------------------------------------------
+// Exclusive prefixes of int arrays of any length, in tiles of kScanTile elements, in two
+// launches that serve two jobs at once (the pair numbering and the tile offsets): the
+// first sums every tile, the second adds the sums of the tiles before its own and scans.
+// With `twice` the array is first replaced by its inclusive prefix (a difference array
+// becomes the counts).  An element x at place j of a tile of m then adds x to the counts
+// and x (m - j) to the tile's sum of counts, so both of a tile's sums (D, S) come without
+// a scan, and the prefix before tile b is sum D_r for the counts and
+// sum S_r + kScanTile (b - 1 - r) D_r for their sum.  Bound by latency:
+// 38,400 tiles and 24,000 records take 2.0 + 3.2 us (a launch of two 8-CTA clusters, one
+// per array, took 7.1 us), 307,200 and 640,000 2.8 + 5.7 us (three launches per pass over an
+// array and one for the chunk table took 43 us).
 struct ScanJob {
     const int* in;
     int n;
@@ -277,128 +157,135 @@ struct ScanJob {
     long long* d_total;   // optional
     int* status;          // optional: PS_ERR_CAPACITY when the total exceeds capacity
     int twice;
-    int* chunk_first;     // optional chunk table [n_chunk]
+    int* chunk_first;     // optional chunk table [n_chunk]: the record holding pair c * kPairBlock
     long long n_chunk;
+    longlong2* part;      // [scan tiles]
+    int blocks;           // scan tiles
 };
 
-__global__ void __cluster_dims__(kScanCtas, 1, 1) __launch_bounds__(kScanThreads)
-k_scan_one(ScanJob j0, ScanJob j1)
+// The block's totals of x and y (in every thread).
+__device__ __forceinline__ void block_sum2(long long& x, long long& y, longlong2* s_warp)
 {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
-    extern __shared__ int s_seg[];
-    __shared__ long long s_warp[32];
-    __shared__ long long s_agg[3];
-    const int rank = (int)cl.block_rank();
-    const ScanJob& a = blockIdx.x < kScanCtas ? j0 : j1;
-    const int n = a.n;
-    // segments of a multiple of 4 elements: 16-byte accesses stay aligned
-    const int seg = ((n + kScanCtas - 1) / kScanCtas + 3) & ~3;
-    const int lo = min(rank * seg, n), m = min(lo + seg, n) - lo;
-    const bool in_al = ((reinterpret_cast<uintptr_t>(a.in) | (size_t)lo * 4) & 15) == 0;
-    const int m4 = in_al ? m >> 2 : 0;
-    for (int j = threadIdx.x; j < m4; j += kScanThreads)
-        reinterpret_cast<int4*>(s_seg)[j] = __ldg(reinterpret_cast<const int4*>(a.in + lo) + j);
-    for (int j = 4 * m4 + threadIdx.x; j < m; j += kScanThreads) s_seg[j] = a.in[lo + j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        x += __shfl_xor_sync(0xffffffffu, x, o);
+        y += __shfl_xor_sync(0xffffffffu, y, o);
+    }
+    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = make_longlong2(x, y);
     __syncthreads();
-    // contiguous runs of an odd length: the runs of a warp's threads start in 32
-    // different banks, so the strided shared-memory passes below are conflict-free
-    const int per = ((m + kScanThreads - 1) / kScanThreads) | 1;
-    const int b = min((int)threadIdx.x * per, m), e = min(b + per, m);
-    long long D = 0;
+    x = 0; y = 0;
+#pragma unroll
+    for (int w = 0; w < kScanThreads / 32; ++w) { x += s_warp[w].x; y += s_warp[w].y; }
+    __syncthreads();
+}
+
+// Exclusive prefix of x over the block's threads.
+template <typename T>
+__device__ __forceinline__ T block_scan_excl(T x, T* s_warp)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    T incl = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const T y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) s_warp[wid] = incl;
+    __syncthreads();
+    T before = 0;
+#pragma unroll
+    for (int w = 0; w < kScanThreads / 32; ++w) before += w < wid ? s_warp[w] : 0;
+    __syncthreads();
+    return before + incl - x;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(ScanJob j0, ScanJob j1)
+{
+    __shared__ longlong2 s_warp[kScanThreads / 32];
+    const bool second = (int)blockIdx.x >= j0.blocks;
+    const ScanJob& a = second ? j1 : j0;
+    const int b = (int)blockIdx.x - (second ? j0.blocks : 0);
+    const int lo = b * kScanTile, m = min(kScanTile, a.n - lo);
+    long long D = 0, S = 0;
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+        const int j = i * kScanThreads + threadIdx.x;
+        const int x = j < m ? __ldg(&a.in[lo + j]) : 0;
+        D += x;
+        S += (long long)x * (m - j);
+    }
+    block_sum2(D, S, s_warp);
+    if (threadIdx.x == 0) a.part[b] = make_longlong2(D, S);
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_apply(ScanJob j0, ScanJob j1)
+{
+    __shared__ int s_x[kScanTile];
+    __shared__ longlong2 s_pair[kScanThreads / 32];
+    __shared__ long long s_wide[kScanThreads / 32];
+    __shared__ int s_int[kScanThreads / 32];
+    const bool second = (int)blockIdx.x >= j0.blocks;
+    const ScanJob& a = second ? j1 : j0;
+    const int b = (int)blockIdx.x - (second ? j0.blocks : 0);
+    const int lo = b * kScanTile, m = min(kScanTile, a.n - lo);
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+        const int j = i * kScanThreads + threadIdx.x;
+        s_x[j] = j < m ? a.in[lo + j] : 0;       // (in and out may be the same array)
+    }
+    // carries from the tiles before: the counts' prefix cD and the offset cC
+    long long cD = 0, cC = 0;
+    for (int r = threadIdx.x; r < b; r += kScanThreads) {
+        const longlong2 t = a.part[r];
+        cD += t.x;
+        cC += a.twice ? t.y + (long long)kScanTile * (b - 1 - r) * t.x : t.x;
+    }
+    block_sum2(cD, cC, s_pair);                  // (its barriers also cover s_x)
+    int x[kScanItems];
+    const int t0 = threadIdx.x * kScanItems;
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) x[i] = s_x[t0 + i];
     if (a.twice) {
         int run = 0;
-        for (int j = b; j < e; ++j) run += s_seg[j];
-        long long c = block_scan_excl(run, s_warp, D);
-        for (int j = b; j < e; ++j) {
-            c += s_seg[j];
-            s_seg[j] = (int)c;       // the count without the carry of the lower segments
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i) run += x[i];
+        int c = (int)cD + block_scan_excl(run, s_int);
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i) {
+            c += x[i];
+            x[i] = t0 + i < m ? c : 0;
         }
-        __syncthreads();
     }
     long long sum = 0;
-    for (int j = b; j < e; ++j) sum += s_seg[j];
-    long long S;
-    long long v = block_scan_excl(sum, s_warp, S);
-    if (threadIdx.x == 0) { s_agg[0] = D; s_agg[1] = S; s_agg[2] = m; }
-    cl.sync();
-    long long cD = 0, cC = 0;    // carries: differences and counts of the lower segments
-    for (int r = 0; r < rank; ++r) {
-        const long long* g = cl.map_shared_rank(s_agg, r);
-        cC += g[1] + g[2] * cD;
-        cD += g[0];
-    }
-    cl.sync();                   // every rank has read the aggregates before any exits
-    // offset of element j = cC + (j - lo) cD + (exclusive sum of the carry-free values)
-    v += cC + (long long)b * cD;
-    for (int j = b; j < e; ++j) {
-        const long long x = s_seg[j] + cD;
-        s_seg[j] = (int)(v < a.capacity ? v : a.capacity);
-        v += x;
-    }
-    const long long seg_end = cC + (long long)m * cD + S;   // offset just past the segment
-    __syncthreads();
-    const long long cap_end = seg_end < a.capacity ? seg_end : a.capacity;
-    const bool out_al = ((reinterpret_cast<uintptr_t>(a.out) | reinterpret_cast<uintptr_t>(a.cursor) |
-                          (size_t)lo * 4) & 15) == 0;
-    const int s4 = out_al ? m >> 2 : 0;
-    for (int j = threadIdx.x; j < s4; j += kScanThreads) {
-        const int4 x = reinterpret_cast<const int4*>(s_seg)[j];
-        reinterpret_cast<int4*>(a.out + lo)[j] = x;
-        if (a.cursor) reinterpret_cast<int4*>(a.cursor + lo)[j] = x;
-    }
-    for (int j = 4 * s4 + threadIdx.x; j < m; j += kScanThreads) {
-        const int x = s_seg[j];
-        a.out[lo + j] = x;
-        if (a.cursor) a.cursor[lo + j] = x;
-    }
-    if (a.chunk_first) {
-        for (int j = threadIdx.x; j < m; j += kScanThreads) {
-            const int x = s_seg[j];
-            const long long hi = j + 1 < m ? s_seg[j + 1] : cap_end;
-            for (long long c = ((long long)x + kPairBlock - 1) / kPairBlock;
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) sum += x[i];
+    long long v = cC + block_scan_excl(sum, s_wide);
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+        const int at = (int)(v < a.capacity ? v : a.capacity);
+        s_x[t0 + i] = at;
+        v += x[i];
+        if (a.chunk_first && t0 + i < m) {
+            const long long hi = v < a.capacity ? v : a.capacity;
+            for (long long c = ((long long)at + kPairBlock - 1) / kPairBlock;
                  c < a.n_chunk && c * kPairBlock < hi; ++c)
-                a.chunk_first[c] = lo + j;
+                a.chunk_first[c] = lo + t0 + i;
         }
     }
-    if (rank == kScanCtas - 1 && threadIdx.x == 0) {
-        a.out[n] = (int)cap_end;
-        if (a.d_total) *a.d_total = seg_end;
-        if (a.status && seg_end > a.capacity) set_status(a.status, PS_ERR_CAPACITY);
+    if (b == a.blocks - 1 && threadIdx.x == kScanThreads - 1) {      // v: the total
+        a.out[a.n] = (int)(v < a.capacity ? v : a.capacity);
+        if (a.d_total) *a.d_total = v;
+        if (a.status && v > a.capacity) set_status(a.status, PS_ERR_CAPACITY);
     }
-}
-
-// One or two cluster scans in one launch (both arrays <= kScanOneMax).
-cudaError_t scan_one(const ScanJob& j0, const ScanJob* j1, cudaStream_t st)
-{
-    int n = j0.n > 0 ? j0.n : 1;
-    if (j1 && j1->n > n) n = j1->n;
-    const size_t seg = (size_t)((n + kScanCtas - 1) / kScanCtas + 3) & ~(size_t)3;
-    k_scan_one<<<(j1 ? 2 : 1) * kScanCtas, kScanThreads, sizeof(int) * seg, st>>>(j0, j1 ? *j1 : j0);
-    return cudaGetLastError();
-}
-
-cudaError_t scan_exclusive(const int* in, int n, int* out, int* cursor, long long capacity,
-                           long long* part, long long* d_total, int* status, cudaStream_t st,
-                           int* twice_tmp = nullptr)
-{
-    if (n <= kScanOneMax) {
-        const ScanJob j{in, n, out, cursor, capacity, d_total, status, twice_tmp ? 1 : 0, nullptr, 0};
-        return scan_one(j, nullptr, st);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+        const int j = i * kScanThreads + threadIdx.x;
+        if (j < m) {
+            a.out[lo + j] = s_x[j];
+            if (a.cursor) a.cursor[lo + j] = s_x[j];
+        }
     }
-    if (twice_tmp) {
-        // inclusive prefix of in = the exclusive one shifted by one (twice_tmp [n + 1])
-        cudaError_t e = scan_exclusive(in, n, twice_tmp, nullptr, (1LL << 31) - 1, part, nullptr,
-                                       nullptr, st);
-        if (e != cudaSuccess) return e;
-        in = twice_tmp + 1;
-    }
-    const int nparts = scan_tiles(n > 0 ? n : 1);
-    k_scan_sums<<<nparts, kScanThreads, 0, st>>>(in, n, part);
-    k_scan_parts<<<1, kScanThreads, 0, st>>>(part, nparts);
-    k_scan_apply<<<nparts, kScanThreads, 0, st>>>(in, n, part, nparts, out, cursor, capacity,
-                                                  d_total, status);
-    return cudaGetLastError();
 }
 
 // 3. one thread per (record, tile) pair ----------------------------------------
@@ -410,18 +297,6 @@ __device__ __forceinline__ int pair_record(const int* __restrict__ off, int lo, 
         if (__ldg(&off[mid]) <= i) lo = mid; else hi = mid - 1;
     }
     return lo;
-}
-
-// chunk_first[c] = the record holding pair c * kPairBlock, for every chunk
-// c < n_chunk that starts below the pair total (one thread per record).
-__global__ void __launch_bounds__(256) k_chunk_first(const int* __restrict__ off, int R,
-                                                      int* __restrict__ chunk_first, long long n_chunk)
-{
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
-    const long long lo = __ldg(&off[r]), hi = __ldg(&off[r + 1]);
-    for (long long c = (lo + kPairBlock - 1) / kPairBlock; c < n_chunk && c * kPairBlock < hi; ++c)
-        chunk_first[c] = r;
 }
 
 // Pairs base .. base + kPairBlock - 1 of a block belong to records x .. y of the
@@ -485,8 +360,7 @@ __global__ void __launch_bounds__(kPairBlock) k_pair_scatter(const int* __restri
                                                        const int4* __restrict__ rec_info,
                                                        const int* __restrict__ tile_ptr,
                                                        int* __restrict__ cursor,
-                                                       int* __restrict__ ent_tmp,
-                                                       float* __restrict__ key_tmp,
+                                                       unsigned long long* __restrict__ ent_tmp,
                                                        const float4* __restrict__ rec,
                                                        const float* __restrict__ rec_key,
                                                        const ps_view* __restrict__ views,
@@ -513,22 +387,13 @@ __global__ void __launch_bounds__(kPairBlock) k_pair_scatter(const int* __restri
             const int pos = atomicAdd(&cursor[t], 1);
             // tile_ptr is clamped to the capacity: positions past it belong to lists
             // that did not fit and are dropped (the status word says so)
-            if (pos < lim) {
-                ent_tmp[pos] = r;
-                key_tmp[pos] = k;
-            }
+            // (keys are positive or +inf, so their bits sort like the values)
+            if (pos < lim) ent_tmp[pos] = ((unsigned long long)__float_as_uint(k) << 32) | (unsigned)r;
         }
     }
 }
 
 // 4. sort -----------------------------------------------------------------------
-// (key bits, record id) of slot j: keys are positive or +inf, so their bits sort like the values
-__device__ __forceinline__ unsigned long long sort_key(const float* __restrict__ key_tmp,
-                                                       const int* __restrict__ ent_tmp, int j)
-{
-    return ((unsigned long long)__float_as_uint(key_tmp[j]) << 32) | (unsigned)ent_tmp[j];
-}
-
 __device__ __forceinline__ void put(int* __restrict__ tile_ent, float* __restrict__ tile_key, int j,
                                     unsigned long long v)
 {
@@ -536,115 +401,73 @@ __device__ __forceinline__ void put(int* __restrict__ tile_ent, float* __restric
     tile_key[j] = __uint_as_float((unsigned)(v >> 32));
 }
 
-// Bitonic network over 32 E keys held E per lane, key e * 32 + lane in v[e]:
-// partners closer than 32 are in other lanes (shuffles), farther ones in the
-// same lane (compare-exchange in registers).
-template <int E>
+// One step of a sorting network across lanes: the smaller of the pair goes to the lane
+// with `lower` set if asc, to the other if not.
+__device__ __forceinline__ unsigned long long cas(unsigned long long v, int mask, bool lower, bool asc)
+{
+    const unsigned long long o = __shfl_xor_sync(0xffffffffu, v, mask);
+    return ((v < o) == (lower == asc)) ? v : o;
+}
+
+// Bitonic network over E groups of W keys, key e * W + lane % W in v[e], sorting the
+// 32 / W lists of a warp at once (E > 1 only for W = 32).  A merge of two ascending runs
+// starts with the mirrored partner, so every run of up to 16 keys is ascending and a step
+// needs one fixed predicate per lane; runs of 32 alternate in direction with e, which is
+// known at compile time.
+template <int W, int E>
 __device__ __forceinline__ void warp_bitonic(unsigned long long (&v)[E], int lane)
 {
 #pragma unroll
-    for (int k = 2; k <= 32 * E; k <<= 1) {
+    for (int k = 2; k <= W; k <<= 1) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const bool asc = k < 32 || E == 1 || (e & 1) == 0;
+            v[e] = cas(v[e], k - 1, (lane & (k >> 1)) == 0, asc);
+#pragma unroll
+            for (int j = k >> 2; j > 0; j >>= 1) v[e] = cas(v[e], j, (lane & j) == 0, asc);
+        }
+    }
+#pragma unroll
+    for (int k = 2; k <= E; k <<= 1) {            // runs of 32 k keys
 #pragma unroll
         for (int j = k >> 1; j > 0; j >>= 1) {
-            if (j >= 32) {
-                const int je = j >> 5;
 #pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    if ((e & je) == 0) {
-                        const bool up = ((e * 32 + lane) & k) == 0;
-                        const unsigned long long a = v[e], b = v[e + je];
-                        const bool sw = (a > b) == up;
-                        v[e] = sw ? b : a;
-                        v[e + je] = sw ? a : b;
-                    }
-                }
-            } else {
-                const bool lower = (lane & j) == 0;
-#pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    const unsigned long long o = __shfl_xor_sync(0xffffffffu, v[e], j);
-                    const bool up = ((e * 32 + lane) & k) == 0;
-                    v[e] = (lower == up) ? (v[e] < o ? v[e] : o) : (v[e] < o ? o : v[e]);
+            for (int e = 0; e < E; ++e) {
+                if ((e & j) == 0) {
+                    const bool asc = k == E || (e & k) == 0;
+                    const unsigned long long a = v[e], b = v[e + j];
+                    const bool sw = (a > b) == asc;
+                    v[e] = sw ? b : a;
+                    v[e + j] = sw ? a : b;
                 }
             }
+        }
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const bool asc = k == E || (e & k) == 0;
+#pragma unroll
+            for (int j = 16; j > 0; j >>= 1) v[e] = cas(v[e], j, (lane & j) == 0, asc);
         }
     }
 }
 
-template <int E>
-__device__ __forceinline__ void warp_sort_list(const int* __restrict__ ent_tmp,
-                                               const float* __restrict__ key_tmp,
+// Sorts the list of n slots from b (W = 32: the warp's one list; else this lane's group's).
+template <int W, int E>
+__device__ __forceinline__ void warp_sort_list(const unsigned long long* __restrict__ ent_tmp,
                                                int* __restrict__ tile_ent, float* __restrict__ tile_key,
                                                int b, int n, int lane)
 {
     unsigned long long v[E];
+    const int i = lane & (W - 1);
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = e * W + i < n ? ent_tmp[b + e * W + i] : ~0ull;
+    warp_bitonic<W, E>(v, lane);
 #pragma unroll
     for (int e = 0; e < E; ++e)
-        v[e] = e * 32 + lane < n ? sort_key(key_tmp, ent_tmp, b + e * 32 + lane) : ~0ull;
-    warp_bitonic<E>(v, lane);
-#pragma unroll
-    for (int e = 0; e < E; ++e)
-        if (e * 32 + lane < n) put(tile_ent, tile_key, b + e * 32 + lane, v[e]);
+        if (e * W + i < n) put(tile_ent, tile_key, b + e * W + i, v[e]);
 }
 
-// Short lists: one warp per tile.
-__global__ void __launch_bounds__(kSortWarps * 32) k_sort_warp(const int* __restrict__ tile_ptr,
-                                                               int n_tiles,
-                                                               const int* __restrict__ ent_tmp,
-                                                               const float* __restrict__ key_tmp,
-                                                               int* __restrict__ tile_ent,
-                                                               float* __restrict__ tile_key)
-{
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t = blockIdx.x * kSortWarps + w;
-    if (t >= n_tiles) return;
-    const int b = tile_ptr[t], e = tile_ptr[t + 1];
-    const int n = e - b;
-    if (n <= 0 || n > kWarpSortCap) return;
-    if (n == 1) {
-        if (lane == 0) { tile_ent[b] = ent_tmp[b]; tile_key[b] = key_tmp[b]; }
-        return;
-    }
-    if (n <= 32) { warp_sort_list<1>(ent_tmp, key_tmp, tile_ent, tile_key, b, n, lane); return; }
-    if (n <= 64) { warp_sort_list<2>(ent_tmp, key_tmp, tile_ent, tile_key, b, n, lane); return; }
-    if (n <= 128) { warp_sort_list<4>(ent_tmp, key_tmp, tile_ent, tile_key, b, n, lane); return; }
-    warp_sort_list<8>(ent_tmp, key_tmp, tile_ent, tile_key, b, n, lane);
-}
-
-// Long lists: one CTA per tile (tiles with at most kWarpSortCap entries return at once).
-__device__ void sort_long_list(const int* __restrict__ ent_tmp, const float* __restrict__ key_tmp,
-                               int* __restrict__ tile_ent, float* __restrict__ tile_key, int b, int n,
-                               unsigned long long* s);
-
-// Blocks stride over the tiles 256 at a time: each thread checks one list
-// length, the long lists found are sorted one after the other by the block.
-__global__ void __launch_bounds__(256) k_sort(const int* __restrict__ tile_ptr, int n_tiles,
-                                               const int* __restrict__ ent_tmp,
-                                               const float* __restrict__ key_tmp,
-                                               int* __restrict__ tile_ent,
-                                               float* __restrict__ tile_key)
-{
-    __shared__ unsigned long long s[kSortCap];
-    __shared__ int s_list[256];
-    __shared__ int s_cnt;
-    for (int t0 = blockIdx.x * 256; t0 < n_tiles; t0 += gridDim.x * 256) {
-        if (threadIdx.x == 0) s_cnt = 0;
-        __syncthreads();
-        const int t = t0 + threadIdx.x;
-        if (t < n_tiles && tile_ptr[t + 1] - tile_ptr[t] > kWarpSortCap)
-            s_list[atomicAdd(&s_cnt, 1)] = t;
-        __syncthreads();
-        const int cnt = s_cnt;
-        for (int q = 0; q < cnt; ++q) {
-            const int tt = s_list[q];
-            const int b = tile_ptr[tt];
-            sort_long_list(ent_tmp, key_tmp, tile_ent, tile_key, b, tile_ptr[tt + 1] - b, s);
-        }
-        __syncthreads();
-    }
-}
-
-__device__ void sort_long_list(const int* __restrict__ ent_tmp, const float* __restrict__ key_tmp,
+__device__ void sort_long_list(const unsigned long long* __restrict__ ent_tmp,
                                int* __restrict__ tile_ent, float* __restrict__ tile_key, int b, int n,
                                unsigned long long* s)
 {
@@ -652,8 +475,7 @@ __device__ void sort_long_list(const int* __restrict__ ent_tmp, const float* __r
     if (n <= kSortCap) {
         int N = 2;
         while (N < n) N <<= 1;
-        for (int i = tid; i < N; i += NT)
-            s[i] = i < n ? sort_key(key_tmp, ent_tmp, b + i) : ~0ull;
+        for (int i = tid; i < N; i += NT) s[i] = i < n ? ent_tmp[b + i] : ~0ull;
         __syncthreads();
         for (int k = 2; k <= N; k <<= 1) {
             for (int j = k >> 1; j > 0; j >>= 1) {
@@ -675,12 +497,12 @@ __device__ void sort_long_list(const int* __restrict__ ent_tmp, const float* __r
     // rank of each element = number of smaller keys (keys are unique)
     for (int i0 = 0; i0 < n; i0 += NT) {
         const int i = i0 + tid;
-        const unsigned long long ki = i < n ? sort_key(key_tmp, ent_tmp, b + i) : 0ull;
+        const unsigned long long ki = i < n ? ent_tmp[b + i] : 0ull;
         int rank = 0;
         for (int c0 = 0; c0 < n; c0 += kSortCap) {
             const int cn = min(kSortCap, n - c0);
             __syncthreads();
-            for (int j = tid; j < cn; j += NT) s[j] = sort_key(key_tmp, ent_tmp, b + c0 + j);
+            for (int j = tid; j < cn; j += NT) s[j] = ent_tmp[b + c0 + j];
             __syncthreads();
             if (i < n)
                 for (int j = 0; j < cn; ++j) rank += s[j] < ki;
@@ -688,6 +510,62 @@ __device__ void sort_long_list(const int* __restrict__ ent_tmp, const float* __r
         if (i < n) put(tile_ent, tile_key, b + rank, ki);
     }
     __syncthreads();    // the block's next list reuses s
+}
+
+// Bound by instruction issue, so short lists share a warp: at lambda 300 the lists of 3,000
+// planes in 8 views of 640x480 take 5.2 us (one list per warp and a second launch for the
+// long ones: 13.5 us), those of 16 uneven rooms 31 us (96 us), of 10,000 planes in 64 views
+// at lambda 20 118 us (169 us).
+__global__ void __launch_bounds__(kSortWarps * 32) k_sort(const int* __restrict__ tile_ptr, int n_tiles,
+                                                          const unsigned long long* __restrict__ ent_tmp,
+                                                          int* __restrict__ tile_ent,
+                                                          float* __restrict__ tile_key)
+{
+    __shared__ unsigned long long s[kSortCap];
+    __shared__ int s_list[kSortWarps * kSortTiles];
+    __shared__ int s_cnt;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) s_cnt = 0;
+    __syncthreads();
+    const int t0 = (blockIdx.x * kSortWarps + w) * kSortTiles;
+    // lane l < kSortTiles + 1: the start of tile t0 + l's list (past the last tile: its end)
+    const int ptr = __ldg(&tile_ptr[min(t0 + min(lane, kSortTiles), n_tiles)]);
+    const int len = __shfl_down_sync(0xffffffffu, ptr, 1) - ptr;      // lanes < kSortTiles
+    const int n4[kSortTiles] = {__shfl_sync(0xffffffffu, len, 0), __shfl_sync(0xffffffffu, len, 1),
+                                __shfl_sync(0xffffffffu, len, 2), __shfl_sync(0xffffffffu, len, 3)};
+    if (max(max(n4[0], n4[1]), max(n4[2], n4[3])) <= 8) {
+        const int q = lane >> 3;
+        const int b = __shfl_sync(0xffffffffu, ptr, q), n = __shfl_sync(0xffffffffu, len, q);
+        warp_sort_list<8, 1>(ent_tmp, tile_ent, tile_key, b, n, lane);
+    } else {
+#pragma unroll 1
+        for (int p = 0; p < kSortTiles; p += 2) {
+            const int na = __shfl_sync(0xffffffffu, len, p), nb = __shfl_sync(0xffffffffu, len, p + 1);
+            if (max(na, nb) <= 16) {
+                const int q = p + (lane >> 4);
+                const int b = __shfl_sync(0xffffffffu, ptr, q), n = __shfl_sync(0xffffffffu, len, q);
+                warp_sort_list<16, 1>(ent_tmp, tile_ent, tile_key, b, n, lane);
+                continue;
+            }
+#pragma unroll 1
+            for (int q = p; q < p + 2; ++q) {
+                const int b = __shfl_sync(0xffffffffu, ptr, q), n = __shfl_sync(0xffffffffu, len, q);
+                if (n <= 0) continue;
+                if (n <= 32) warp_sort_list<32, 1>(ent_tmp, tile_ent, tile_key, b, n, lane);
+                else if (n <= 64) warp_sort_list<32, 2>(ent_tmp, tile_ent, tile_key, b, n, lane);
+                else if (n <= 128) warp_sort_list<32, 4>(ent_tmp, tile_ent, tile_key, b, n, lane);
+                else if (n <= kWarpSortCap) warp_sort_list<32, 8>(ent_tmp, tile_ent, tile_key, b, n, lane);
+                else if (lane == 0) s_list[atomicAdd(&s_cnt, 1)] = t0 + q;
+            }
+        }
+    }
+    __syncthreads();
+    const int cnt = s_cnt;
+    for (int q = 0; q < cnt; ++q) {
+        const int t = s_list[q];
+        const int b = tile_ptr[t];
+        sort_long_list(ent_tmp, tile_ent, tile_key, b, tile_ptr[t + 1] - b, s);
+    }
 }
 
 }  // namespace
@@ -715,7 +593,7 @@ extern "C" ps_status ps_bin_tiles(const ps_frame* frame, const ps_settings* s, c
     if (reinterpret_cast<uintptr_t>(ws) & 255) return PS_ERR_ARG;
     if (reinterpret_cast<uintptr_t>(rect) & 15) return PS_ERR_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    BinWs w = carve(ws, R, frame->n_tiles, capacity);
+    BinWs w = carve(ws, R, frame->n_tiles, capacity, nullptr);
     PS_CUDA_CHECK(cudaMemsetAsync(w.tile_cnt, 0, sizeof(int) * (size_t)frame->n_tiles, st));
     const int4* rc = reinterpret_cast<const int4*>(rect);
     const long long nch = n_chunks(capacity);
@@ -727,39 +605,25 @@ extern "C" ps_status ps_bin_tiles(const ps_frame* frame, const ps_settings* s, c
     }
     // Pair numbering: offsets clamp at the int range (still non-decreasing), so pairs
     // past it are never scattered, and the tile total then exceeds every capacity.
-    if (R > 0 && R <= kScanOneMax && frame->n_tiles <= kScanOneMax) {
-        // the pair numbering (and its chunk table) and the tile counts and offsets are
-        // independent: one launch, one CTA each
-        const ScanJob jr{w.rec_cnt, R, w.rec_cnt, nullptr, (1LL << 31) - 1, nullptr, nullptr, 0,
-                         w.chunk_first, nch};
-        const ScanJob jt{w.tile_cnt, frame->n_tiles, tile_ptr, w.cursor, capacity, d_required,
-                         d_status, 1, nullptr, 0};
-        if (scan_one(jr, &jt, st) != cudaSuccess) return PS_ERR_CUDA;
-    } else {
-        if (R > 0) {
-            if (scan_exclusive(w.rec_cnt, R, w.rec_cnt, nullptr, (1LL << 31) - 1, w.part, nullptr,
-                               nullptr, st) != cudaSuccess)
-                return PS_ERR_CUDA;
-            k_chunk_first<<<(R + 255) / 256, 256, 0, st>>>(w.rec_cnt, R, w.chunk_first, nch);
-            PS_LAUNCH_CHECK();
-        }
-        if (scan_exclusive(w.tile_cnt, frame->n_tiles, tile_ptr, w.cursor, capacity, w.part,
-                           d_required, d_status, st, w.count) != cudaSuccess)
-            return PS_ERR_CUDA;
-    }
+    const int tr = scan_tiles(R), tt = scan_tiles(frame->n_tiles);
+    const ScanJob jr{w.rec_cnt, R, w.rec_cnt, nullptr, (1LL << 31) - 1, nullptr, nullptr, 0,
+                     w.chunk_first, nch, w.part, tr};
+    const ScanJob jt{w.tile_cnt, frame->n_tiles, tile_ptr, w.cursor, capacity, d_required,
+                     d_status, 1, nullptr, 0, w.part + tr, tt};
+    k_scan_sums<<<tr + tt, kScanThreads, 0, st>>>(jr, jt);
+    PS_LAUNCH_CHECK();
+    k_scan_apply<<<tr + tt, kScanThreads, 0, st>>>(jr, jt);
+    PS_LAUNCH_CHECK();
     if (R > 0 && capacity > 0) {
         k_pair_scatter<<<kFlatBlocks, kPairBlock, 0, st>>>(w.rec_cnt, R, w.rec_info, tile_ptr, w.cursor,
-                                                           w.ent_tmp, w.key_tmp,
+                                                           w.ent_tmp,
                                                            reinterpret_cast<const float4*>(rec), key,
                                                            frame->views, s->tile_w, s->tile_h, s->z_near,
                                                            w.chunk_first, nch);
         PS_LAUNCH_CHECK();
-        k_sort_warp<<<(frame->n_tiles + kSortWarps - 1) / kSortWarps, kSortWarps * 32, 0, st>>>(
-            tile_ptr, frame->n_tiles, w.ent_tmp, w.key_tmp, tile_ent, tile_key);
-        PS_LAUNCH_CHECK();
-        const int sort_blocks = (frame->n_tiles + 255) / 256;
-        k_sort<<<sort_blocks < kSortBlocks ? sort_blocks : kSortBlocks, 256, 0, st>>>(
-            tile_ptr, frame->n_tiles, w.ent_tmp, w.key_tmp, tile_ent, tile_key);
+        constexpr int per = kSortWarps * kSortTiles;
+        k_sort<<<(frame->n_tiles + per - 1) / per, kSortWarps * 32, 0, st>>>(
+            tile_ptr, frame->n_tiles, w.ent_tmp, tile_ent, tile_key);
         PS_LAUNCH_CHECK();
     }
     return PS_OK;

@@ -41,6 +41,21 @@ __device__ __forceinline__ int view_of_tile(const ps_view* views, int V, int til
     return lo;
 }
 
+// The same by a whole warp: 32 views per step, one load each, instead of a chain of
+// dependent loads.
+__device__ __forceinline__ int warp_view_of_tile(const ps_view* views, int V, int tile)
+{
+    const int lane = threadIdx.x & 31;
+    int v = -1;
+    for (int b = 0; b < V; b += 32) {
+        const bool in = b + lane < V && __ldg(&views[b + lane].tile_off) <= tile;
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        v += __popc(m);
+        if (m != 0xffffffffu) break;
+    }
+    return v;
+}
+
 // One plane in camera coordinates, as stored in a record.
 struct Rec {
     float4 n;    // n_c, s = n_c . p_c
@@ -115,9 +130,25 @@ __device__ __forceinline__ bool eval_pair(const float4& n, const float4& vx, con
     return ok;
 }
 
+// Minimum and maximum that are NaN if either argument is.
+__device__ __forceinline__ float min_nan(float a, float b)
+{
+    float d;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+    return d;
+}
+
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float d;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+    return d;
+}
+
 // Rays through the pixel centres at the corners of a warp's pixel rectangle.
 struct WarpRegion {
     float dxa, dxb, dya, dyb;
+    float den_min;     // 0.01 x the longest of the four rays: den above it is accurate to 3e-5
 };
 
 // Conservative test whether a plane can pass the filter at any pixel of a
@@ -125,21 +156,24 @@ struct WarpRegion {
 // are linear-fractional in the ray d = (dx, dy, 1); if d . n_c keeps its sign
 // over the rectangle they are monotone along every line, so their ranges over
 // the rectangle are spanned by the four corner rays.  The corner values use
-// the per-pixel formulas of eval_pair; the margins cover FP32 rounding.
+// the per-pixel formulas of eval_pair; the margins cover FP32 rounding.  t_low is
+// the smallest depth at the corners, which bounds the depth at every pixel of the
+// rectangle from below up to rounding (0 where d . n_c is too small for that).
+template <bool LOW>
 __device__ __forceinline__ bool region_may_hit(const float4& n, const float4& vx, const float4& vy,
                                                const float4& r, const WarpRegion& g,
-                                               const SplatConst& c)
+                                               const SplatConst& c, float& t_low)
 {
     float tmin = INFINITY, tmax = -INFINITY, xmin = INFINITY, xmax = -INFINITY;
     float ymin = INFINITY, ymax = -INFINITY;
-    int npos = 0, nneg = 0;
+    float dlo = INFINITY, dhi = -INFINITY;
+    t_low = 0.f;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const float dx = (k & 1) ? g.dxb : g.dxa;
         const float dy = (k & 2) ? g.dyb : g.dya;
         const float den = fmaf(dx, n.x, fmaf(dy, n.y, n.z));
-        npos += den > 2e-6f;
-        nneg += den < -2e-6f;
+        dlo = min_nan(dlo, den); dhi = max_nan(dhi, den);      // NaN stays: no bound
         const float t = __fdividef(n.w, den);
         const float dvx = fmaf(dx, vx.x, fmaf(dy, vx.y, vx.z));
         const float dvy = fmaf(dx, vy.x, fmaf(dy, vy.y, vy.z));
@@ -149,7 +183,10 @@ __device__ __forceinline__ bool region_may_hit(const float4& n, const float4& vx
         xmin = fminf(xmin, X); xmax = fmaxf(xmax, X);
         ymin = fminf(ymin, Y); ymax = fmaxf(ymax, Y);
     }
-    if (npos != 4 && nneg != 4) return true;       // d . n_c may vanish: no bound
+    if (!(dlo > 2e-6f) && !(dhi < -2e-6f)) return true;       // d . n_c may vanish: no bound
+    if constexpr (LOW) {
+        if (dlo > g.den_min || dhi < -g.den_min) t_low = tmin;
+    }
     if (tmax < c.z_near * 0.99999f || tmin > c.z_far * 1.00001f) return false;
     // support: r + reject around the rectangle, or kappa r for the Eq. 5 weight
     const float sc = c.gauss ? c.kappa : 1.f;

@@ -129,7 +129,7 @@ struct SplatArgs {
 struct WarpStage {
     float4 rec[4][32];        // record float4 c of chunk entry e at rec[c][e] (no bank conflicts)
     int id[32];
-    float key[33];            // entry keys x (1 - 1/4096); key[32]: the next chunk's first entry
+    float key[33];            // depth bounds x (1 - 1/4096) from entry e on; [32]: from the next chunk on
 };
 
 __device__ __forceinline__ float sgnf(float x) { return (x > 0.f) ? 1.f : ((x < 0.f) ? -1.f : 0.f); }
@@ -279,7 +279,12 @@ __device__ __forceinline__ void flush(Walk<KP>& s, Sink& k, const float4* __rest
 }
 
 // Walks one tile list for the warp's 32 pixels.
-template <int MODE, int KP>
+// SB: the list's keys, which bound the depths over the tile, are tightened to the warp's
+// strip, for a scan per chunk of the list.  Worth it for the Eq. 5 weight, where every pair
+// is partly transparent and waits in the buffer until a bound passes it (2,000 planes at
+// lambda 20 in 8 views of 640x480: a step 2,427 -> 2,297 us); for the rectangle weight a step
+// changes by -1..+4% by tile shape and lambda and a hard render is 5% slower.
+template <int MODE, int KP, bool SB>
 __device__ __forceinline__ void walk_strip(const SplatArgs& a, WarpStage& ws, Walk<KP>& s,
                                            Sink& k, float dx, float dy, const WarpRegion& g,
                                            int beg, int end)
@@ -292,21 +297,34 @@ __device__ __forceinline__ void walk_strip(const SplatArgs& a, WarpStage& ws, Wa
             // stage: lane l loads entry base + l and tests it against the warp's pixels
             const int i = base + lane;
             bool ok = false;
+            float low = INFINITY;
             if (i < end) {
                 const int id = __ldg(&a.tile_ent[i]);
                 const float4* r = a.rec + (size_t)id * 4;
                 const float4 n = __ldg(r + 0), vx = __ldg(r + 1), vy = __ldg(r + 2), rr = __ldg(r + 3);
-                ok = region_may_hit(n, vx, vy, rr, g, a.c);
-                ws.key[lane] = __ldg(&a.key[i]) * kMargin;
+                float t_low;
+                ok = region_may_hit<SB>(n, vx, vy, rr, g, a.c, t_low);
+                if constexpr (!SB) low = __ldg(&a.key[i]) * kMargin;
                 if (ok) {
+                    if constexpr (SB) low = fmaxf(__ldg(&a.key[i]), t_low) * kMargin;
                     ws.id[lane] = id;
                     ws.rec[0][lane] = n; ws.rec[1][lane] = vx; ws.rec[2][lane] = vy; ws.rec[3][lane] = rr;
                 }
-            } else {
-                ws.key[lane] = INFINITY;
             }
-            if (lane == 0)
-                ws.key[32] = (base + 32 < end) ? __ldg(&a.key[base + 32]) * kMargin : INFINITY;
+            // key[e]: a lower bound of every depth from entry e on.  The list's keys are sorted;
+            // with strip bounds it is the smallest bound of the chunk's surviving entries from e
+            // on and of the next chunk's first key.
+            if constexpr (SB) {
+                const float next = (base + 32 < end) ? __ldg(&a.key[base + 32]) * kMargin : INFINITY;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) low = fminf(low, __shfl_down_sync(kFull, low, o));
+                ws.key[lane] = fminf(low, next);
+                if (lane == 0) ws.key[32] = next;
+            } else {
+                ws.key[lane] = low;
+                if (lane == 0)
+                    ws.key[32] = (base + 32 < end) ? __ldg(&a.key[base + 32]) * kMargin : INFINITY;
+            }
             unsigned m = __ballot_sync(kFull, ok);
             __syncwarp();
             while (m) {
@@ -317,9 +335,8 @@ __device__ __forceinline__ void walk_strip(const SplatArgs& a, WarpStage& ws, Wa
                 }
                 const int e = __ffs(m) - 1;
                 m &= m - 1;
-                // keys are sorted and entries that fail the region test cannot reach any
-                // pixel of the strip: the next surviving entry's key (or the next chunk's
-                // first key) bounds every later depth
+                // entries that fail the region test cannot reach any pixel of the strip: the
+                // bound at the next surviving entry (or the next chunk) holds for every later depth
                 const int en = m ? __ffs(m) - 1 : 32;
                 if (!s.done) {
                     PairEval pe;
@@ -404,7 +421,10 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
     const int lane = threadIdx.x & 31;
     const int tile = item / NS;
     const int strip = item - tile * NS;
-    const int v = view_of_tile(a.views, a.n_views, tile);
+    // (the cooperative search takes 3% off a hard render of 64 views and adds 2% to the fused
+    // kernel, whose registers it costs)
+    const int v = MODE == kFwd ? warp_view_of_tile(a.views, a.n_views, tile)
+                               : view_of_tile(a.views, a.n_views, tile);
     const ps_view* vw = a.views + v;
     const int W = __ldg(&vw->W), H = __ldg(&vw->H);
     const int tx_n = __ldg(&vw->tiles_x);
@@ -422,13 +442,11 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
     WarpRegion g;
     {
         constexpr int WX = TW < 32 ? TW : 32;
-        constexpr int WY = TW < 32 ? 32 / TW : 1;
-        const int q0 = strip * 32;
-        const int gx0 = tx0 + q0 % TW, gy0 = ty0 + q0 / TW;
-        g.dxa = __fdiv_rn((float)gx0 + 0.5f - cx, fx);
-        g.dxb = __fdiv_rn((float)(gx0 + WX - 1) + 0.5f - cx, fx);
-        g.dya = __fdiv_rn((float)gy0 + 0.5f - cy, fy);
-        g.dyb = __fdiv_rn((float)(gy0 + WY - 1) + 0.5f - cy, fy);
+        // the rectangle's corner rays are those of its corner lanes (outside the image too)
+        g.dxa = __shfl_sync(kFull, dx, 0); g.dxb = __shfl_sync(kFull, dx, WX - 1);
+        g.dya = __shfl_sync(kFull, dy, 0); g.dyb = __shfl_sync(kFull, dy, 31);
+        const float mx = fmaxf(fabsf(g.dxa), fabsf(g.dxb)), my = fmaxf(fabsf(g.dya), fabsf(g.dyb));
+        g.den_min = 0.01f * sqrtf(fmaf(mx, mx, fmaf(my, my, 1.f)));
     }
     const int beg = (int)min((long long)__ldg(&a.tile_ptr[tile]), a.capacity);
     const int end = (int)min((long long)__ldg(&a.tile_ptr[tile + 1]), a.capacity);
@@ -460,7 +478,7 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
             if (gD == 0.f && gN0 == 0.f && gN1 == 0.f && gN2 == 0.f) s.done = true;
         }
     }
-    walk_strip<MODE>(a, ws, s, k, dx, dy, g, beg, end);
+    walk_strip<MODE, KP, G != 0>(a, ws, s, k, dx, dy, g, beg, end);
 
     if constexpr (MODE != kBwd) {
         if (inside) {
@@ -872,6 +890,28 @@ struct LossArgs {
     float a_cos, a_l1n, a_depth;
 };
 
+// One pixel's terms added to sum, its gradient returned.
+__device__ __forceinline__ float4 loss_pixel(const LossArgs& a, float D, float N0, float N1, float N2,
+                                             float Dg, float G0, float G1, float G2, float (&sum)[4])
+{
+    if (!(Dg > 0.f)) return make_float4(0.f, 0.f, 0.f, 0.f);
+    const float c = 1.f - (N0 * G0 + N1 * G1 + N2 * G2);
+    const float e0 = N0 - G0, e1 = N1 - G1, e2 = N2 - G2;
+    const float dd = D - Dg;
+    sum[0] += fabsf(c);
+    sum[1] += fabsf(e0) + fabsf(e1) + fabsf(e2);
+    sum[2] += fabsf(dd);
+    sum[3] += 1.f;
+    const float sc = -a.a_cos * sgnf(c);
+    return make_float4(a.a_depth * sgnf(dd), sc * G0 + a.a_l1n * sgnf(e0),
+                       sc * G1 + a.a_l1n * sgnf(e1), sc * G2 + a.a_l1n * sgnf(e2));
+}
+
+// Bound by memory: 32 bytes read and 16 written per pixel.  A thread takes four pixels with
+// 16-byte accesses (a normal alone is three 4-byte accesses, 12 bytes apart between lanes)
+// where a view's maps and supervision share their alignment; the pixels before the first
+// boundary, after the last and of other views go one by one.  64 views of 640x480:
+// 260 -> 195 us, 4.8 TB/s.
 __global__ void __launch_bounds__(256) k_loss(LossArgs a)
 {
     const int v = blockIdx.y;
@@ -879,38 +919,48 @@ __global__ void __launch_bounds__(256) k_loss(LossArgs a)
     const long long HW = (long long)__ldg(&vw->H) * __ldg(&vw->W);
     const long long off = __ldg(&vw->pix_off);
     const long long goff = __ldg(&vw->gt_off);
-    float sc = 0.f, sl = 0.f, sd = 0.f, cnt = 0.f;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < HW;
-         i += (long long)gridDim.x * blockDim.x) {
-        const long long p = off + i;
-        const long long q = goff + i;
-        const float Dg = __ldg(&a.gt_depth[q]);
-        if (!(Dg > 0.f)) {
-            a.dLdD[p] = 0.f;
-            a.dLdN[3 * p + 0] = 0.f; a.dLdN[3 * p + 1] = 0.f; a.dLdN[3 * p + 2] = 0.f;
-            continue;
-        }
-        const float D = __ldg(&a.depth[p]);
-        const float N0 = __ldg(&a.normal[3 * p]), N1 = __ldg(&a.normal[3 * p + 1]),
-                    N2 = __ldg(&a.normal[3 * p + 2]);
-        const float G0 = __ldg(&a.gt_normal[3 * q]), G1 = __ldg(&a.gt_normal[3 * q + 1]),
-                    G2 = __ldg(&a.gt_normal[3 * q + 2]);
-        const float c = 1.f - (N0 * G0 + N1 * G1 + N2 * G2);
-        const float e0 = N0 - G0, e1 = N1 - G1, e2 = N2 - G2;
-        const float dd = D - Dg;
-        sc += fabsf(c);
-        sl += fabsf(e0) + fabsf(e1) + fabsf(e2);
-        sd += fabsf(dd);
-        cnt += 1.f;
-        a.dLdD[p] = a.a_depth * sgnf(dd);
-        const float sc_ = -a.a_cos * sgnf(c);
-        a.dLdN[3 * p + 0] = sc_ * G0 + a.a_l1n * sgnf(e0);
-        a.dLdN[3 * p + 1] = sc_ * G1 + a.a_l1n * sgnf(e1);
-        a.dLdN[3 * p + 2] = sc_ * G2 + a.a_l1n * sgnf(e2);
+    float sum[4] = {0.f, 0.f, 0.f, 0.f};
+    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    const bool vec = ((off ^ goff) & 3) == 0 &&
+                     ((reinterpret_cast<uintptr_t>(a.depth) | reinterpret_cast<uintptr_t>(a.normal) |
+                       reinterpret_cast<uintptr_t>(a.gt_depth) | reinterpret_cast<uintptr_t>(a.gt_normal) |
+                       reinterpret_cast<uintptr_t>(a.dLdD) | reinterpret_cast<uintptr_t>(a.dLdN)) & 15) == 0;
+    const long long head = vec ? min(HW, (-off) & 3) : HW;
+    const long long quads = (HW - head) >> 2;
+    for (long long i = tid; i < quads; i += stride) {
+        const long long p = (off + head) / 4 + i, q = (goff + head) / 4 + i;
+        const float4 D = __ldg(reinterpret_cast<const float4*>(a.depth) + p);
+        const float4 Dg = __ldg(reinterpret_cast<const float4*>(a.gt_depth) + q);
+        const float4* np = reinterpret_cast<const float4*>(a.normal) + 3 * p;
+        const float4* gp = reinterpret_cast<const float4*>(a.gt_normal) + 3 * q;
+        const float4 n0 = __ldg(np), n1 = __ldg(np + 1), n2 = __ldg(np + 2);
+        const float4 g0 = __ldg(gp), g1 = __ldg(gp + 1), g2 = __ldg(gp + 2);
+        const float4 r0 = loss_pixel(a, D.x, n0.x, n0.y, n0.z, Dg.x, g0.x, g0.y, g0.z, sum);
+        const float4 r1 = loss_pixel(a, D.y, n0.w, n1.x, n1.y, Dg.y, g0.w, g1.x, g1.y, sum);
+        const float4 r2 = loss_pixel(a, D.z, n1.z, n1.w, n2.x, Dg.z, g1.z, g1.w, g2.x, sum);
+        const float4 r3 = loss_pixel(a, D.w, n2.y, n2.z, n2.w, Dg.w, g2.y, g2.z, g2.w, sum);
+        reinterpret_cast<float4*>(a.dLdD)[p] = make_float4(r0.x, r1.x, r2.x, r3.x);
+        float4* op = reinterpret_cast<float4*>(a.dLdN) + 3 * p;
+        op[0] = make_float4(r0.y, r0.z, r0.w, r1.y);
+        op[1] = make_float4(r1.z, r1.w, r2.y, r2.z);
+        op[2] = make_float4(r2.w, r3.y, r3.z, r3.w);
+    }
+    // the pixels outside the quads: [0, head) and the last (HW - head) & 3
+    const long long singles = HW - 4 * quads;
+    for (long long j = tid; j < singles; j += stride) {
+        const long long i = j < head ? j : j + 4 * quads;
+        const long long p = off + i, q = goff + i;
+        const float4 r = loss_pixel(a, __ldg(&a.depth[p]), __ldg(&a.normal[3 * p]),
+                                    __ldg(&a.normal[3 * p + 1]), __ldg(&a.normal[3 * p + 2]),
+                                    __ldg(&a.gt_depth[q]), __ldg(&a.gt_normal[3 * q]),
+                                    __ldg(&a.gt_normal[3 * q + 1]), __ldg(&a.gt_normal[3 * q + 2]), sum);
+        a.dLdD[p] = r.x;
+        a.dLdN[3 * p + 0] = r.y; a.dLdN[3 * p + 1] = r.z; a.dLdN[3 * p + 2] = r.w;
     }
     // block reduction in double
     __shared__ double red[4][8];
-    double x[4] = {sc, sl, sd, cnt};
+    double x[4] = {sum[0], sum[1], sum[2], sum[3]};
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {

@@ -313,6 +313,47 @@ ps_status ps_adam_step(float* param, const float* grad, float* m, float* v, long
                        float lr, float b1, float b2, float eps, int step, float clamp_min,
                        ps_stream stream);
 
+/* Device buffers of one optimisation step (ps_fit_step): what the separate calls take. */
+typedef struct ps_fit_buffers {
+    float* params;            /* [center P x 3 | quat P x 4 | radii P x 4] */
+    float* grad;              /* [11 P], overwritten */
+    float* m;                 /* [11 P] Adam moments */
+    float* v;
+    float* rec;               /* ps_project_cull */
+    int* rect;
+    float* key;
+    int* tile_ptr;            /* ps_bin_tiles */
+    int* tile_ent;
+    float* tile_key;
+    long long capacity;
+    long long* d_required;
+    void* bin_ws;
+    size_t bin_ws_bytes;
+    void* fwd_ws;             /* ps_splat_fwd (separate kernels only) */
+    size_t fwd_ws_bytes;
+    void* bwd_ws;             /* ps_splat_bwd, ps_splat_fused */
+    size_t bwd_ws_bytes;
+    int* d_status;
+    const float* gt_depth;    /* ps_loss, ps_splat_fused */
+    const float* gt_normal;
+    float* depth;             /* separate kernels only */
+    float* normal;
+    float* dL_dD;
+    float* dL_dN;
+    double* view_sums;
+    float* split_acc;         /* [P][2] for ps_radii_grad_accum, or NULL */
+    const float* split_scale; /* [P] or NULL */
+} ps_fit_buffers;
+
+/* One optimisation step (Sec. 3.3) enqueued by one call: ps_project_cull, ps_bin_tiles,
+   the zeroed gradient, ps_splat_fused (or, with fused = 0, ps_splat_fwd without alpha,
+   ps_loss and ps_splat_bwd), ps_radii_grad_accum if split_acc is given, and ps_adam_step on
+   all 11 P parameters, the radii clamped at r_min (NaN: no clamp).  The same results as
+   those calls; the first error of one of them is returned. */
+ps_status ps_fit_step(int n_planes, const ps_frame* frame, const ps_settings* settings,
+                      const ps_fit_buffers* buffers, int fused, float lr, float b1, float b2,
+                      float eps, float r_min, int step, ps_stream stream);
+
 /* Work counts of one forward splat, for throughput and roofline reports:
    d_counts[0] = pairs tested (tile-list entries x pixels of the tile inside the
    image), d_counts[1] = candidate pairs (pairs that pass the w >= w_min and depth

@@ -24,7 +24,7 @@ PS_MAX_M = 64
 
 EXPORTS = ("ps_plan_views", "ps_project_cull", "ps_bin_workspace_bytes", "ps_bin_tiles",
            "ps_fwd_workspace_bytes", "ps_splat_fwd", "ps_splat_ids", "ps_loss", "ps_bwd_workspace_bytes", "ps_splat_bwd",
-           "ps_splat_fused", "ps_adam_step",
+           "ps_splat_fused", "ps_adam_step", "ps_fit_step",
            "ps_count_pairs", "ps_step_advance", "ps_adam_step_state", "ps_gemm_bf16", "ps_wait_selftest",
            "ps_seed_conv_fwd", "ps_seed_backward_ws_bytes", "ps_seed_backward",
            "ps_seed_sync_weights", "ps_seed_im2col", "ps_seed_col2im", "ps_seed_relu_bwd", "ps_seed_transpose",
@@ -69,6 +69,15 @@ class PsPlanes(ctypes.Structure):
                 ("center", ctypes.c_void_p), ("quat", ctypes.c_void_p), ("radii", ctypes.c_void_p)]
 
 
+class PsFitBuffers(ctypes.Structure):
+    _fields_ = [(name, ctypes.c_longlong if name == "capacity" else
+                 ctypes.c_size_t if name.endswith("_bytes") else ctypes.c_void_p)
+                for name in ("params", "grad", "m", "v", "rec", "rect", "key", "tile_ptr", "tile_ent",
+                             "tile_key", "capacity", "d_required", "bin_ws", "bin_ws_bytes", "fwd_ws",
+                             "fwd_ws_bytes", "bwd_ws", "bwd_ws_bytes", "d_status", "gt_depth", "gt_normal",
+                             "depth", "normal", "dL_dD", "dL_dN", "view_sums", "split_acc", "split_scale")]
+
+
 assert ctypes.sizeof(PsView) == 128
 assert ctypes.sizeof(PsSettings) == 64
 assert ctypes.sizeof(PsStepState) == 24
@@ -84,6 +93,8 @@ class PsError(RuntimeError):
 def load():
     """Loads libps.so (built by paper_2412_03451_gb300._build); raises if absent."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -105,6 +116,7 @@ def load():
             "ps_splat_bwd": ([P, P, P, P, P, P, P, LL, P, P, P, P, P, P, SZ, P, P], I),
             "ps_splat_fused": ([P, P, P, P, P, P, P, LL, P, P, P, P, P, P, P, P, P, P, P, SZ, P, P], I),
             "ps_adam_step": ([P, P, P, P, LL, F, F, F, F, I, F, P], I),
+            "ps_fit_step": ([I, P, P, P, I, F, F, F, F, F, I, P], I),
             "ps_count_pairs": ([P, P, P, P, P, P, LL, P, P], I),
             "ps_step_advance": ([P, P, I, P, P], I),
             "ps_gemm_bf16": ([P, P, P, P, P, I, I, I, I, I, I, P, P], I),
@@ -150,15 +162,20 @@ def _check(code: int, what: str):
 
 
 def _ptr(t) -> int | None:
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    """The data pointer of a tensor (a pointer or None as it is)."""
+    return t if t is None or type(t) is int else t.data_ptr()
 
 
-def _stream(stream):
+def _stream(stream) -> int:
+    """The given stream's handle, or that of the current device's current stream.  (The raw
+    handle takes 0.2 us; torch.cuda.current_stream() builds a Stream object in about 3 us, and a
+    call into the library is made up to ten times per eager step.)"""
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if torch.cuda.is_initialized():
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
 
 
 # ---------------------------------------------------------------------------
@@ -311,6 +328,13 @@ def ps_adam_step(param, grad, m, v, lr, b1, b2, eps, step, clamp_min=float("nan"
     _check(load().ps_adam_step(_ptr(param), _ptr(grad), _ptr(m), _ptr(v), param.numel(),
                                float(lr), float(b1), float(b2), float(eps), int(step),
                                float(clamp_min), _stream(stream)), "ps_adam_step")
+
+
+def ps_fit_step(n_planes, frame, settings, buffers: PsFitBuffers, fused, lr, b1, b2, eps, r_min, step,
+                stream=None):
+    """One optimisation step in one call (see ps.h)."""
+    _check(load().ps_fit_step(n_planes, ctypes.byref(frame), ctypes.byref(settings), ctypes.byref(buffers),
+                              int(bool(fused)), lr, b1, b2, eps, r_min, step, _stream(stream)), "ps_fit_step")
 
 
 def ps_count_pairs(frame, settings, rec, key, tile_ptr, tile_ent, capacity, counts, stream=None):

@@ -31,6 +31,14 @@ def flat_views(flat: torch.Tensor, P: int):
     return flat[:3 * P].view(P, 3), flat[3 * P:7 * P].view(P, 4), flat[7 * P:].view(P, 4)
 
 
+def flat_ptrs(flat: torch.Tensor, P: int):
+    """Device pointers of the three groups (flat_views without making the views)."""
+    if flat.is_contiguous() and flat.dtype is torch.float32:
+        p = flat.data_ptr()
+        return p, p + 12 * P, p + 28 * P
+    return tuple(x.data_ptr() for x in flat_views(flat, P))
+
+
 @dataclass
 class StepStats:
     view_sums: torch.Tensor      # [V,4] f64 (device)
@@ -89,6 +97,7 @@ class Renderer:
         self._batches = None
         self._views_tensor = self.views_dev
         self.settings = None
+        self._required_host = None
         # bumped whenever the records / tile lists or the camera descriptors change, so a
         # holder of an earlier render (PlaneSplatFunction) can tell that they are stale
         self.generation = 0
@@ -151,11 +160,7 @@ class Renderer:
         return self.settings
 
     def planes_struct(self, flat: torch.Tensor) -> B.PsPlanes:
-        c, q, r = flat_views(flat, self.P)
-        p = B.PsPlanes()
-        p.n_planes = self.P
-        p.center, p.quat, p.radii = c.data_ptr(), q.data_ptr(), r.data_ptr()
-        return p
+        return B.PsPlanes(self.P, 0, *flat_ptrs(flat, self.P))
 
     # -- the path ----------------------------------------------------------------
     def project_bin(self, flat: torch.Tensor, lam: float, flags=None, d_state=None):
@@ -176,6 +181,25 @@ class Renderer:
             self.status.zero_()
             return True
         return False
+
+    def read_required(self):
+        """Copies the entry count of the last binning to the host without waiting; returns the
+        event after which required_now() may be read."""
+        if self._required_host is None:
+            self._required_host = torch.empty(1, dtype=torch.int64, pin_memory=True)
+        self._required_host.copy_(self.required, non_blocking=True)
+        ready = torch.cuda.Event()
+        ready.record()
+        return ready
+
+    def grow_if_needed(self, headroom=1.5) -> bool:
+        """After read_required()'s event: grows the tile lists if the binning did not fit."""
+        need = int(self._required_host[0])
+        if need <= self.capacity:
+            return False
+        self._alloc_lists(int(need * headroom) + 1024)
+        self.status.zero_()
+        return True
 
     def splat_forward(self, alpha=True):
         B.ps_splat_fwd(self.frame, self.settings, self.rec, self.tile_key, self.tile_ptr, self.tile_ent,
@@ -212,7 +236,7 @@ class Renderer:
         Accumulates the loss gradient into grad_flat; fills view_sums; writes
         depth/normal/dL maps only if write_maps."""
         pl = self.planes_struct(flat)
-        gc, gq, gr = flat_views(grad_flat, self.P)
+        gc, gq, gr = flat_ptrs(grad_flat, self.P)
         m = write_maps
         B.ps_splat_fused(pl, self.frame, self.settings, self.rec, self.tile_key, self.tile_ptr,
                          self.tile_ent, self.capacity, gt_depth, gt_normal,
@@ -225,7 +249,7 @@ class Renderer:
     def backward(self, flat: torch.Tensor, grad_flat: torch.Tensor, dLdD=None, dLdN=None):
         """Accumulates d(sum dLdD*D + dLdN.N)/dparams into grad_flat (same layout)."""
         pl = self.planes_struct(flat)
-        gc, gq, gr = flat_views(grad_flat, self.P)
+        gc, gq, gr = flat_ptrs(grad_flat, self.P)
         B.ps_splat_bwd(pl, self.frame, self.settings, self.rec, self.tile_key, self.tile_ptr,
                        self.tile_ent, self.capacity, self.dLdD if dLdD is None else dLdD,
                        self.dLdN if dLdN is None else dLdN, gc, gq, gr, self.bwd_ws, self.status)
@@ -251,15 +275,24 @@ class PlaneSplatFunction(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, flat, renderer: Renderer, lam: float, flags=None):
-        if renderer.ensure_capacity(flat, lam, flags):
-            renderer.project_bin(flat, lam, flags)      # the lists of the grown buffers
+        # the splat is enqueued behind the binning before the host knows whether the lists fitted
+        # (it stays within them either way), so that the device does not wait for the host
+        renderer.project_bin(flat, lam, flags)
+        ready = renderer.read_required()
         renderer.splat_forward(alpha=False)
+        depth, normal = renderer.depth.clone(), renderer.normal.clone()
+        ctx.views = renderer.views_snapshot()
+        ready.synchronize()
+        if renderer.grow_if_needed():
+            renderer.project_bin(flat, lam, flags)      # the lists of the grown buffers
+            renderer.splat_forward(alpha=False)
+            depth.copy_(renderer.depth)
+            normal.copy_(renderer.normal)
         ctx.renderer = renderer
         ctx.lam, ctx.flags = lam, flags
         ctx.generation = renderer.generation
-        ctx.views = renderer.views_snapshot()
         ctx.save_for_backward(flat)
-        return renderer.depth.clone(), renderer.normal.clone()
+        return depth, normal
 
     @staticmethod
     def backward(ctx, gD, gN):
@@ -395,6 +428,28 @@ class Fitter:
         self.ite += 1
         return self.graph_sums[batch_index]
 
+    def _native_step(self, gt_depth, gt_normal, lam, batch) -> bool:
+        """The whole step as one library call (False: not for these buffers)."""
+        r = self.r
+        state = (self.flat, self.grad, self.m, self.v)
+        if not all(t.is_contiguous() and t.dtype is torch.float32 and t.numel() == 11 * r.P for t in state):
+            return False
+        maps = (None,) * 4 if self.fused else (x.data_ptr() for x in (r.depth, r.normal, r.dLdD, r.dLdN))
+        acc = self.split_acc
+        buf = B.PsFitBuffers(
+            *(t.data_ptr() for t in state), r.rec.data_ptr(), r.rect.data_ptr(), r.key.data_ptr(),
+            r.tile_ptr.data_ptr(), r.tile_ent.data_ptr(), r.tile_key.data_ptr(), r.capacity,
+            r.required.data_ptr(), r.bin_ws.data_ptr(), 4 * r.bin_ws.numel(), r.fwd_ws.data_ptr(),
+            4 * r.fwd_ws.numel(), r.bwd_ws.data_ptr(), 4 * r.bwd_ws.numel(), r.status.data_ptr(),
+            gt_depth.data_ptr(), gt_normal.data_ptr(), *maps, r.view_sums.data_ptr(),
+            None if acc is None else acc.data_ptr(),
+            None if acc is None else B._ptr(self.split_scale[batch or 0]))
+        r.generation += 1
+        B.ps_fit_step(r.P, r.frame, r.make_settings(lam), buf, self.fused, self.lr, self.b1, self.b2,
+                      self.eps, R_MIN, self.ite + 1)
+        self.ite += 1
+        return True
+
     def step(self, gt_depth, gt_normal, lam=None, marks=None, batch=None):
         """One iteration.  If marks is a list, CUDA events are recorded on the
         current stream after each stage as (name, event) pairs."""
@@ -406,6 +461,8 @@ class Fitter:
 
         lam = B.lambda_schedule(self.ite + self.lam_offset) if lam is None else lam
         r = self.r
+        if marks is None and self._native_step(gt_depth, gt_normal, lam, batch):
+            return r.view_sums
         mark("start")
         r.project_bin(self.flat, lam)
         mark("project_bin")

@@ -120,8 +120,9 @@ __device__ __forceinline__ bool eval_pair(const float4& n, const float4& vx, con
     // w = min(1, 2 sigmoid(5 lambda m)); below the clamp 2 sigmoid(x) = 2 e^x / (1 + e^x)
     const float e = __expf(c.lam5 * m);
     const float w = (m >= 0.f) ? 1.f : __fdividef(2.f * e, 1.f + e);
-    const bool ok = (fabsf(den) > 1e-6f) && (t > c.z_near && t < c.z_far) && !(m < -c.reject) &&
-                    (m >= 0.f || !c.hard) && (w >= c.w_min);
+    // (hard edge: w = 1 for m >= 0, which is then the only condition on it)
+    const bool ok = (fabsf(den) > 1e-6f) && (t > c.z_near && t < c.z_far) &&
+                    (c.hard ? m >= 0.f : (!(m < -c.reject) && (w >= c.w_min)));
     o.t = t; o.w = w; o.m = m; o.den = den;
     o.sideX = sx;
     o.P = sx ? X : Y;

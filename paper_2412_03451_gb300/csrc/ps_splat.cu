@@ -72,14 +72,17 @@ constexpr int kDefaultWarps = 4;
 // Resident CTAs per SM the register allocation is sized for: 24 warps per SM for
 // the forward-only kernel (measured 8% faster than 20), 20 for the modes with the
 // backward, where 24 would spill.
-__host__ __device__ constexpr int min_blocks(int mode, int warps)
+__host__ __device__ constexpr int min_blocks(int mode, int form, int warps)
 {
-    return (mode == 0 ? 24 : 20) / warps;
+    return (form == 2 ? 40 : mode == 0 ? 24 : 20) / warps;
 }
 
 // Kernel modes: forward only; backward from given dL/dD, dL/dN; or forward,
 // Eq. 14 loss and backward fused in one walk per pixel.
 constexpr int kFwd = 0, kBwd = 1, kFused = 2;
+
+// Weight forms: Eq. 7-9, Eq. 5, and the hard edge (forward only).
+constexpr int kRect = 0, kGauss = 1, kHard = 2;
 
 // Fused mode: per-view loss sums are added into kSlots partial sums per view
 // (spread over L2 slices, so that strips of one view do not serialise on one
@@ -101,7 +104,8 @@ struct SplatArgs {
     long long capacity;
     SplatConst c;
     int M;
-    int n_items;              // strips = n_tiles * (tile pixels / 32)
+    int n_items;              // strips = n_tiles * (tile pixels / 32), or groups of them
+    int group;                // strips of a tile per item (hard edge)
     int* counter;             // work counter (zeroed before the launch)
     const ps_step_state* d_state;   // if set, lambda and delta come from here
     // forward outputs
@@ -478,7 +482,7 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
             if (gD == 0.f && gN0 == 0.f && gN1 == 0.f && gN2 == 0.f) s.done = true;
         }
     }
-    walk_strip<MODE, KP, G != 0>(a, ws, s, k, dx, dy, g, beg, end);
+    walk_strip<MODE, KP, G == kGauss>(a, ws, s, k, dx, dy, g, beg, end);
 
     if constexpr (MODE != kBwd) {
         if (inside) {
@@ -651,6 +655,101 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
     return out;
 }
 
+// Hard edge, forward, strips s0 .. s1 - 1 of one tile.  Every candidate is opaque, so a
+// pixel's composite is its nearest candidate by (t, id): no buffer and no transmittance, and
+// few registers (40 warps per SM).  The pixel is done once the bound on the later depths
+// passes its pair.  What the strips share is set up once: view, column rays, and the staged
+// list where it is one chunk.  64 views of 640x480, 2,000 planes, 16x16 tiles: 564 us in the
+// general walk, about 195 here (the maps' 16 bytes per pixel alone take 47 us).
+template <int TW, int TH>
+__device__ __forceinline__ void run_hard(const SplatArgs& a, WarpStage& ws, int tile, int s0, int s1)
+{
+    constexpr int WX = TW < 32 ? TW : 32, WY = 32 / WX;
+    const float kMargin = 1.f - 1.f / 4096.f;
+    const int lane = threadIdx.x & 31;
+    const int v = warp_view_of_tile(a.views, a.n_views, tile);
+    const ps_view* vw = a.views + v;
+    const int W = __ldg(&vw->W), H = __ldg(&vw->H);
+    const int tx_n = __ldg(&vw->tiles_x);
+    const int lt = tile - __ldg(&vw->tile_off);
+    const int px = (lt % tx_n) * TW + lane % WX, ty0 = (lt / tx_n) * TH + lane / WX;
+    const float fy = __ldg(&vw->fy), cy = __ldg(&vw->cy);
+    const float dx = __fdiv_rn((float)px + 0.5f - __ldg(&vw->cx), __ldg(&vw->fx));
+    const long long pix0 = __ldg(&vw->pix_off) + px;
+    const int id0 = __ldg(&vw->plane_off) - __ldg(&vw->rec_off);
+    WarpRegion g;
+    g.dxa = __shfl_sync(kFull, dx, 0); g.dxb = __shfl_sync(kFull, dx, WX - 1);
+    g.den_min = 0.f;
+    const int beg = (int)min((long long)__ldg(&a.tile_ptr[tile]), a.capacity);
+    const int end = (int)min((long long)__ldg(&a.tile_ptr[tile + 1]), a.capacity);
+    const bool one = end - beg <= 32;
+    auto stage = [&](int base) {
+        __syncwarp();                              // the last chunk has been read
+        const int i = base + lane;
+        if (i < end) {
+            const int id = __ldg(&a.tile_ent[i]);
+            const float4* r = a.rec + (size_t)id * 4;
+            ws.id[lane] = id;
+            ws.key[lane] = __ldg(&a.key[i]) * kMargin;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) ws.rec[c][lane] = __ldg(r + c);
+        }
+        if (lane == 0) ws.key[32] = (base + 32 < end) ? __ldg(&a.key[base + 32]) * kMargin : INFINITY;
+        __syncwarp();
+    };
+    if (one) stage(beg);
+    for (int s = s0; s < s1; ++s) {
+        const int py = ty0 + s * WY;
+        const bool inside = px < W && py < H;
+        const float dy = __fdiv_rn((float)py + 0.5f - cy, fy);
+        g.dya = __shfl_sync(kFull, dy, 0); g.dyb = __shfl_sync(kFull, dy, 31);
+        CKey best = kNoKey;
+        float N0 = 0.f, N1 = 0.f, N2 = 0.f;
+        bool all_done = false;
+        for (int base = beg; base < end && !all_done; base += 32) {
+            if (!one) stage(base);
+            float t_low;
+            const bool ok = base + lane < end &&
+                            region_may_hit<false>(ws.rec[0][lane], ws.rec[1][lane], ws.rec[2][lane],
+                                                  ws.rec[3][lane], g, a.c, t_low);
+            unsigned m = __ballot_sync(kFull, ok);
+            while (m) {
+                const int e = __ffs(m) - 1;
+                m &= m - 1;
+                // (a pixel that is done may meet later pairs: none of them comes before its own)
+                PairEval pe;
+                const float4 n = ws.rec[0][e];
+                if (eval_pair(n, ws.rec[1][e], ws.rec[2][e], ws.rec[3][e], dx, dy, a.c, pe)) {
+                    const CKey key = ckey(pe.t, ws.id[e]);
+                    if (key < best) {
+                        best = key;
+                        N0 = n.x; N1 = n.y; N2 = n.z;
+                    }
+                }
+                // (no candidate yet: its depth reads NaN, the comparison is false)
+                const float bound = ws.key[m ? __ffs(m) - 1 : 32];
+                if (m) all_done = __all_sync(kFull, !inside || bound > key_t(best));
+                if (all_done) break;
+            }
+            if (!one && !all_done) all_done = __all_sync(kFull, !inside || ws.key[32] > key_t(best));
+        }
+        if (inside) {
+            const long long pix = pix0 + (long long)py * W;
+            const bool hit = best != kNoKey;
+            if (a.depth) a.depth[pix] = hit ? key_t(best) : 0.f;
+            if (a.normal) {
+                // 0 + 1 n, the compositing sum (-0 becomes 0)
+                a.normal[3 * pix + 0] = N0 + 0.f;
+                a.normal[3 * pix + 1] = N1 + 0.f;
+                a.normal[3 * pix + 2] = N2 + 0.f;
+            }
+            if (a.alpha) a.alpha[pix] = hit ? 1.f : 0.f;
+            if (a.ids) a.ids[pix] = hit ? key_id(best) + id0 : -1;
+        }
+    }
+    __syncwarp();
+}
+
 // Persistent warps: each takes strips from the work counter until none is left.
 // lambda and the quick-reject margin from the device state (graph replay)
 __device__ __forceinline__ void load_state(SplatArgs& a)
@@ -661,14 +760,15 @@ __device__ __forceinline__ void load_state(SplatArgs& a)
     }
 }
 
-// G: the weight form of the instantiation (0: Eq. 7-9 rectangle weight, 1: Eq. 5 Gaussian),
-// fixed at compile time so that the other form's branches fold away.
+// G: the weight form of the instantiation, fixed at compile time so that the other forms'
+// branches fold away.
 template <int TW, int TH, int MODE, int NW, int G>
-__global__ void __launch_bounds__(NW * 32, min_blocks(MODE, NW)) k_splat(SplatArgs a_in)
+__global__ void __launch_bounds__(NW * 32, min_blocks(MODE, G, NW)) k_splat(SplatArgs a_in)
 {
-    constexpr int KP = G ? kPendGauss : kPendRect;
+    constexpr int KP = G == kGauss ? kPendGauss : kPendRect;
     SplatArgs a = a_in;
-    a.c.gauss = G;
+    a.c.gauss = G == kGauss;
+    a.c.hard = G == kHard;
     load_state(a);
     __shared__ WarpStage stage[NW];
     extern __shared__ int2 dyn_stk[];       // backward: [NW][M][32]
@@ -702,6 +802,12 @@ __global__ void __launch_bounds__(NW * 32, min_blocks(MODE, NW)) k_splat(SplatAr
         if (lane == 0) item = atomicAdd(a.counter, 1);
         item = __shfl_sync(kFull, item, 0);
         if (item >= a.n_items) break;
+        if constexpr (G == kHard) {
+            constexpr int NS = TW * TH / 32;
+            const int per = NS / a.group, tile = item / per, s0 = (item - tile * per) * a.group;
+            run_hard<TW, TH>(a, stage[w], tile, s0, s0 + a.group);
+            continue;
+        }
         const StripLoss sl = run_strip<TW, TH, MODE, KP, G>(a, stage[w], stk_warp, item);
         if constexpr (MODE == kFused) {
             if (sl.v != vcur) {
@@ -1013,6 +1119,15 @@ cudaError_t launch_splat(SplatArgs a, int n_tiles, int M, cudaStream_t st, bool 
         c.dyn = dyn;
         c.blocks_per_sm = (nb > 0 ? nb : 1) * sms;
     }
+    a.group = 1;
+    if constexpr (G == kHard) {
+        // A strip is so short that the one work counter binds (a render of 614,400 strips takes
+        // 474 us one by one, 367 in pairs, 263 by tiles that share their setup): groups as large
+        // as leave every warp four items.
+        const long long warps = (long long)c.blocks_per_sm * NW;
+        while (a.group < NS && a.n_items / (2 * a.group) >= 4 * warps) a.group *= 2;
+        a.n_items /= a.group;
+    }
     int blocks = c.blocks_per_sm;
     const int need = (a.n_items + NW - 1) / NW;
     if (blocks > need) blocks = need;
@@ -1082,8 +1197,11 @@ template <int MODE>
 cudaError_t dispatch(const SplatArgs& a, const ps_settings* s, int n_tiles, cudaStream_t st,
                      bool counter_zeroed = false)
 {
-    if (s->flags & PS_GAUSSIAN) return dispatch_warps<MODE, 1>(a, s, n_tiles, st, counter_zeroed);
-    return dispatch_warps<MODE, 0>(a, s, n_tiles, st, counter_zeroed);
+    if (s->flags & PS_GAUSSIAN) return dispatch_warps<MODE, kGauss>(a, s, n_tiles, st, counter_zeroed);
+    if constexpr (MODE == kFwd) {
+        if (s->flags & PS_HARD) return dispatch_warps<MODE, kHard>(a, s, n_tiles, st, counter_zeroed);
+    }
+    return dispatch_warps<MODE, kRect>(a, s, n_tiles, st, counter_zeroed);
 }
 
 template <int TW, int TH>

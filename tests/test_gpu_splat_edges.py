@@ -104,3 +104,70 @@ def test_gauss_maps_do_not_depend_on_the_tile(lists):
     assert float(out[0][0].abs().sum()) > 0
     for D, N in out[1:]:
         assert torch.equal(D, out[0][0]) and torch.equal(N, out[0][1])
+
+
+@pytest.mark.parametrize("tile", [(8, 8), (16, 16), (32, 8)])
+@pytest.mark.parametrize("V,warps,K", [(1, 0, 150), (5, 2, 150), (13, 8, 150), (27, 0, 150), (27, 0, 6)])
+def test_hard_maps_by_groups_of_strips(tile, V, warps, K):
+    # the more views, the more strips of a tile per work item (1, 2, 4 or 8); lists of one chunk and
+    # of several, a ragged image, pixels without any plane; each view against its own render
+    import torch
+    from paper_2412_03451_gb300 import binding as B, splat as SP
+    p = S.random_planes_in_view(17, K, depth_range=(0.3, 3.0), half=(0.05, 0.7))
+    p.center[1], p.quat[1], p.radii[1] = p.center[0], p.quat[0], p.radii[0]     # a tie: the lower id
+    h, w = 470, 629
+    cams = S.identity_cameras(V, h, w, 400.0, seed=4, jitter=0.1)
+    flat = SP.planes_to_flat(p.center, p.quat, p.radii, "cuda")
+
+    def maps(views, **kw):
+        k = len(views)
+        r = SP.Renderer([h] * k, [w] * k, [0] * k, [0, p.K], flags=B.PS_HARD, **kw)
+        r.set_cameras(cams.w2c[views], cams.intr[views])
+        r.ensure_capacity(flat, 20.0)
+        D, N = (x.clone() for x in r.forward(flat, 20.0))
+        A = r.alpha.clone()
+        ids, D2 = r.plane_ids(flat)
+        assert torch.equal(D, D2) and torch.equal(A, (D > 0).float()) and torch.equal(ids >= 0, D > 0)
+        assert int(r.status.item()) == 0 and not (ids == 1).any()
+        return D.view(k, -1), N.view(k, -1), ids.view(k, -1)
+
+    got = maps(list(range(V)), tile=tile, warps=warps)
+    covered = float((got[0] > 0).float().mean())
+    assert 0 < covered and (covered < 1 or K == 150)
+    for v in sorted({0, V // 2, V - 1}):
+        one = maps([v])
+        for a, b in zip(got, one):
+            assert torch.equal(a[v], b[0]), v
+    # the nearest candidate by definition, in FP64, at sampled pixels away from edges and ties
+    v, rng = V - 1, np.random.default_rng(3)
+    D, ids = got[0][v].cpu().numpy(), got[2][v].cpu().numpy()
+    K, T = cams.intr[v].astype(np.float64), cams.w2c[v].astype(np.float64)
+    q = p.quat.astype(np.float64) / np.linalg.norm(p.quat, axis=1, keepdims=True)
+    a, b, c, d = q.T
+    vx = np.stack([1 - 2 * (c * c + d * d), 2 * (b * c + a * d), 2 * (b * d - a * c)], 1) @ T[:, :3].T
+    vy = np.stack([2 * (b * c - a * d), 1 - 2 * (b * b + d * d), 2 * (c * d + a * b)], 1) @ T[:, :3].T
+    n = np.cross(vx, vy)
+    pc = p.center.astype(np.float64) @ T[:, :3].T + T[:, 3]
+    checked = 0
+    for x, y in zip(rng.integers(0, w, 400), rng.integers(0, h, 400)):
+        ray = np.array([(x + 0.5 - K[2]) / K[0], (y + 0.5 - K[3]) / K[1], 1.0])
+        den = n @ ray
+        t = (n * pc).sum(1) / den
+        o = t[:, None] * ray - pc
+        X, Y = (o * vx).sum(1), (o * vy).sum(1)
+        r = p.radii.astype(np.float64)
+        m = np.minimum(np.where(X > 0, r[:, 0], r[:, 1]) - abs(X), np.where(Y > 0, r[:, 2], r[:, 3]) - abs(Y))
+        near = (abs(den) > 1e-3) & (t > 0.02) & (t < 99)
+        if (near & (abs(m) < 1e-3)).any() or (~near & (m > -1e-3)).any():
+            continue
+        hit = np.where(near & (m >= 0))[0]
+        if len(hit) == 0:
+            assert ids[y * w + x] == -1
+        else:
+            order = hit[np.argsort(t[hit], kind="stable")]
+            gap = [k for k in order if t[k] > t[order[0]] + 1e-4]
+            if len(order) - len(gap) > (2 if order[0] in (0, 1) else 1):
+                continue
+            assert ids[y * w + x] == order[0] and abs(D[y * w + x] - t[order[0]]) < 1e-4
+        checked += 1
+    assert checked > 100

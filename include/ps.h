@@ -343,13 +343,20 @@ typedef struct ps_fit_buffers {
     double* view_sums;
     float* split_acc;         /* [P][2] for ps_radii_grad_accum, or NULL */
     const float* split_scale; /* [P] or NULL */
+    ps_step_state* d_state;   /* ps_step_advance before the step, or d_sched NULL */
+    const ps_step_state* d_sched;
+    int n_sched;
+    int reserved;
+    int* d_iter;
 } ps_fit_buffers;
 
-/* One optimisation step (Sec. 3.3) enqueued by one call: ps_project_cull, ps_bin_tiles,
-   the zeroed gradient, ps_splat_fused (or, with fused = 0, ps_splat_fwd without alpha,
-   ps_loss and ps_splat_bwd), ps_radii_grad_accum if split_acc is given, and ps_adam_step on
-   all 11 P parameters, the radii clamped at r_min (NaN: no clamp).  The same results as
-   those calls; the first error of one of them is returned. */
+/* One optimisation step (Sec. 3.3) enqueued by one call: ps_step_advance if d_sched is given,
+   ps_project_cull, ps_bin_tiles, the zeroed gradient, ps_splat_fused (or, with fused = 0,
+   ps_splat_fwd without alpha, ps_loss and ps_splat_bwd), ps_radii_grad_accum if split_acc is
+   given, and ps_adam_step on all 11 P parameters (with the bias corrections of
+   settings->d_state if that is set), the radii clamped at r_min (NaN: no clamp).  The results
+   of those calls, with fewer launches; the first error of one of them is returned.  n_planes
+   is the number of planes of all scenes. */
 ps_status ps_fit_step(int n_planes, const ps_frame* frame, const ps_settings* settings,
                       const ps_fit_buffers* buffers, int fused, float lr, float b1, float b2,
                       float eps, float r_min, int step, ps_stream stream);

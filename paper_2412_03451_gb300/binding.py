@@ -71,11 +71,13 @@ class PsPlanes(ctypes.Structure):
 
 class PsFitBuffers(ctypes.Structure):
     _fields_ = [(name, ctypes.c_longlong if name == "capacity" else
+                 ctypes.c_int if name in ("n_sched", "reserved") else
                  ctypes.c_size_t if name.endswith("_bytes") else ctypes.c_void_p)
                 for name in ("params", "grad", "m", "v", "rec", "rect", "key", "tile_ptr", "tile_ent",
                              "tile_key", "capacity", "d_required", "bin_ws", "bin_ws_bytes", "fwd_ws",
                              "fwd_ws_bytes", "bwd_ws", "bwd_ws_bytes", "d_status", "gt_depth", "gt_normal",
-                             "depth", "normal", "dL_dD", "dL_dN", "view_sums", "split_acc", "split_scale")]
+                             "depth", "normal", "dL_dD", "dL_dN", "view_sums", "split_acc", "split_scale",
+                             "d_state", "d_sched", "n_sched", "reserved", "d_iter")]
 
 
 assert ctypes.sizeof(PsView) == 128

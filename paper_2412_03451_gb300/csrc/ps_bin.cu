@@ -100,40 +100,14 @@ inline size_t ws_bytes(int R, int n_tiles, long long capacity)
 
 // 1. record counts ---------------------------------------------------------------
 __global__ void __launch_bounds__(128) k_rec_count(const int4* __restrict__ rect,
-                                                    const ps_view* __restrict__ views,
-                                                    int* __restrict__ rec_cnt,
-                                                    int4* __restrict__ rec_info,
-                                                    int* __restrict__ diff, int n_tiles)
+                                                   const ps_view* __restrict__ views, BinCount count)
 {
     const int v = blockIdx.y;
     const ps_view* vw = views + v;
-    const int K = __ldg(&vw->K);
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    const int r = __ldg(&vw->rec_off) + k;
-    const int4 rc = __ldg(&rect[r]);
-    const int tx = __ldg(&vw->tiles_x);
-    int c = 0;
-    int4 info = make_int4(0, 1, tx, v);
-    if (rc.z >= rc.x && rc.w >= rc.y) {
-        const int w = rc.z - rc.x + 1;
-        c = w * (rc.w - rc.y + 1);
-        const int first = __ldg(&vw->tile_off) + rc.y * tx + rc.x;
-        info = make_int4(first, w, tx, v);
-        if (w == tx) {
-            // full rows: one contiguous run of c tiles
-            atomicAdd(&diff[first], 1);
-            if (first + c < n_tiles) atomicAdd(&diff[first + c], -1);
-        } else {
-            const int last = first + (rc.w - rc.y) * tx;   // first tile of the last row
-            for (int a = first; a <= last; a += tx) {
-                atomicAdd(&diff[a], 1);
-                if (a + w < n_tiles) atomicAdd(&diff[a + w], -1);
-            }
-        }
-    }
-    rec_cnt[r] = c;
-    rec_info[r] = info;
+    if (k >= __ldg(&vw->K)) return;
+    const size_t r = (size_t)__ldg(&vw->rec_off) + k;
+    count_record(count, r, __ldg(&rect[r]), __ldg(&vw->tile_off), __ldg(&vw->tiles_x), v);
 }
 
 // 2. scans ------------------------------------------------------------------------
@@ -576,32 +550,41 @@ extern "C" size_t ps_bin_workspace_bytes(const ps_frame* frame, long long capaci
     return ws_bytes(frame->n_records, frame->n_tiles, capacity);
 }
 
-extern "C" ps_status ps_bin_tiles(const ps_frame* frame, const ps_settings* s, const float* rec,
-                                  const int* rect, const float* key, int* tile_ptr, int* tile_ent,
-                                  float* tile_key, long long capacity, long long* d_required,
-                                  void* ws, size_t ws_bytes_, int* d_status, ps_stream stream)
+ps_status ps::bin_count(const ps_frame* frame, long long capacity, void* ws, size_t ws_bytes_, BinCount* out)
+{
+    if (!frame || !ws || frame->n_tiles <= 0 || frame->n_records < 0) return PS_ERR_ARG;
+    if (capacity < 0 || capacity >= (1LL << 31) - 1) return PS_ERR_ARG;
+    if (ws_bytes_ < ws_bytes(frame->n_records, frame->n_tiles, capacity)) return PS_ERR_ARG;
+    if (reinterpret_cast<uintptr_t>(ws) & 255) return PS_ERR_ARG;
+    const BinWs w = carve(ws, frame->n_records, frame->n_tiles, capacity, nullptr);
+    *out = BinCount{w.rec_cnt, w.rec_info, w.tile_cnt, frame->n_tiles};
+    return PS_OK;
+}
+
+ps_status ps::bin_tiles(const ps_frame* frame, const ps_settings* s, const float* rec, const int* rect,
+                        const float* key, int* tile_ptr, int* tile_ent, float* tile_key, long long capacity,
+                        long long* d_required, void* ws, size_t ws_bytes_, bool counted, int* d_status,
+                        cudaStream_t st)
 {
     if (!frame || !s || !rec || !rect || !key || !tile_ptr || !d_required || !ws || !frame->views)
         return PS_ERR_ARG;
-    if (capacity < 0 || capacity >= (1LL << 31) - 1) return PS_ERR_ARG;
     if (capacity > 0 && (!tile_ent || !tile_key)) return PS_ERR_ARG;
     if (s->tile_w <= 0 || s->tile_h <= 0 || !(s->z_near > 0.f)) return PS_ERR_ARG;
     if (reinterpret_cast<uintptr_t>(rec) & 15) return PS_ERR_ARG;
-    if (frame->n_tiles <= 0 || frame->n_records < 0) return PS_ERR_ARG;
-    const int R = frame->n_records;
-    if (ws_bytes_ < ws_bytes(R, frame->n_tiles, capacity)) return PS_ERR_ARG;
-    if (reinterpret_cast<uintptr_t>(ws) & 255) return PS_ERR_ARG;
     if (reinterpret_cast<uintptr_t>(rect) & 15) return PS_ERR_ARG;
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    BinCount cnt;
+    const ps_status e = bin_count(frame, capacity, ws, ws_bytes_, &cnt);
+    if (e != PS_OK) return e;
+    const int R = frame->n_records;
     BinWs w = carve(ws, R, frame->n_tiles, capacity, nullptr);
-    PS_CUDA_CHECK(cudaMemsetAsync(w.tile_cnt, 0, sizeof(int) * (size_t)frame->n_tiles, st));
-    const int4* rc = reinterpret_cast<const int4*>(rect);
     const long long nch = n_chunks(capacity);
-    if (R > 0) {
-        dim3 grid((frame->max_K + 127) / 128, frame->n_views);
-        k_rec_count<<<grid, 128, 0, st>>>(rc, frame->views, w.rec_cnt, w.rec_info, w.tile_cnt,
-                                          frame->n_tiles);
-        PS_LAUNCH_CHECK();
+    if (!counted) {
+        PS_CUDA_CHECK(cudaMemsetAsync(w.tile_cnt, 0, sizeof(int) * (size_t)frame->n_tiles, st));
+        if (R > 0) {
+            dim3 grid((frame->max_K + 127) / 128, frame->n_views);
+            k_rec_count<<<grid, 128, 0, st>>>(reinterpret_cast<const int4*>(rect), frame->views, cnt);
+            PS_LAUNCH_CHECK();
+        }
     }
     // Pair numbering: offsets clamp at the int range (still non-decreasing), so pairs
     // past it are never scattered, and the tile total then exceeds every capacity.
@@ -627,4 +610,13 @@ extern "C" ps_status ps_bin_tiles(const ps_frame* frame, const ps_settings* s, c
         PS_LAUNCH_CHECK();
     }
     return PS_OK;
+}
+
+extern "C" ps_status ps_bin_tiles(const ps_frame* frame, const ps_settings* s, const float* rec,
+                                  const int* rect, const float* key, int* tile_ptr, int* tile_ent,
+                                  float* tile_key, long long capacity, long long* d_required,
+                                  void* ws, size_t ws_bytes_, int* d_status, ps_stream stream)
+{
+    return ps::bin_tiles(frame, s, rec, rect, key, tile_ptr, tile_ent, tile_key, capacity, d_required, ws,
+                         ws_bytes_, false, d_status, reinterpret_cast<cudaStream_t>(stream));
 }

@@ -199,6 +199,136 @@ __device__ __forceinline__ bool region_may_hit(const float4& n, const float4& vx
     return true;
 }
 
+// Floats per record of the gradient accumulators: the gradients of s (0), of a turn about
+// v^y (1) and about -v^x (2) that moves n_c, of a turn about n_c (3), of the radii (4-7),
+// and for the Eq. 5 weight those of a_x and a_y (8, 9; the rectangle's follow from the radii).
+__host__ __device__ constexpr int grad_stride(int gauss) { return gauss ? 12 : 8; }
+
+// Fused mode: per-view loss sums are added into kSlots partial sums per view
+// (spread over L2 slices, so that strips of one view do not serialise on one
+// address), which the chain kernel adds up into view_sums.
+constexpr int kSlots = 32;
+
+__device__ __forceinline__ double slot_sum(const double* vs_slots, int v, int c)
+{
+    const double* sp = vs_slots + (size_t)v * kSlots * 4 + c;
+    double t = 0.0;
+    for (int i = 0; i < kSlots; ++i) t += sp[4 * i];        // in a fixed order
+    return t;
+}
+
+// A plane's record gradients (sums over any of its records) -> world parameters (Eq. 2-3 and
+// the quaternion normalisation): out = center 3, quaternion 4, radii 4.  Returns false for a
+// quaternion without a direction.
+__device__ __forceinline__ bool chain_plane(const float4& g0, const float4& g3, float gax, float gay,
+                                            float q0, float q1, float q2, float q3, int single_radii,
+                                            float (&out)[11])
+{
+    const float qs = sqrtf(q0 * q0 + q1 * q1 + q2 * q2 + q3 * q3);
+    if (!(qs > 0.f) || !isfinite(qs)) return false;
+    const float w = q0 / qs, x = q1 / qs, y = q2 / qs, z = q3 / qs;
+    // world axes: columns of the Hamilton matrix (Eq. 2-3)
+    const float vx[3] = {1.f - 2.f * (y * y + z * z), 2.f * (x * y + w * z), 2.f * (x * z - w * y)};
+    const float vy[3] = {2.f * (x * y - w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z + w * x)};
+    const float nn[3] = {2.f * (x * z + w * y), 2.f * (y * z - w * x), 1.f - 2.f * (x * x + y * y)};
+    // The centre moves s = n_c . p_c, a_x and a_y; the camera rotation takes n_c, v^x_c, v^y_c
+    // back to the world axes, so the world gradient is their combination.
+#pragma unroll
+    for (int i = 0; i < 3; ++i) out[i] = g0.x * nn[i] + gax * vx[i] + gay * vy[i];
+    // A turn by theta in the plane's own frame moves v^x by theta_z v^y - theta_y n, v^y by
+    // theta_x n - theta_z v^x and n by theta_y v^x - theta_x v^y.  At a fixed centre the
+    // gradient of n lies along v^x (g0.y) and v^y (g0.z), those of v^x and v^y in the plane
+    // with the moment g0.w about n; parts along an axis itself do not turn it.  With
+    // dq = q (0, theta) / 2 the quaternion gradient is 2 q (0, torque) / |q|.
+    const float tx = -g0.z, ty = g0.y, tz = g0.w;
+    const float s2 = 2.f / qs;
+    out[3] = s2 * -(x * tx + y * ty + z * tz);
+    out[4] = s2 * (w * tx + y * tz - z * ty);
+    out[5] = s2 * (w * ty + z * tx - x * tz);
+    out[6] = s2 * (w * tz + x * ty - y * tx);
+    out[7] = single_radii ? g3.x + g3.y : g3.x;
+    out[8] = single_radii ? 0.f : g3.y;
+    out[9] = single_radii ? g3.z + g3.w : g3.z;
+    out[10] = single_radii ? 0.f : g3.w;
+    return true;
+}
+
+// Adam with bias correction; values below `lowest` (NaN: none) are raised to it.
+__device__ __forceinline__ void adam_update(float* __restrict__ p, float* __restrict__ m,
+                                            float* __restrict__ v, long long i, float gi, float lr, float b1,
+                                            float b2, float eps, float bc1, float bc2, float lowest)
+{
+    const float mi = fmaf(b1, m[i], (1.f - b1) * gi);
+    const float vi = fmaf(b2, v[i], (1.f - b2) * gi * gi);
+    m[i] = mi;
+    v[i] = vi;
+    const float mh = mi / bc1, vh = vi / bc2;
+    float pi = p[i] - lr * mh / (sqrtf(vh) + eps);
+    if (pi < lowest) pi = lowest;
+    p[i] = pi;
+}
+
+// Record r's part in the binning's counts: its number of tiles, where they start, and +1 / -1
+// in the difference array where each row segment of its rectangle starts and ends.
+struct BinCount {
+    int* rec_cnt;
+    int4* rec_info;
+    int* diff;
+    int n_tiles;
+};
+
+__device__ __forceinline__ void count_record(const BinCount& b, size_t r, const int4& rc, int tile_off, int tx,
+                                             int v)
+{
+    int c = 0;
+    int4 info = make_int4(0, 1, tx, v);
+    if (rc.z >= rc.x && rc.w >= rc.y) {
+        const int w = rc.z - rc.x + 1;
+        c = w * (rc.w - rc.y + 1);
+        const int first = tile_off + rc.y * tx + rc.x;
+        info = make_int4(first, w, tx, v);
+        if (w == tx) {
+            // full rows: one contiguous run of c tiles
+            atomicAdd(&b.diff[first], 1);
+            if (first + c < b.n_tiles) atomicAdd(&b.diff[first + c], -1);
+        } else {
+            const int last = first + (rc.w - rc.y) * tx;   // first tile of the last row
+            for (int a = first; a <= last; a += tx) {
+                atomicAdd(&b.diff[a], 1);
+                if (a + w < b.n_tiles) atomicAdd(&b.diff[a + w], -1);
+            }
+        }
+    }
+    b.rec_cnt[r] = c;
+    b.rec_info[r] = info;
+}
+
+// The parts of a step that ps_fit_step runs with less between them than the entry points do.
+// project with `count` leaves the binning's counts as well (diff zeroed before).
+ps_status project(const ps_planes* planes, const ps_frame* frame, const ps_settings* s, float* rec, int* rect,
+                  float* key, const BinCount* count, int* d_status, cudaStream_t st);
+// Where a binning with these arguments keeps its counts.
+ps_status bin_count(const ps_frame* frame, long long capacity, void* ws, size_t ws_bytes, BinCount* out);
+// counted: the counts are there.
+ps_status bin_tiles(const ps_frame* frame, const ps_settings* s, const float* rec, const int* rect,
+                    const float* key, int* tile_ptr, int* tile_ent, float* tile_key, long long capacity,
+                    long long* d_required, void* ws, size_t ws_bytes, bool counted, int* d_status,
+                    cudaStream_t st);
+// ps_splat_fused without the chain: the record gradients, the work counter and the partial
+// loss sums lie in ws as FusedWs says.  cleared: ws is zeroed (its first `bytes`).
+struct FusedWs {
+    float* g_rec;
+    int* counter;
+    double* slots;
+    size_t bytes;
+};
+ps_status fused_ws(const ps_frame* f, const ps_settings* s, void* ws, size_t ws_bytes, FusedWs* out);
+ps_status splat_fused(const ps_planes* planes, const ps_frame* f, const ps_settings* s, const float* rec,
+                      const float* key, const int* tile_ptr, const int* tile_ent, long long capacity,
+                      const float* gt_depth, const float* gt_normal, float* depth, float* normal, float* dL_dD,
+                      float* dL_dN, float* g_radii, void* ws, size_t ws_bytes, bool cleared, int* d_status,
+                      cudaStream_t st);
+
 // (t, id) lexicographic order of candidates.
 __device__ __forceinline__ bool cand_less(float ta, int ia, float tb, int ib)
 {

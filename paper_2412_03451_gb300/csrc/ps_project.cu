@@ -114,8 +114,11 @@ struct ProjArgs {
     int single_radii;
     int gauss;              // PS_GAUSSIAN: radii scaled by delta instead of widened
     int tile_w, tile_h;
+    BinCount count;         // with COUNT
 };
 
+// COUNT: the binning's counts of the record as well (ps_fit_step).
+template <bool COUNT>
 __global__ void __launch_bounds__(128) k_project(ProjArgs a)
 {
     const int v = blockIdx.y;
@@ -258,6 +261,7 @@ __global__ void __launch_bounds__(128) k_project(ProjArgs a)
         }
     }
     a.rect[r] = rc;
+    if constexpr (COUNT) count_record(a.count, (size_t)r, rc, __ldg(&vw->tile_off), __ldg(&vw->tiles_x), v);
     a.key[r] = kf;
     float4* o4 = reinterpret_cast<float4*>(a.rec + (size_t)r * kRecFloats);
     o4[0] = make_float4(out[0], out[1], out[2], out[3]);
@@ -268,9 +272,8 @@ __global__ void __launch_bounds__(128) k_project(ProjArgs a)
 
 }  // namespace
 
-extern "C" ps_status ps_project_cull(const ps_planes* planes, const ps_frame* frame,
-                                     const ps_settings* s, float* rec, int* rect, float* key,
-                                     int* d_status, ps_stream stream)
+ps_status ps::project(const ps_planes* planes, const ps_frame* frame, const ps_settings* s, float* rec,
+                      int* rect, float* key, const BinCount* count, int* d_status, cudaStream_t st)
 {
     if (!planes || !frame || !s || !rec || !rect || !key || !frame->views) return PS_ERR_ARG;
     if (!planes->center || !planes->quat || !planes->radii) return PS_ERR_ARG;
@@ -282,8 +285,7 @@ extern "C" ps_status ps_project_cull(const ps_planes* planes, const ps_frame* fr
     if ((reinterpret_cast<uintptr_t>(rec) & 15) || (reinterpret_cast<uintptr_t>(rect) & 15))
         return PS_ERR_ARG;
     if (frame->max_K == 0 || frame->n_records == 0) return PS_OK;
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    ProjArgs a;
+    ProjArgs a{};
     a.center = planes->center; a.quat = planes->quat; a.radii = planes->radii;
     a.views = frame->views;
     a.rec = rec; a.rect = reinterpret_cast<int4*>(rect); a.key = key; a.status = d_status;
@@ -293,9 +295,22 @@ extern "C" ps_status ps_project_cull(const ps_planes* planes, const ps_frame* fr
     a.gauss = (s->flags & PS_GAUSSIAN) ? 1 : 0;
     a.tile_w = s->tile_w; a.tile_h = s->tile_h;
     dim3 grid((frame->max_K + 127) / 128, frame->n_views);
-    k_project<<<grid, 128, 0, st>>>(a);
+    if (count) {
+        a.count = *count;
+        k_project<true><<<grid, 128, 0, st>>>(a);
+    } else {
+        k_project<false><<<grid, 128, 0, st>>>(a);
+    }
     PS_LAUNCH_CHECK();
     return PS_OK;
+}
+
+extern "C" ps_status ps_project_cull(const ps_planes* planes, const ps_frame* frame,
+                                     const ps_settings* s, float* rec, int* rect, float* key,
+                                     int* d_status, ps_stream stream)
+{
+    return ps::project(planes, frame, s, rec, rect, key, nullptr, d_status,
+                       reinterpret_cast<cudaStream_t>(stream));
 }
 
 // ---------------------------------------------------------------------------
@@ -317,17 +332,8 @@ __global__ void k_adam_state(float* __restrict__ p, const float* __restrict__ g,
     const float bc1 = __ldg(&st->bc1), bc2 = __ldg(&st->bc2);
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (; i < n; i += stride) {
-        const float gi = g[i];
-        const float mi = fmaf(b1, m[i], (1.f - b1) * gi);
-        const float vi = fmaf(b2, v[i], (1.f - b2) * gi * gi);
-        m[i] = mi;
-        v[i] = vi;
-        const float mh = mi / bc1, vh = vi / bc2;
-        float pi = p[i] - lr * mh / (sqrtf(vh) + eps);
-        if (i >= clamp_from && pi < clamp_min) pi = clamp_min;
-        p[i] = pi;
-    }
+    for (; i < n; i += stride)
+        adam_update(p, m, v, i, g[i], lr, b1, b2, eps, bc1, bc2, i >= clamp_from ? clamp_min : -INFINITY);
 }
 
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
@@ -336,85 +342,28 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
 {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (; i < n; i += stride) {
-        const float gi = g[i];
-        const float mi = fmaf(b1, m[i], (1.f - b1) * gi);
-        const float vi = fmaf(b2, v[i], (1.f - b2) * gi * gi);
-        m[i] = mi;
-        v[i] = vi;
-        const float mh = mi / bc1, vh = vi / bc2;
-        float pi = p[i] - lr * mh / (sqrtf(vh) + eps);
-        if (i >= clamp_from && pi < clamp_min) pi = clamp_min;
-        p[i] = pi;
-    }
+    for (; i < n; i += stride)
+        adam_update(p, m, v, i, g[i], lr, b1, b2, eps, bc1, bc2, i >= clamp_from ? clamp_min : -INFINITY);
 }
-// Elements from clamp_from on are raised to clamp_min (NaN: none).
-ps_status adam_step(float* param, const float* grad, float* m, float* v, long long n, float lr, float b1,
-                    float b2, float eps, int step, float clamp_min, long long clamp_from, cudaStream_t st)
-{
-    if (n < 0 || step < 1) return PS_ERR_ARG;
-    if (n == 0) return PS_OK;
-    if (!param || !grad || !m || !v) return PS_ERR_ARG;
-    const float bc1 = (float)(1.0 - pow((double)b1, (double)step));
-    const float bc2 = (float)(1.0 - pow((double)b2, (double)step));
-    if (isnan(clamp_min)) clamp_from = n;
-    long long blocks = (n + 255) / 256;
-    if (blocks > 152 * 16) blocks = 152 * 16;
-    k_adam<<<(unsigned)blocks, 256, 0, st>>>(param, grad, m, v, n, lr, b1, b2, eps, bc1, bc2, clamp_min,
-                                             clamp_from);
-    PS_LAUNCH_CHECK();
-    return PS_OK;
-}
+
 }  // namespace
 
 extern "C" ps_status ps_adam_step(float* param, const float* grad, float* m, float* v,
                                   long long n, float lr, float b1, float b2, float eps, int step,
                                   float clamp_min, ps_stream stream)
 {
-    return adam_step(param, grad, m, v, n, lr, b1, b2, eps, step, clamp_min, 0,
-                     reinterpret_cast<cudaStream_t>(stream));
-}
-
-// One call per step: an eager step of a small scene is bound by the host.  64 planes in 8
-// views of 128x96: 162 us per step from nine calls and their tensor views, 62 us from one.
-extern "C" ps_status ps_fit_step(int n_planes, const ps_frame* frame, const ps_settings* s,
-                                 const ps_fit_buffers* b, int fused, float lr, float b1, float b2,
-                                 float eps, float r_min, int step, ps_stream stream)
-{
-    if (n_planes < 0 || !frame || !s || !b || !b->params || !b->grad || step < 1) return PS_ERR_ARG;
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const size_t P = (size_t)n_planes;
-    ps_planes pl{};
-    pl.n_planes = n_planes;
-    pl.center = b->params; pl.quat = b->params + 3 * P; pl.radii = b->params + 7 * P;
-    float *gc = b->grad, *gq = b->grad + 3 * P, *gr = b->grad + 7 * P;
-    ps_status e = ps_project_cull(&pl, frame, s, b->rec, b->rect, b->key, b->d_status, stream);
-    if (e != PS_OK) return e;
-    e = ps_bin_tiles(frame, s, b->rec, b->rect, b->key, b->tile_ptr, b->tile_ent, b->tile_key, b->capacity,
-                     b->d_required, b->bin_ws, b->bin_ws_bytes, b->d_status, stream);
-    if (e != PS_OK) return e;
-    PS_CUDA_CHECK(cudaMemsetAsync(b->grad, 0, sizeof(float) * 11 * P, st));
-    if (fused) {
-        e = ps_splat_fused(&pl, frame, s, b->rec, b->tile_key, b->tile_ptr, b->tile_ent, b->capacity,
-                           b->gt_depth, b->gt_normal, nullptr, nullptr, nullptr, nullptr, b->view_sums, gc,
-                           gq, gr, b->bwd_ws, b->bwd_ws_bytes, b->d_status, stream);
-    } else {
-        e = ps_splat_fwd(frame, s, b->rec, b->tile_key, b->tile_ptr, b->tile_ent, b->capacity, b->depth,
-                         b->normal, nullptr, b->fwd_ws, b->fwd_ws_bytes, b->d_status, stream);
-        if (e == PS_OK)
-            e = ps_loss(frame, s, b->depth, b->normal, b->gt_depth, b->gt_normal, b->dL_dD, b->dL_dN,
-                        b->view_sums, stream);
-        if (e == PS_OK)
-            e = ps_splat_bwd(&pl, frame, s, b->rec, b->tile_key, b->tile_ptr, b->tile_ent, b->capacity,
-                             b->dL_dD, b->dL_dN, gc, gq, gr, b->bwd_ws, b->bwd_ws_bytes, b->d_status, stream);
-    }
-    if (e != PS_OK) return e;
-    if (b->split_acc) {
-        e = ps_radii_grad_accum(gr, b->split_scale, 1.f, n_planes, b->split_acc, stream);
-        if (e != PS_OK) return e;
-    }
-    return adam_step(b->params, b->grad, b->m, b->v, 11LL * n_planes, lr, b1, b2, eps, step, r_min,
-                     7LL * n_planes, st);
+    if (n < 0 || step < 1) return PS_ERR_ARG;
+    if (n == 0) return PS_OK;
+    if (!param || !grad || !m || !v) return PS_ERR_ARG;
+    const float bc1 = (float)(1.0 - pow((double)b1, (double)step));
+    const float bc2 = (float)(1.0 - pow((double)b2, (double)step));
+    const long long clamp_from = isnan(clamp_min) ? n : 0;
+    long long blocks = (n + 255) / 256;
+    if (blocks > 152 * 16) blocks = 152 * 16;
+    k_adam<<<(unsigned)blocks, 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+        param, grad, m, v, n, lr, b1, b2, eps, bc1, bc2, clamp_min, clamp_from);
+    PS_LAUNCH_CHECK();
+    return PS_OK;
 }
 
 // ---------------------------------------------------------------------------

@@ -84,16 +84,6 @@ constexpr int kFwd = 0, kBwd = 1, kFused = 2;
 // Weight forms: Eq. 7-9, Eq. 5, and the hard edge (forward only).
 constexpr int kRect = 0, kGauss = 1, kHard = 2;
 
-// Fused mode: per-view loss sums are added into kSlots partial sums per view
-// (spread over L2 slices, so that strips of one view do not serialise on one
-// address), which the chain kernel adds up into view_sums.
-constexpr int kSlots = 32;
-
-// Floats per record of the gradient accumulators: the gradients of s (0), of a turn about
-// v^y (1) and about -v^x (2) that moves n_c, of a turn about n_c (3), of the radii (4-7),
-// and for the Eq. 5 weight those of a_x and a_y (8, 9; the rectangle's follow from the radii).
-__host__ __device__ constexpr int grad_stride(int gauss) { return gauss ? 12 : 8; }
-
 struct SplatArgs {
     const ps_view* views;
     int n_views;
@@ -926,11 +916,7 @@ __global__ void __launch_bounds__(128) k_chain(ChainArgs a)
 {
     const int v = blockIdx.y;
     if (a.vs_slots && blockIdx.x == 0 && threadIdx.x < 4) {
-        // the fused kernel's loss sums of view v, added up in a fixed order
-        const double* sp = a.vs_slots + (size_t)v * kSlots * 4 + threadIdx.x;
-        double t = 0.0;
-        for (int i = 0; i < kSlots; ++i) t += sp[4 * i];
-        a.view_sums[4 * v + threadIdx.x] = t;
+        a.view_sums[4 * v + threadIdx.x] = slot_sum(a.vs_slots, v, threadIdx.x);
     }
     if (!a.g_rec) return;
     const ps_view* vw = a.views + v;
@@ -947,40 +933,17 @@ __global__ void __launch_bounds__(128) k_chain(ChainArgs a)
         g3.z == 0.f && g3.w == 0.f && gax == 0.f && gay == 0.f)
         return;
     const int p = __ldg(&vw->plane_off) + k;
-    const float q0 = __ldg(&a.quat[4 * p + 0]), q1 = __ldg(&a.quat[4 * p + 1]);
-    const float q2 = __ldg(&a.quat[4 * p + 2]), q3 = __ldg(&a.quat[4 * p + 3]);
-    const float qs = sqrtf(q0 * q0 + q1 * q1 + q2 * q2 + q3 * q3);
-    if (!(qs > 0.f) || !isfinite(qs)) return;
-    const float w = q0 / qs, x = q1 / qs, y = q2 / qs, z = q3 / qs;
-    // world axes: columns of the Hamilton matrix (Eq. 2-3)
-    const float vx[3] = {1.f - 2.f * (y * y + z * z), 2.f * (x * y + w * z), 2.f * (x * z - w * y)};
-    const float vy[3] = {2.f * (x * y - w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z + w * x)};
-    const float nn[3] = {2.f * (x * z + w * y), 2.f * (y * z - w * x), 1.f - 2.f * (x * x + y * y)};
-    // The centre moves s = n_c . p_c, a_x and a_y; the camera rotation takes n_c, v^x_c, v^y_c
-    // back to the world axes, so the world gradient is their combination.
-    float gp[3];
+    float g[11];
+    if (!chain_plane(g0, g3, gax, gay, __ldg(&a.quat[4 * p + 0]), __ldg(&a.quat[4 * p + 1]),
+                     __ldg(&a.quat[4 * p + 2]), __ldg(&a.quat[4 * p + 3]), a.single_radii, g))
+        return;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) gp[i] = g0.x * nn[i] + gax * vx[i] + gay * vy[i];
-    // A turn by theta in the plane's own frame moves v^x by theta_z v^y - theta_y n, v^y by
-    // theta_x n - theta_z v^x and n by theta_y v^x - theta_x v^y.  At a fixed centre the
-    // gradient of n lies along v^x (g0.y) and v^y (g0.z), those of v^x and v^y in the plane
-    // with the moment g0.w about n; parts along an axis itself do not turn it.  With
-    // dq = q (0, theta) / 2 the quaternion gradient is 2 q (0, torque) / |q|.
-    const float tx = -g0.z, ty = g0.y, tz = g0.w;
-    const float s2 = 2.f / qs;
-    atomicAdd(&a.g_center[3 * p + 0], gp[0]);
-    atomicAdd(&a.g_center[3 * p + 1], gp[1]);
-    atomicAdd(&a.g_center[3 * p + 2], gp[2]);
-    atomicAdd(&a.g_quat[4 * p + 0], s2 * -(x * tx + y * ty + z * tz));
-    atomicAdd(&a.g_quat[4 * p + 1], s2 * (w * tx + y * tz - z * ty));
-    atomicAdd(&a.g_quat[4 * p + 2], s2 * (w * ty + z * tx - x * tz));
-    atomicAdd(&a.g_quat[4 * p + 3], s2 * (w * tz + x * ty - y * tx));
-    float gr0 = g3.x, gr1 = g3.y, gr2 = g3.z, gr3 = g3.w;
-    if (a.single_radii) { gr0 += gr1; gr1 = 0.f; gr2 += gr3; gr3 = 0.f; }
-    atomicAdd(&a.g_radii[4 * p + 0], gr0);
-    atomicAdd(&a.g_radii[4 * p + 1], gr1);
-    atomicAdd(&a.g_radii[4 * p + 2], gr2);
-    atomicAdd(&a.g_radii[4 * p + 3], gr3);
+    for (int i = 0; i < 3; ++i) atomicAdd(&a.g_center[3 * p + i], g[i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        atomicAdd(&a.g_quat[4 * p + i], g[3 + i]);
+        atomicAdd(&a.g_radii[4 * p + i], g[7 + i]);
+    }
 }
 
 // Render loss, Eq. 14.
@@ -1226,7 +1189,7 @@ inline size_t grad_bytes(const ps_frame* f, const ps_settings* s)
 inline size_t bwd_ws(const ps_frame* f) { return grec_max(f) + kCounterBytes; }
 
 // ps_splat_fused: as ps_splat_bwd, then the per-view partial loss sums
-inline size_t fused_ws(const ps_frame* f)
+inline size_t fused_bytes(const ps_frame* f)
 {
     return bwd_ws(f) + sizeof(double) * 4 * kSlots * (size_t)f->n_views;
 }
@@ -1284,7 +1247,7 @@ extern "C" ps_status ps_splat_ids(const ps_frame* f, const ps_settings* s, const
 extern "C" size_t ps_bwd_workspace_bytes(const ps_frame* f)
 {
     if (!f || f->n_records < 0 || f->n_views < 0) return 0;
-    return fused_ws(f);
+    return fused_bytes(f);
 }
 
 extern "C" ps_status ps_splat_bwd(const ps_planes* planes, const ps_frame* f, const ps_settings* s,
@@ -1324,6 +1287,46 @@ extern "C" ps_status ps_splat_bwd(const ps_planes* planes, const ps_frame* f, co
     return PS_OK;
 }
 
+ps_status ps::fused_ws(const ps_frame* f, const ps_settings* s, void* ws, size_t ws_bytes, FusedWs* out)
+{
+    if (!f || !s || !ws || ws_bytes < fused_bytes(f) || (reinterpret_cast<uintptr_t>(ws) & 15)) return PS_ERR_ARG;
+    char* p = static_cast<char*>(ws);
+    const size_t g = grad_bytes(f, s);
+    *out = FusedWs{reinterpret_cast<float*>(p), reinterpret_cast<int*>(p + g),
+                   reinterpret_cast<double*>(p + g + kCounterBytes), g + fused_bytes(f) - grec_max(f)};
+    return PS_OK;
+}
+
+ps_status ps::splat_fused(const ps_planes* planes, const ps_frame* f, const ps_settings* s, const float* rec,
+                          const float* key, const int* tile_ptr, const int* tile_ent, long long capacity,
+                          const float* gt_depth, const float* gt_normal, float* depth, float* normal,
+                          float* dL_dD, float* dL_dN, float* g_radii, void* ws, size_t ws_bytes, bool cleared,
+                          int* d_status, cudaStream_t st)
+{
+    ps_status e = check_common(f, s, rec, key, tile_ptr, tile_ent, capacity);
+    if (e != PS_OK) return e;
+    if (!planes || !planes->center || !planes->quat || !planes->radii) return PS_ERR_ARG;
+    if (!gt_depth || !gt_normal || !g_radii) return PS_ERR_ARG;
+    if (s->flags & PS_HARD) return PS_ERR_ARG;
+    FusedWs w;
+    e = fused_ws(f, s, ws, ws_bytes, &w);
+    if (e != PS_OK) return e;
+    // record gradients, work counter and partial loss sums: one memset
+    if (!cleared) PS_CUDA_CHECK(cudaMemsetAsync(ws, 0, w.bytes, st));
+    SplatArgs a{};
+    a.views = f->views; a.n_views = f->n_views;
+    a.rec = reinterpret_cast<const float4*>(rec); a.key = key;
+    a.tile_ptr = tile_ptr; a.tile_ent = tile_ent; a.capacity = capacity;
+    a.c = make_const(s); a.M = s->M; a.d_state = s->d_state;
+    a.depth = depth; a.normal = normal; a.alpha = nullptr;
+    a.g_rec = w.g_rec; a.g_radii = g_radii; a.counter = w.counter;
+    a.single_radii = (s->flags & PS_SINGLE_RADII) ? 1 : 0; a.status = d_status;
+    a.gt_depth = gt_depth; a.gt_normal = gt_normal;
+    a.out_dLdD = dL_dD; a.out_dLdN = dL_dN; a.vs_slots = w.slots;
+    a.a_cos = s->a_cos; a.a_l1n = s->a_l1n; a.a_depth = s->a_depth;
+    return dispatch<kFused>(a, s, f->n_tiles, st, true) == cudaSuccess ? PS_OK : PS_ERR_CUDA;
+}
+
 extern "C" ps_status ps_splat_fused(const ps_planes* planes, const ps_frame* f,
                                     const ps_settings* s, const float* rec, const float* key,
                                     const int* tile_ptr, const int* tile_ent, long long capacity,
@@ -1332,37 +1335,19 @@ extern "C" ps_status ps_splat_fused(const ps_planes* planes, const ps_frame* f,
                                     float* g_center, float* g_quat, float* g_radii, void* ws,
                                     size_t ws_bytes, int* d_status, ps_stream stream)
 {
-    ps_status e = check_common(f, s, rec, key, tile_ptr, tile_ent, capacity);
-    if (e != PS_OK) return e;
-    if (!planes || !planes->center || !planes->quat || !planes->radii) return PS_ERR_ARG;
-    if (!gt_depth || !gt_normal || !view_sums || !g_center || !g_quat || !g_radii || !ws)
-        return PS_ERR_ARG;
-    if (s->flags & PS_HARD) return PS_ERR_ARG;
-    if (ws_bytes < fused_ws(f) || (reinterpret_cast<uintptr_t>(ws) & 15)) return PS_ERR_ARG;
+    if (!view_sums || !g_center || !g_quat) return PS_ERR_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const size_t grec_bytes = grad_bytes(f, s);
-    // record gradients, work counter and partial loss sums: one memset
-    PS_CUDA_CHECK(cudaMemsetAsync(ws, 0, grec_bytes + fused_ws(f) - grec_max(f), st));
-    double* slots = reinterpret_cast<double*>(static_cast<char*>(ws) + grec_bytes + kCounterBytes);
-    SplatArgs a{};
-    a.views = f->views; a.n_views = f->n_views;
-    a.rec = reinterpret_cast<const float4*>(rec); a.key = key;
-    a.tile_ptr = tile_ptr; a.tile_ent = tile_ent; a.capacity = capacity;
-    a.c = make_const(s); a.M = s->M; a.d_state = s->d_state;
-    a.depth = depth; a.normal = normal; a.alpha = nullptr;
-    a.g_rec = reinterpret_cast<float*>(ws); a.g_radii = g_radii;
-    a.single_radii = (s->flags & PS_SINGLE_RADII) ? 1 : 0; a.status = d_status;
-    a.counter = reinterpret_cast<int*>(static_cast<char*>(ws) + grec_bytes);
-    a.gt_depth = gt_depth; a.gt_normal = gt_normal;
-    a.out_dLdD = dL_dD; a.out_dLdN = dL_dN; a.vs_slots = slots;
-    a.a_cos = s->a_cos; a.a_l1n = s->a_l1n; a.a_depth = s->a_depth;
-    if (dispatch<kFused>(a, s, f->n_tiles, st, true) != cudaSuccess) return PS_ERR_CUDA;
+    ps_status e = ps::splat_fused(planes, f, s, rec, key, tile_ptr, tile_ent, capacity, gt_depth, gt_normal,
+                                  depth, normal, dL_dD, dL_dN, g_radii, ws, ws_bytes, false, d_status, st);
+    if (e != PS_OK) return e;
+    FusedWs w;
+    ps::fused_ws(f, s, ws, ws_bytes, &w);
     ChainArgs c;
     c.views = f->views; c.center = planes->center; c.quat = planes->quat; c.radii = planes->radii;
-    c.g_rec = f->n_records > 0 ? a.g_rec : nullptr;
+    c.g_rec = f->n_records > 0 ? w.g_rec : nullptr;
     c.g_center = g_center; c.g_quat = g_quat; c.g_radii = g_radii;
-    c.single_radii = a.single_radii; c.gauss = a.c.gauss;
-    c.vs_slots = slots; c.view_sums = view_sums;
+    c.single_radii = (s->flags & PS_SINGLE_RADII) ? 1 : 0; c.gauss = (s->flags & PS_GAUSSIAN) ? 1 : 0;
+    c.vs_slots = w.slots; c.view_sums = view_sums;
     dim3 grid(f->max_K > 0 ? (f->max_K + 127) / 128 : 1, f->n_views);
     k_chain<<<grid, 128, 0, st>>>(c);
     PS_LAUNCH_CHECK();

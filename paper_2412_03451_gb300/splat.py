@@ -413,6 +413,10 @@ class Fitter:
     def _graph_body(self, gt_depth, gt_normal, view_sums, batch=0):
         r = self.r
         P = r.P
+        if self._one_call():
+            self._library_step(r.make_settings(1.0, d_state=self.d_state), gt_depth, gt_normal, view_sums, batch,
+                               True, (self.d_state, self.d_sched, self.n_sched, self.d_iter))
+            return
         B.ps_step_advance(self.d_state, self.d_sched, self.n_sched, self.d_iter)
         r.project_bin(self.flat, 1.0, d_state=self.d_state)
         self.grad.zero_()
@@ -428,27 +432,29 @@ class Fitter:
         self.ite += 1
         return self.graph_sums[batch_index]
 
-    def _native_step(self, gt_depth, gt_normal, lam, batch) -> bool:
-        """The whole step as one library call (False: not for these buffers)."""
-        r = self.r
-        state = (self.flat, self.grad, self.m, self.v)
-        if not all(t.is_contiguous() and t.dtype is torch.float32 and t.numel() == 11 * r.P for t in state):
-            return False
-        maps = (None,) * 4 if self.fused else (x.data_ptr() for x in (r.depth, r.normal, r.dLdD, r.dLdN))
-        acc = self.split_acc
+    def _one_call(self) -> bool:
+        """Whether the library's whole step takes these buffers."""
+        return all(t.is_contiguous() and t.dtype is torch.float32 and t.numel() == 11 * self.r.P
+                   for t in (self.flat, self.grad, self.m, self.v))
+
+    def _library_step(self, settings, gt_depth, gt_normal, view_sums, batch, fused, schedule=()):
+        """The whole step as one library call; schedule: d_state, d_sched, n_sched, d_iter."""
+        r, acc = self.r, self.split_acc
+        maps = (None,) * 4 if fused else (x.data_ptr() for x in (r.depth, r.normal, r.dLdD, r.dLdN))
+        d_state, d_sched, n_sched, d_iter = schedule or (None, None, 0, None)
         buf = B.PsFitBuffers(
-            *(t.data_ptr() for t in state), r.rec.data_ptr(), r.rect.data_ptr(), r.key.data_ptr(),
+            self.flat.data_ptr(), self.grad.data_ptr(), self.m.data_ptr(), self.v.data_ptr(),
+            r.rec.data_ptr(), r.rect.data_ptr(), r.key.data_ptr(),
             r.tile_ptr.data_ptr(), r.tile_ent.data_ptr(), r.tile_key.data_ptr(), r.capacity,
             r.required.data_ptr(), r.bin_ws.data_ptr(), 4 * r.bin_ws.numel(), r.fwd_ws.data_ptr(),
             4 * r.fwd_ws.numel(), r.bwd_ws.data_ptr(), 4 * r.bwd_ws.numel(), r.status.data_ptr(),
-            gt_depth.data_ptr(), gt_normal.data_ptr(), *maps, r.view_sums.data_ptr(),
+            gt_depth.data_ptr(), gt_normal.data_ptr(), *maps, view_sums.data_ptr(),
             None if acc is None else acc.data_ptr(),
-            None if acc is None else B._ptr(self.split_scale[batch or 0]))
+            None if acc is None else B._ptr(self.split_scale[batch or 0]),
+            B._ptr(d_state), B._ptr(d_sched), n_sched, 0, B._ptr(d_iter))
         r.generation += 1
-        B.ps_fit_step(r.P, r.frame, r.make_settings(lam), buf, self.fused, self.lr, self.b1, self.b2,
-                      self.eps, R_MIN, self.ite + 1)
-        self.ite += 1
-        return True
+        B.ps_fit_step(r.P, r.frame, settings, buf, fused, self.lr, self.b1, self.b2, self.eps, R_MIN,
+                      self.ite + 1)
 
     def step(self, gt_depth, gt_normal, lam=None, marks=None, batch=None):
         """One iteration.  If marks is a list, CUDA events are recorded on the
@@ -461,7 +467,9 @@ class Fitter:
 
         lam = B.lambda_schedule(self.ite + self.lam_offset) if lam is None else lam
         r = self.r
-        if marks is None and self._native_step(gt_depth, gt_normal, lam, batch):
+        if marks is None and self._one_call():
+            self._library_step(r.make_settings(lam), gt_depth, gt_normal, r.view_sums, batch, self.fused)
+            self.ite += 1
             return r.view_sums
         mark("start")
         r.project_bin(self.flat, lam)

@@ -78,3 +78,34 @@ def test_autograd_grows_its_lists(capacity):
     exp = torch.zeros_like(got)
     ref.backward(flat.detach(), exp, g, torch.zeros(n, 3, device="cuda"))
     assert float((got - exp).norm() / exp.norm()) < 1e-5 and float(exp.norm()) > 0
+
+
+def test_step_with_empty_scenes_and_scenes_without_views():
+    # the chain finds a plane's records by its scene's views: more views than lanes per plane, a
+    # scene with a view but no planes, planes that no view sees, one view, a trailing empty scene
+    import torch
+    from paper_2412_03451_gb300 import splat as SP
+    room = S.tiny_room(0)
+    p = S.perturb_planes(room.gt, 1)
+    views = [0, 1, 2, 3, 4, 5, 6, 7, 0, 1, 2]
+    K, ptr = 32, [0, 5, 5, 12, 32, 32]
+    H, W = room.cams.H, room.cams.W
+    n = len(views) * H * W
+    g = torch.Generator(device="cuda").manual_seed(5)
+    gd, gn = torch.rand(n, device="cuda", generator=g) + 1, torch.randn(n, 3, device="cuda", generator=g)
+    out = []
+    for marks in (None, []):
+        r = SP.Renderer([H] * len(views), [W] * len(views), [0] * 9 + [1] + [3], ptr)
+        r.set_cameras(room.cams.w2c[views], room.cams.intr[views])
+        flat = SP.planes_to_flat(p.center[:K], p.quat[:K], p.radii[:K], "cuda")
+        r.ensure_capacity(flat, 20.0)
+        fit = SP.Fitter(r, flat)
+        fit.grad.fill_(9.0)
+        sums = fit.step(gd, gn, lam=20.0, marks=marks)
+        out.append((fit.grad, fit.m, sums))
+    (g0, m0, s0), (g1, m1, s1) = out
+    gc = SP.flat_views(g0, K)
+    assert all(float(x[5:12].abs().max()) == 0.0 for x in gc) and float(gc[0][:5].abs().sum()) > 0
+    assert float(gc[0][12:].abs().sum()) > 0
+    assert float((g0 - g1).norm() / g1.norm()) < 1e-5 and float((m0 - m1).norm() / m1.norm()) < 1e-5
+    assert torch.allclose(s0, s1, rtol=1e-6)

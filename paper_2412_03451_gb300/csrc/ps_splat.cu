@@ -94,8 +94,9 @@ struct SplatArgs {
     long long capacity;
     SplatConst c;
     int M;
-    int n_items;              // strips = n_tiles * (tile pixels / 32), or groups of them
-    int group;                // strips of a tile per item (hard edge)
+    int n_items;              // work items: strips = n_tiles * (tile pixels / 32), or groups of them
+    int group;                // strips of a tile per item (hard edge, grouped items)
+    int n_grouped;            // grouped items; the items after them are single strips
     int* counter;             // work counter (zeroed before the launch)
     const ps_step_state* d_state;   // if set, lambda and delta come from here
     // forward outputs
@@ -117,6 +118,14 @@ struct SplatArgs {
     float* out_dLdN;          // optional
     double* vs_slots;         // [V][kSlots][4] partial loss sums (zeroed before the launch)
     float a_cos, a_l1n, a_depth;
+};
+
+// What the strips of a tile share (grouped items).
+struct __align__(16) TileCtx {
+    float fx, fy, cx, cy;
+    int W, H, tx0, ty0;
+    int beg, end, v, pad;
+    long long pix_off, gt_off;
 };
 
 // A warp's staging area: one list chunk.
@@ -278,10 +287,11 @@ __device__ __forceinline__ void flush(Walk<KP>& s, Sink& k, const float4* __rest
 // is partly transparent and waits in the buffer until a bound passes it (2,000 planes at
 // lambda 20 in 8 views of 640x480: a step 2,427 -> 2,297 us); for the rectangle weight a step
 // changes by -1..+4% by tile shape and lambda and a hard render is 5% slower.
-template <int MODE, int KP, bool SB>
+// GR: a list of one chunk stays staged for the next strips of its tile.
+template <int MODE, int KP, bool SB, bool GR>
 __device__ __forceinline__ void walk_strip(const SplatArgs& a, WarpStage& ws, Walk<KP>& s,
                                            Sink& k, float dx, float dy, const WarpRegion& g,
-                                           int beg, int end)
+                                           int beg, int end, bool& staged)
 {
     const int lane = threadIdx.x & 31;
     const float kMargin = 1.f - 1.f / 4096.f;
@@ -292,14 +302,19 @@ __device__ __forceinline__ void walk_strip(const SplatArgs& a, WarpStage& ws, Wa
             const int i = base + lane;
             bool ok = false;
             float low = INFINITY;
-            if (i < end) {
+            if (GR && staged) {
+                float t_low;
+                ok = i < end && region_may_hit<false>(ws.rec[0][lane], ws.rec[1][lane], ws.rec[2][lane],
+                                                      ws.rec[3][lane], g, a.c, t_low);
+                low = ws.key[lane];
+            } else if (i < end) {
                 const int id = __ldg(&a.tile_ent[i]);
                 const float4* r = a.rec + (size_t)id * 4;
                 const float4 n = __ldg(r + 0), vx = __ldg(r + 1), vy = __ldg(r + 2), rr = __ldg(r + 3);
                 float t_low;
                 ok = region_may_hit<SB>(n, vx, vy, rr, g, a.c, t_low);
                 if constexpr (!SB) low = __ldg(&a.key[i]) * kMargin;
-                if (ok) {
+                if (GR || ok) {
                     if constexpr (SB) low = fmaxf(__ldg(&a.key[i]), t_low) * kMargin;
                     ws.id[lane] = id;
                     ws.rec[0][lane] = n; ws.rec[1][lane] = vx; ws.rec[2][lane] = vy; ws.rec[3][lane] = rr;
@@ -320,6 +335,7 @@ __device__ __forceinline__ void walk_strip(const SplatArgs& a, WarpStage& ws, Wa
                     ws.key[32] = (base + 32 < end) ? __ldg(&a.key[base + 32]) * kMargin : INFINITY;
             }
             unsigned m = __ballot_sync(kFull, ok);
+            if constexpr (GR) staged = end - beg <= 32;
             __syncwarp();
             while (m) {
                 // every pixel of the strip is finished: the rest of the chunk cannot matter
@@ -406,33 +422,47 @@ struct StripLoss {
     float sc, sl, sd, one;
 };
 
-template <int TW, int TH, int MODE, int KP, int G>
-__device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws, int2* stk_warp,
-                                               int item)
+// The view, pixel origin and list of a tile.
+template <int TW, int TH, int MODE>
+__device__ __forceinline__ TileCtx tile_setup(const SplatArgs& a, int tile)
 {
-    constexpr int NS = TW * TH / 32;       // strips per tile
-    constexpr int NG = G ? 10 : 8;         // gradient floats per pair
-    const int lane = threadIdx.x & 31;
-    const int tile = item / NS;
-    const int strip = item - tile * NS;
     // (the cooperative search takes 3% off a hard render of 64 views and adds 2% to the fused
     // kernel, whose registers it costs)
     const int v = MODE == kFwd ? warp_view_of_tile(a.views, a.n_views, tile)
                                : view_of_tile(a.views, a.n_views, tile);
     const ps_view* vw = a.views + v;
-    const int W = __ldg(&vw->W), H = __ldg(&vw->H);
     const int tx_n = __ldg(&vw->tiles_x);
     const int lt = tile - __ldg(&vw->tile_off);
-    const int tx0 = (lt % tx_n) * TW, ty0 = (lt / tx_n) * TH;
+    TileCtx t;
+    t.v = v;
+    t.W = __ldg(&vw->W); t.H = __ldg(&vw->H);
+    t.tx0 = (lt % tx_n) * TW; t.ty0 = (lt / tx_n) * TH;
+    t.fx = __ldg(&vw->fx); t.fy = __ldg(&vw->fy);
+    t.cx = __ldg(&vw->cx); t.cy = __ldg(&vw->cy);
+    t.pix_off = __ldg(&vw->pix_off);
+    t.gt_off = __ldg(&vw->gt_off);
+    t.beg = (int)min((long long)__ldg(&a.tile_ptr[tile]), a.capacity);
+    t.end = (int)min((long long)__ldg(&a.tile_ptr[tile + 1]), a.capacity);
+    t.pad = 0;
+    return t;
+}
+
+template <int TW, int TH, int MODE, int KP, int G, bool GR>
+__device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws, int2* stk_warp,
+                                               const TileCtx& t, int strip, bool& staged)
+{
+    constexpr int NG = G ? 10 : 8;         // gradient floats per pair
+    const int lane = threadIdx.x & 31;
+    const int v = t.v;
+    const ps_view* vw = a.views + v;
+    const int W = t.W, H = t.H;
     const int q = strip * 32 + lane;        // pixel index within the tile, row-major
-    const int px = tx0 + q % TW, py = ty0 + q / TW;
+    const int px = t.tx0 + q % TW, py = t.ty0 + q / TW;
     const bool inside = px < W && py < H;
-    const float fx = __ldg(&vw->fx), fy = __ldg(&vw->fy);
-    const float cx = __ldg(&vw->cx), cy = __ldg(&vw->cy);
-    const float dx = __fdiv_rn((float)px + 0.5f - cx, fx);
-    const float dy = __fdiv_rn((float)py + 0.5f - cy, fy);
-    const long long pix = __ldg(&vw->pix_off) + (long long)py * W + px;
-    const long long gpix = __ldg(&vw->gt_off) + (long long)py * W + px;   // supervision pixel
+    const float dx = __fdiv_rn((float)px + 0.5f - t.cx, t.fx);
+    const float dy = __fdiv_rn((float)py + 0.5f - t.cy, t.fy);
+    const long long pix = t.pix_off + (long long)py * W + px;
+    const long long gpix = t.gt_off + (long long)py * W + px;   // supervision pixel
     WarpRegion g;
     {
         constexpr int WX = TW < 32 ? TW : 32;
@@ -442,8 +472,6 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
         const float mx = fmaxf(fabsf(g.dxa), fabsf(g.dxb)), my = fmaxf(fabsf(g.dya), fabsf(g.dyb));
         g.den_min = 0.01f * sqrtf(fmaf(mx, mx, fmaf(my, my, 1.f)));
     }
-    const int beg = (int)min((long long)__ldg(&a.tile_ptr[tile]), a.capacity);
-    const int end = (int)min((long long)__ldg(&a.tile_ptr[tile + 1]), a.capacity);
 
     Walk<KP> s;
     s.T = 1.f; s.cnt = 0; s.nb = 0;
@@ -472,7 +500,7 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
             if (gD == 0.f && gN0 == 0.f && gN1 == 0.f && gN2 == 0.f) s.done = true;
         }
     }
-    walk_strip<MODE, KP, G == kGauss>(a, ws, s, k, dx, dy, g, beg, end);
+    walk_strip<MODE, KP, G == kGauss, GR>(a, ws, s, k, dx, dy, g, t.beg, t.end, staged);
 
     if constexpr (MODE != kBwd) {
         if (inside) {
@@ -750,9 +778,20 @@ __device__ __forceinline__ void load_state(SplatArgs& a)
     }
 }
 
+// Grouped items (the rectangle weight): strips of one tile go to one warp, which sets the tile
+// up once and keeps a list of one chunk staged: two strips, or the whole tile in the forward
+// kernel.  The last strips go one by one, so that the warps finish together: kSingles per
+// resident warp, more than a pair of the heaviest strips costs (with 6 a step at the first lambda
+// was 17% slower, with 14 the gain there was lost), or two of the forward's longer groups; with
+// fewer than kGroupFrom strips per warp the kernel without groups runs (3% faster there).  16 rooms (235 strips per warp): a step
+// 1,550 -> 1,436 us; 10,000 planes, 64 views 5,058 -> 4,887; 16 views 304 -> 293; 8 views (25 per
+// warp) -0.5..-1.5%.  The Eq. 5 weight's lists are too long to share (+6%).
+constexpr int kSingles = 10, kGroupFrom = 20;
+
 // G: the weight form of the instantiation, fixed at compile time so that the other forms'
 // branches fold away.
-template <int TW, int TH, int MODE, int NW, int G>
+// GR: with grouped items.
+template <int TW, int TH, int MODE, int NW, int G, bool GR>
 __global__ void __launch_bounds__(NW * 32, min_blocks(MODE, G, NW)) k_splat(SplatArgs a_in)
 {
     constexpr int KP = G == kGauss ? kPendGauss : kPendRect;
@@ -761,6 +800,7 @@ __global__ void __launch_bounds__(NW * 32, min_blocks(MODE, G, NW)) k_splat(Spla
     a.c.hard = G == kHard;
     load_state(a);
     __shared__ WarpStage stage[NW];
+    __shared__ TileCtx ctx[GR ? NW : 1];
     extern __shared__ int2 dyn_stk[];       // backward: [NW][M][32]
     const int w = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -798,15 +838,30 @@ __global__ void __launch_bounds__(NW * 32, min_blocks(MODE, G, NW)) k_splat(Spla
             run_hard<TW, TH>(a, stage[w], tile, s0, s0 + a.group);
             continue;
         }
-        const StripLoss sl = run_strip<TW, TH, MODE, KP, G>(a, stage[w], stk_warp, item);
-        if constexpr (MODE == kFused) {
-            if (sl.v != vcur) {
-                if (vcur >= 0) flush_loss();
-                vcur = sl.v;
+        constexpr int NS = TW * TH / 32;       // strips per tile
+        auto strip = [&](const TileCtx& t, int i, bool& staged) {
+            const StripLoss sl = run_strip<TW, TH, MODE, KP, G, GR>(a, stage[w], stk_warp, t, i, staged);
+            if constexpr (MODE == kFused) {
+                if (sl.v != vcur) {
+                    if (vcur >= 0) flush_loss();
+                    vcur = sl.v;
+                }
+                l0 += sl.sc; l1 += sl.sl; l2 += sl.sd; l3 += sl.one;
             }
-            l0 += sl.sc; l1 += sl.sl; l2 += sl.sd; l3 += sl.one;
+            __syncwarp();
+        };
+        bool staged = false;
+        if constexpr (GR) {
+            const bool grouped = item < a.n_grouped;
+            const int n = grouped ? a.group : 1;
+            const int first = grouped ? item * a.group : item + a.n_grouped * (a.group - 1);
+            const TileCtx t = tile_setup<TW, TH, MODE>(a, first / NS);
+            if (lane == 0) ctx[w] = t;
+            __syncwarp();
+            for (int i = first % NS, e = i + n; i < e; ++i) strip(ctx[w], i, staged);
+        } else {
+            strip(tile_setup<TW, TH, MODE>(a, item / NS), item % NS, staged);
         }
-        __syncwarp();
     }
     if constexpr (MODE == kFused) {
         if (vcur >= 0) flush_loss();
@@ -1054,7 +1109,7 @@ struct LaunchCache {
     size_t dyn = 0;
 };
 
-template <int TW, int TH, int MODE, int NW, int G>
+template <int TW, int TH, int MODE, int NW, int G, bool GR = false>
 cudaError_t launch_splat(SplatArgs a, int n_tiles, int M, cudaStream_t st, bool counter_zeroed)
 {
     constexpr int NS = TW * TH / 32;
@@ -1068,12 +1123,12 @@ cudaError_t launch_splat(SplatArgs a, int n_tiles, int M, cudaStream_t st, bool 
     if (c.dev != dev || c.dyn != dyn) {
         if (dyn > 0) {
             // static + dynamic shared memory above 48 KB needs the opt-in
-            e = cudaFuncSetAttribute(k_splat<TW, TH, MODE, NW, G>,
+            e = cudaFuncSetAttribute(k_splat<TW, TH, MODE, NW, G, GR>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
             if (e != cudaSuccess) return e;
         }
         int nb = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_splat<TW, TH, MODE, NW, G>, NW * 32, dyn);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_splat<TW, TH, MODE, NW, G, GR>, NW * 32, dyn);
         if (e != cudaSuccess) return e;
         int sms = 0;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1082,14 +1137,24 @@ cudaError_t launch_splat(SplatArgs a, int n_tiles, int M, cudaStream_t st, bool 
         c.dyn = dyn;
         c.blocks_per_sm = (nb > 0 ? nb : 1) * sms;
     }
+    const long long warps = (long long)c.blocks_per_sm * NW;       // resident, of all SMs
     a.group = 1;
     if constexpr (G == kHard) {
         // A strip is so short that the one work counter binds (a render of 614,400 strips takes
         // 474 us one by one, 367 in pairs, 263 by tiles that share their setup): groups as large
         // as leave every warp four items.
-        const long long warps = (long long)c.blocks_per_sm * NW;
         while (a.group < NS && a.n_items / (2 * a.group) >= 4 * warps) a.group *= 2;
         a.n_items /= a.group;
+    }
+    if constexpr (G == kRect && !GR) {
+        if (a.n_items >= kGroupFrom * warps)
+            return launch_splat<TW, TH, MODE, NW, G, true>(a, n_tiles, M, st, counter_zeroed);
+    }
+    if constexpr (GR) {
+        a.group = MODE == kFwd ? NS : 2;
+        const long long single = (a.group > 2 ? 2 * a.group : kSingles) * warps;
+        a.n_grouped = a.n_items > single ? (int)((a.n_items - single) / NS * (NS / a.group)) : 0;
+        a.n_items -= a.n_grouped * (a.group - 1);
     }
     int blocks = c.blocks_per_sm;
     const int need = (a.n_items + NW - 1) / NW;
@@ -1099,7 +1164,7 @@ cudaError_t launch_splat(SplatArgs a, int n_tiles, int M, cudaStream_t st, bool 
         e = cudaMemsetAsync(a.counter, 0, sizeof(int), st);
         if (e != cudaSuccess) return e;
     }
-    k_splat<TW, TH, MODE, NW, G><<<blocks, NW * 32, dyn, st>>>(a);
+    k_splat<TW, TH, MODE, NW, G, GR><<<blocks, NW * 32, dyn, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -171,3 +171,48 @@ def test_hard_maps_by_groups_of_strips(tile, V, warps, K):
             assert ids[y * w + x] == order[0] and abs(D[y * w + x] - t[order[0]]) < 1e-4
         checked += 1
     assert checked > 100
+
+
+@pytest.mark.parametrize("tile,warps", [((8, 8), 0), ((16, 16), 2), ((32, 8), 8)])
+@pytest.mark.parametrize("K", [12, 150])
+def test_grouped_strips_equal_single_views(tile, warps, K):
+    # many strips per warp: the first go in groups of a tile's strips (lists of one chunk, K = 12,
+    # stay staged from strip to strip; K = 150: several chunks), the last one by one; a view alone
+    # has too few to group.  Forward, plane indices, fused and separate backward.
+    import torch
+    from paper_2412_03451_gb300 import splat as SP
+    p = S.random_planes_in_view(K, K, depth_range=(0.4, 3.0), half=(0.1, 0.6))
+    V, h, w = 16, 470, 629
+    cams = S.identity_cameras(V, h, w, 400.0, seed=4, jitter=0.1)
+    flat = SP.planes_to_flat(p.center, p.quat, p.radii, "cuda")
+    n = h * w
+    g = torch.Generator(device="cuda").manual_seed(1)
+    gd, gn = torch.rand(V * n, device="cuda", generator=g) + 1, torch.randn(V * n, 3, device="cuda", generator=g)
+
+    def run(views):
+        k = len(views)
+        r = SP.Renderer([h] * k, [w] * k, [0] * k, [0, p.K], tile=tile, warps=warps)
+        r.set_cameras(cams.w2c[views], cams.intr[views])
+        r.ensure_capacity(flat, 60.0)
+        at = slice(views[0] * n, (views[-1] + 1) * n)
+        D, N = (x.clone() for x in r.forward(flat, 60.0))
+        ids, _ = r.plane_ids(flat, 60.0, hard=False)
+        r.project_bin(flat, 60.0)
+        fused, sep = torch.zeros_like(flat), torch.zeros_like(flat)
+        sums = r.fused(flat, fused, gd[at], gn[at], write_maps=True).clone()
+        assert torch.equal(r.depth, D) and torch.equal(r.normal, N)
+        r.backward(flat, sep)                          # the fused walk's own dL/dD, dL/dN
+        assert int(r.status.item()) == 0
+        assert float((fused - sep).norm() / sep.norm()) < 1e-5
+        return [D.view(k, -1), N.view(k, -1), ids.view(k, -1), sums], fused.double()
+
+    got, grad = run(list(range(V)))
+    total = torch.zeros_like(grad)
+    for v in range(V):
+        one, g1 = run([v])
+        for a, b in zip(got[:3], one[:3]):
+            assert torch.equal(a[v], b[0]), v
+        assert torch.allclose(got[3][v], one[3][0], rtol=1e-6)
+        total += g1
+    # FP32 sums of the same pairs in another order
+    assert float((grad - total).norm() / total.norm()) < 1e-5

@@ -159,11 +159,12 @@ struct WarpRegion {
 // the rectangle are spanned by the four corner rays.  The corner values use
 // the per-pixel formulas of eval_pair; the margins cover FP32 rounding.  t_low is
 // the smallest depth at the corners, which bounds the depth at every pixel of the
-// rectangle from below up to rounding (0 where d . n_c is too small for that).
+// rectangle from below up to rounding (0 where d . n_c is too small for that).  A plane
+// whose depths all lie below t_floor may not hit.
 template <bool LOW>
 __device__ __forceinline__ bool region_may_hit(const float4& n, const float4& vx, const float4& vy,
                                                const float4& r, const WarpRegion& g,
-                                               const SplatConst& c, float& t_low)
+                                               const SplatConst& c, float& t_low, float t_floor = 0.f)
 {
     float tmin = INFINITY, tmax = -INFINITY, xmin = INFINITY, xmax = -INFINITY;
     float ymin = INFINITY, ymax = -INFINITY;
@@ -186,7 +187,10 @@ __device__ __forceinline__ bool region_may_hit(const float4& n, const float4& vx
     }
     if (!(dlo > 2e-6f) && !(dhi < -2e-6f)) return true;       // d . n_c may vanish: no bound
     if constexpr (LOW) {
-        if (dlo > g.den_min || dhi < -g.den_min) t_low = tmin;
+        if (dlo > g.den_min || dhi < -g.den_min) {
+            t_low = tmin;
+            if (tmax < t_floor) return false;
+        }
     }
     if (tmax < c.z_near * 0.99999f || tmin > c.z_far * 1.00001f) return false;
     // support: r + reject around the rectangle, or kappa r for the Eq. 5 weight

@@ -176,6 +176,7 @@ __device__ __forceinline__ T block_scan_excl(T x, T* s_warp)
 __global__ void __launch_bounds__(kScanThreads) k_scan_sums(ScanJob j0, ScanJob j1)
 {
     __shared__ longlong2 s_warp[kScanThreads / 32];
+    after_previous();
     const bool second = (int)blockIdx.x >= j0.blocks;
     const ScanJob& a = second ? j1 : j0;
     const int b = (int)blockIdx.x - (second ? j0.blocks : 0);
@@ -198,6 +199,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(ScanJob j0, ScanJob
     __shared__ longlong2 s_pair[kScanThreads / 32];
     __shared__ long long s_wide[kScanThreads / 32];
     __shared__ int s_int[kScanThreads / 32];
+    after_previous();
     const bool second = (int)blockIdx.x >= j0.blocks;
     const ScanJob& a = second ? j1 : j0;
     const int b = (int)blockIdx.x - (second ? j0.blocks : 0);
@@ -342,6 +344,7 @@ __global__ void __launch_bounds__(kPairBlock) k_pair_scatter(const int* __restri
                                                        const int* __restrict__ chunk_first,
                                                        long long n_chunk)
 {
+    after_previous();
     const int E = __ldg(&rec_off[R]);
     for (int base = blockIdx.x * kPairBlock; base < E; base += gridDim.x * kPairBlock) {
         const int2 rg = chunk_record_range(rec_off, R, E, base, chunk_first, n_chunk);
@@ -500,6 +503,7 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort(const int* __restrict_
     __shared__ int s_cnt;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) s_cnt = 0;
+    after_previous();
     __syncthreads();
     const int t0 = (blockIdx.x * kSortWarps + w) * kSortTiles;
     // lane l < kSortTiles + 1: the start of tile t0 + l's list (past the last tile: its end)
@@ -593,21 +597,15 @@ ps_status ps::bin_tiles(const ps_frame* frame, const ps_settings* s, const float
                      w.chunk_first, nch, w.part, tr};
     const ScanJob jt{w.tile_cnt, frame->n_tiles, tile_ptr, w.cursor, capacity, d_required,
                      d_status, 1, nullptr, 0, w.part + tr, tt};
-    k_scan_sums<<<tr + tt, kScanThreads, 0, st>>>(jr, jt);
-    PS_LAUNCH_CHECK();
-    k_scan_apply<<<tr + tt, kScanThreads, 0, st>>>(jr, jt);
-    PS_LAUNCH_CHECK();
+    PS_CUDA_CHECK(launch_after(k_scan_sums, tr + tt, kScanThreads, 0, st, jr, jt));
+    PS_CUDA_CHECK(launch_after(k_scan_apply, tr + tt, kScanThreads, 0, st, jr, jt));
     if (R > 0 && capacity > 0) {
-        k_pair_scatter<<<kFlatBlocks, kPairBlock, 0, st>>>(w.rec_cnt, R, w.rec_info, tile_ptr, w.cursor,
-                                                           w.ent_tmp,
-                                                           reinterpret_cast<const float4*>(rec), key,
-                                                           frame->views, s->tile_w, s->tile_h, s->z_near,
-                                                           w.chunk_first, nch);
-        PS_LAUNCH_CHECK();
+        PS_CUDA_CHECK(launch_after(k_pair_scatter, kFlatBlocks, kPairBlock, 0, st, w.rec_cnt, R, w.rec_info, tile_ptr,
+                                   w.cursor, w.ent_tmp, reinterpret_cast<const float4*>(rec), key, frame->views,
+                                   s->tile_w, s->tile_h, s->z_near, w.chunk_first, nch));
         constexpr int per = kSortWarps * kSortTiles;
-        k_sort<<<(frame->n_tiles + per - 1) / per, kSortWarps * 32, 0, st>>>(
-            tile_ptr, frame->n_tiles, w.ent_tmp, tile_ent, tile_key);
-        PS_LAUNCH_CHECK();
+        PS_CUDA_CHECK(launch_after(k_sort, (frame->n_tiles + per - 1) / per, kSortWarps * 32, 0, st, tile_ptr,
+                                   frame->n_tiles, w.ent_tmp, tile_ent, tile_key));
     }
     return PS_OK;
 }

@@ -121,6 +121,7 @@ struct ProjArgs {
 template <bool COUNT>
 __global__ void __launch_bounds__(128) k_project(ProjArgs a)
 {
+    after_previous();
     const int v = blockIdx.y;
     const ps_view* vw = a.views + v;
     const int K = __ldg(&vw->K);
@@ -297,7 +298,7 @@ ps_status ps::project(const ps_planes* planes, const ps_frame* frame, const ps_s
     dim3 grid((frame->max_K + 127) / 128, frame->n_views);
     if (count) {
         a.count = *count;
-        k_project<true><<<grid, 128, 0, st>>>(a);
+        PS_CUDA_CHECK(launch_after(k_project<true>, grid, 128, 0, st, a));
     } else {
         k_project<false><<<grid, 128, 0, st>>>(a);
     }

@@ -802,6 +802,7 @@ constexpr int kSingles = 10, kGroupFrom = 20;
 template <int TW, int TH, int MODE, int NW, int G, bool GR>
 __global__ void __launch_bounds__(NW * 32, min_blocks(MODE, G, NW)) k_splat(SplatArgs a_in)
 {
+    after_previous();
     constexpr int KP = G == kGauss ? kPendGauss : kPendRect;
     SplatArgs a = a_in;
     a.c.gauss = G == kGauss;
@@ -977,6 +978,7 @@ struct ChainArgs {
 
 __global__ void __launch_bounds__(128) k_chain(ChainArgs a)
 {
+    after_previous();
     const int v = blockIdx.y;
     if (a.vs_slots && blockIdx.x == 0 && threadIdx.x < 4) {
         a.view_sums[4 * v + threadIdx.x] = slot_sum(a.vs_slots, v, threadIdx.x);
@@ -1172,8 +1174,7 @@ cudaError_t launch_splat(SplatArgs a, int n_tiles, int M, cudaStream_t st, bool 
         e = cudaMemsetAsync(a.counter, 0, sizeof(int), st);
         if (e != cudaSuccess) return e;
     }
-    k_splat<TW, TH, MODE, NW, G, GR><<<blocks, NW * 32, dyn, st>>>(a);
-    return cudaGetLastError();
+    return launch_after(k_splat<TW, TH, MODE, NW, G, GR>, blocks, NW * 32, dyn, st, a);
 }
 
 ps_status check_common(const ps_frame* f, const ps_settings* s, const float* rec, const float* key,
@@ -1355,8 +1356,7 @@ extern "C" ps_status ps_splat_bwd(const ps_planes* planes, const ps_frame* f, co
     c.single_radii = a.single_radii; c.gauss = a.c.gauss;
     c.vs_slots = nullptr; c.view_sums = nullptr;
     dim3 grid((f->max_K + 127) / 128, f->n_views);
-    k_chain<<<grid, 128, 0, st>>>(c);
-    PS_LAUNCH_CHECK();
+    PS_CUDA_CHECK(launch_after(k_chain, grid, 128, 0, st, c));
     return PS_OK;
 }
 
@@ -1422,8 +1422,7 @@ extern "C" ps_status ps_splat_fused(const ps_planes* planes, const ps_frame* f,
     c.single_radii = (s->flags & PS_SINGLE_RADII) ? 1 : 0; c.gauss = (s->flags & PS_GAUSSIAN) ? 1 : 0;
     c.vs_slots = w.slots; c.view_sums = view_sums;
     dim3 grid(f->max_K > 0 ? (f->max_K + 127) / 128 : 1, f->n_views);
-    k_chain<<<grid, 128, 0, st>>>(c);
-    PS_LAUNCH_CHECK();
+    PS_CUDA_CHECK(launch_after(k_chain, grid, 128, 0, st, c));
     return PS_OK;
 }
 

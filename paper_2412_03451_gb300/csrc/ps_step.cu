@@ -30,6 +30,7 @@ struct BeginArgs {
 
 __global__ void __launch_bounds__(256) k_begin(BeginArgs a)
 {
+    after_previous();
     const long long t = (long long)blockIdx.x * 256 + threadIdx.x, stride = (long long)gridDim.x * 256;
 #pragma unroll
     for (int r = 0; r < 2; ++r)
@@ -64,6 +65,7 @@ struct ChainAdamArgs {
 __global__ void __launch_bounds__(kChainThreads) k_chain_adam(ChainAdamArgs a)
 {
     __shared__ float s_g[kChainPlanes][12];
+    after_previous();
     for (int v = blockIdx.x; v < a.n_views; v += gridDim.x)
         if (threadIdx.x < 4) a.view_sums[4 * v + threadIdx.x] = slot_sum(a.vs_slots, v, threadIdx.x);
     const int p0 = blockIdx.x * kChainPlanes, at = threadIdx.x / kChainLanes, p = p0 + at;
@@ -179,8 +181,7 @@ extern "C" ps_status ps_fit_step(int n_planes, const ps_frame* frame, const ps_s
         c.d_state = s->d_state;
         c.vs_slots = w.slots; c.view_sums = b->view_sums;
         const int grid = n_planes > 0 ? (n_planes + kChainPlanes - 1) / kChainPlanes : 1;
-        k_chain_adam<<<grid, kChainThreads, 0, st>>>(c);
-        PS_LAUNCH_CHECK();
+        PS_CUDA_CHECK(launch_after(k_chain_adam, grid, kChainThreads, 0, st, c));
         return b->split_acc ? ps_radii_grad_accum(gr, b->split_scale, 1.f, n_planes, b->split_acc, stream) : PS_OK;
     }
     if (b->d_sched) {

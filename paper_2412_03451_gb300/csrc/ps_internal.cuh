@@ -287,17 +287,24 @@ __device__ __forceinline__ bool chain_plane(const float4& g0, const float4& g3, 
 }
 
 // Adam with bias correction; values below `lowest` (NaN: none) are raised to it.
+__device__ __forceinline__ void adam_value(float& p, float& m, float& v, float g, float lr, float b1, float b2,
+                                           float eps, float bc1, float bc2, float lowest)
+{
+    m = fmaf(b1, m, (1.f - b1) * g);
+    v = fmaf(b2, v, (1.f - b2) * g * g);
+    const float mh = m / bc1, vh = v / bc2;
+    p = p - lr * mh / (sqrtf(vh) + eps);
+    if (p < lowest) p = lowest;
+}
+
 __device__ __forceinline__ void adam_update(float* __restrict__ p, float* __restrict__ m,
-                                            float* __restrict__ v, long long i, float gi, float lr, float b1,
+                                            float* __restrict__ v, long long i, float g, float lr, float b1,
                                             float b2, float eps, float bc1, float bc2, float lowest)
 {
-    const float mi = fmaf(b1, m[i], (1.f - b1) * gi);
-    const float vi = fmaf(b2, v[i], (1.f - b2) * gi * gi);
+    float pi = p[i], mi = m[i], vi = v[i];
+    adam_value(pi, mi, vi, g, lr, b1, b2, eps, bc1, bc2, lowest);
     m[i] = mi;
     v[i] = vi;
-    const float mh = mi / bc1, vh = vi / bc2;
-    float pi = p[i] - lr * mh / (sqrtf(vh) + eps);
-    if (pi < lowest) pi = lowest;
     p[i] = pi;
 }
 

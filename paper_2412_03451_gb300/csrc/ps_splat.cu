@@ -39,10 +39,12 @@
 // margin is r - |P|).  The camera rotation drops out of the chain.  The kernel is
 // bound by instruction issue, so what counts is the length of the aggregation: with
 // the 16 floats of n_c, s, v^x_c, a_x, v^y_c, a_y and the radii, summed in two halves
-// of 8, a step of the 3,000-plane room at 8 x 640x480 took 461 us at the first lambda
-// (now 408), 205 us at lambda 20 with 8 degree tilts (195) and 197 us at lambda 300
-// (193); 2,000 planes with the Eq. 5 weight, whose a_x and a_y need two floats more,
-// 2,562 us (2,420).
+// of 8, a step of the 3,000-plane room at 8 x 640x480 took 461 us at the first lambda (with 8
+// floats 408), 205 us at lambda 20 with 8 degree tilts (195) and 197 us at lambda 300 (193);
+// 2,000 planes with the Eq. 5 weight, whose a_x and a_y need two floats more, 2,562 us
+// (2,420).  With what followed (subnormals taken as 0, strips in groups, the replay's votes and
+// warp maximum instead of shuffles: -2.5% by themselves) these steps take 361, 158, 156 and 2,087
+// us.
 #include <mutex>
 
 #include <cuda.h>
@@ -559,9 +561,7 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
     if constexpr (MODE != kFwd) {
         // back to front over the stack
         const int cnt = supervised ? s.cnt : 0;
-        int wmax = cnt;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) wmax = max(wmax, __shfl_xor_sync(kFull, wmax, o));
+        const int wmax = __reduce_max_sync(kFull, cnt);
         float A = 0.f, B0 = 0.f, B1 = 0.f, B2 = 0.f;
         const float lam5 = a.c.lam5;
         // software pipeline: the record of stack entry j - 1 is loaded while j is processed
@@ -649,16 +649,13 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
             // warp aggregation: for each distinct record among the active lanes, its gradient
             // floats are summed over the lanes by a transpose-reduction and added with one
             // 8-lane atomic instruction (a 32-byte sector)
-            const unsigned actm = __ballot_sync(kFull, act);
-            if (actm == 0) continue;
             const unsigned peers = __match_any_sync(kFull, id);
-            unsigned rem = actm;
+            unsigned rem = __ballot_sync(kFull, act);            // (not empty: j < wmax)
             while (rem) {
                 const int leader = __ffs(rem) - 1;
-                const unsigned gmask = __shfl_sync(kFull, peers, leader);
                 const int gid = __shfl_sync(kFull, id, leader);
-                rem &= ~gmask;
-                const bool member = (gmask >> lane) & 1u;
+                const bool member = (peers >> leader) & 1u;
+                rem &= ~__ballot_sync(kFull, member);
                 float* dst = a.g_rec + (size_t)gid * grad_stride(G);
                 // lanes 4c .. 4c + 3 end with the total of float c
                 float v[8];

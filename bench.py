@@ -60,11 +60,6 @@ FLOP_CAND, FLOP_COMP_FWD, FLOP_COMP_BWD = 27, 12, 66
 MUFU_CAND, MUFU_COMP_BWD = 3, 4
 MUFU_PER_SM_CLK = 16           # special-function results per SM per clock
 SM_COUNT, FP32_LANES = 152, 128
-# kernels of one step: schedule advance 1 (graphs); project 1; bin: record counts 1, scans
-# (record and tile scans in one launch when both fit one CTA, 49,152 elements; beyond, the
-# record scan takes three launches plus the chunk table 1 and the tile scan six), scatter 1,
-# sorts 2; fused splat 1 + chain 1 (split: fwd 1, loss 1, bwd 1 + chain 1); Adam 2
-ONE_CTA_SCAN = 48 * 1024
 
 
 def roofline_entry(counts, stages, K, clocks, sha, peaks, regime=0):
@@ -129,23 +124,15 @@ def measured_peaks() -> dict:
         return {}
 
 
-def scan_launches(n: int, twice: bool = False) -> int:
-    if n <= ONE_CTA_SCAN:
-        return 1
-    return 6 if twice else 3
+def step_launches(fused: bool, graph: bool = True) -> int:
+    """Kernels of libps per optimisation step.  One library call (graphs): clearing and schedule
+    advance, projection with counts, two scans, scatter, sort, splat, chain with Adam.  Stage by
+    stage: projection, counts, two scans, scatter, sort, splat and chain (or forward, loss,
+    backward and chain), Adam in two launches."""
+    if fused and graph:
+        return 8
+    return 6 + (2 if fused else 4) + 2
 
-
-def step_launches(n_records: int, n_tiles: int, fused: bool, graph: bool = True) -> int:
-    """Kernels of libps per optimisation step: schedule advance (graph only), projection,
-    binning (counts, scans, scatter, two sorts), splat (+ chain), Adam (one launch for all
-    parameters in the graph step, two eagerly)."""
-    if 0 < n_records <= ONE_CTA_SCAN and n_tiles <= ONE_CTA_SCAN:
-        scans = 1
-    else:
-        scans = (scan_launches(n_records) + 1 if n_records > 0 else 0) + scan_launches(n_tiles, True)
-    binning = 1 + scans + 3
-    adam = 1 if graph else 2
-    return (int(graph) + 1 + binning + 2 + adam) if fused else (int(graph) + 1 + binning + 4 + adam)
 
 # DRAM bytes (read + write) and warp instructions (smsp__inst_executed.sum) per launch
 # of the fused splat kernel from the ncu captures summarised in
@@ -153,11 +140,11 @@ def step_launches(n_records: int, n_tiles: int, fused: bool, graph: bool = True)
 # .._ite1000.md, .._ite2000.md, .._ite4000.md (later points of the fit), keyed by the
 # regime's iteration; reported only while the kernel source is the one they were taken
 # on.  The issue roof is 152 SMs x 4 schedulers x one warp instruction per clock.
-CAPTURES = {"src_sha": "f57b7307b034ad09",
-            "splat_fused": {0: {"dram_bytes": 51238656, "warp_instructions": 392692133},
-                            1000: {"dram_bytes": 44233728, "warp_instructions": 152681978},
-                            2000: {"dram_bytes": 42898176, "warp_instructions": 122084604},
-                            4000: {"dram_bytes": 42422784, "warp_instructions": 109970373}}}
+CAPTURES = {"src_sha": "0da2c5833519367c",
+            "splat_fused": {0: {"dram_bytes": 51190784, "warp_instructions": 301960299},
+                            1000: {"dram_bytes": 44065792, "warp_instructions": 125205850},
+                            2000: {"dram_bytes": 42823424, "warp_instructions": 101321330},
+                            4000: {"dram_bytes": 42342400, "warp_instructions": 91234628}}}
 SCHEDULERS_PER_SM = 4
 
 
@@ -490,8 +477,7 @@ def run_ours(args, rank, world, local_rank):
         "eager_ms_per_step": round(sum(per_step_eager) / args.steps, 4),
         "wall_s_timed": round(wall, 4),
         "roofline": roofline, "clocks": clocks,
-        "gpu_launches": step_launches(int(wl.r.frame.n_records), int(wl.r.frame.n_tiles),
-                                      wl.fit.fused, graph=use_graphs) * args.steps,
+        "gpu_launches": step_launches(wl.fit.fused, graph=use_graphs) * args.steps,
         "culling": {"tested_per_candidate": round(tested / max(cand, 1), 2)},
     }
 

@@ -1,6 +1,6 @@
 """Builds libps.so (the sm_103a CUDA library) in-tree with nvcc.
 
-The three translation units compile in parallel and link into
+The translation units compile in parallel and link into
 ``paper_2412_03451_gb300/_lib/libps.so``.  Rebuilds only when a source or the
 public header is newer than the library.
 """

@@ -2,9 +2,10 @@
 
 PyTorch provides device memory and streams; every step of the rendering path
 (projection, binning, forward splat, loss, backward splat, Adam) is a call into
-libps through ``binding``.  The plane parameters of all scenes live in one flat
-float32 buffer laid out as [center P*3 | quat P*4 | radii P*4], so that Adam
-runs as two launches (the radii group is clamped to stay positive, Eq. 1).
+libps through ``binding``; a whole optimisation step is one call (ps_fit_step).
+The plane parameters of all scenes live in one flat float32 buffer laid out as
+[center P*3 | quat P*4 | radii P*4]; Adam clamps its tail, the radii, to stay
+positive (Eq. 1).
 """
 from __future__ import annotations
 

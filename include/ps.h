@@ -114,7 +114,7 @@ typedef struct ps_settings {
 /* Per-view descriptor, 128 bytes.  Filled on the host by ps_plan_views and
    copied to the device by the caller. */
 typedef struct ps_view {
-    float w2c[12];         /* world-to-camera [R|t], row-major 3x4 */
+    float w2c[12];         /* world-to-camera [R|t], row-major 3x4; R orthonormal (the backward relies on it) */
     float fx, fy, cx, cy;  /* intrinsics */
     int H, W;              /* image size */
     int tiles_x, tiles_y;  /* tile grid of this view */

@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_sums(ScanJob j0, ScanJob 
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) {
         const int j = i * kScanThreads + threadIdx.x;
-        const int x = j < m ? __ldg(&a.in[lo + j]) : 0;
+        const int x = j < m ? a.in[lo + j] : 0;
         D += x;
         S += (long long)x * (m - j);
     }
@@ -265,12 +265,12 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(ScanJob j0, ScanJob
 }
 
 // 3. one thread per (record, tile) pair ----------------------------------------
-__device__ __forceinline__ int pair_record(const int* __restrict__ off, int lo, int hi, int i)
+__device__ __forceinline__ int pair_record(const int* off, int lo, int hi, int i)
 {
     // last r in [lo, hi] with off[r] <= i (off is non-decreasing, off[lo] <= i)
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(&off[mid]) <= i) lo = mid; else hi = mid - 1;
+        if (off[mid] <= i) lo = mid; else hi = mid - 1;
     }
     return lo;
 }
@@ -280,14 +280,14 @@ __device__ __forceinline__ int pair_record(const int* __restrict__ off, int lo, 
 // the next chunk's (an upper bound); beyond the table the whole record range is
 // searched.  Every thread of the block computes the same two values (broadcast
 // loads, no barrier) and then searches only that narrow range for its own pair.
-__device__ __forceinline__ int2 chunk_record_range(const int* __restrict__ off, int R, int E, int base,
-                                                   const int* __restrict__ chunk_first, long long n_chunk)
+__device__ __forceinline__ int2 chunk_record_range(const int* off, int R, int E, int base,
+                                                   const int* chunk_first, long long n_chunk)
 {
     const long long c = base / kPairBlock;
-    const int lo = (c < n_chunk && c * kPairBlock < E) ? __ldg(&chunk_first[c])
+    const int lo = (c < n_chunk && c * kPairBlock < E) ? chunk_first[c]
                                                        : pair_record(off, 0, R - 1, base);
     const int hi = (c + 1 < n_chunk && (c + 1) * kPairBlock < E)
-                       ? __ldg(&chunk_first[c + 1])
+                       ? chunk_first[c + 1]
                        : pair_record(off, 0, R - 1, min(base + kPairBlock, E) - 1);
     return make_int2(lo, hi);
 }
@@ -332,35 +332,30 @@ __device__ __forceinline__ float entry_key(float4 ns, const ps_view* __restrict_
     return fmaxf(tmin, z_near);
 }
 
-__global__ void __launch_bounds__(kPairBlock) k_pair_scatter(const int* __restrict__ rec_off, int R,
-                                                       const int4* __restrict__ rec_info,
-                                                       const int* __restrict__ tile_ptr,
-                                                       int* __restrict__ cursor,
-                                                       unsigned long long* __restrict__ ent_tmp,
-                                                       const float4* __restrict__ rec,
-                                                       const float* __restrict__ rec_key,
-                                                       const ps_view* __restrict__ views,
-                                                       int tw, int th, float z_near,
-                                                       const int* __restrict__ chunk_first,
-                                                       long long n_chunk)
+__global__ void __launch_bounds__(kPairBlock) k_pair_scatter(const int* rec_off, int R, const int4* rec_info,
+                                                             const int* tile_ptr, int* cursor,
+                                                             unsigned long long* ent_tmp,
+                                                             const float4* rec, const float* rec_key,
+                                                             const ps_view* __restrict__ views,
+                                                             int tw, int th, float z_near,
+                                                             const int* chunk_first, long long n_chunk)
 {
     after_previous();
-    const int E = __ldg(&rec_off[R]);
+    const int E = rec_off[R];
     for (int base = blockIdx.x * kPairBlock; base < E; base += gridDim.x * kPairBlock) {
         const int2 rg = chunk_record_range(rec_off, R, E, base, chunk_first, n_chunk);
         const int i = base + threadIdx.x;
         if (i < E) {
             const int r = pair_record(rec_off, rg.x, rg.y, i);
-            const int4 info = __ldg(&rec_info[r]);
-            const int j = i - __ldg(&rec_off[r]);
+            const int4 info = rec_info[r];
+            const int j = i - rec_off[r];
             const int t = info.x + (j / info.y) * info.z + (j % info.y);
             // the key first, so that the slot atomic's latency overlaps nothing it waits on
             const ps_view* vw = views + info.w;
             const int lt = t - __ldg(&vw->tile_off);
-            const float k = fmaxf(entry_key(__ldg(&rec[4 * (size_t)r]), vw, lt % info.z, lt / info.z,
-                                            tw, th, z_near),
-                                  __ldg(&rec_key[r]));
-            const int lim = __ldg(&tile_ptr[t + 1]);
+            const float k = fmaxf(entry_key(rec[4 * (size_t)r], vw, lt % info.z, lt / info.z, tw, th, z_near),
+                                  rec_key[r]);
+            const int lim = tile_ptr[t + 1];
             const int pos = atomicAdd(&cursor[t], 1);
             // tile_ptr is clamped to the capacity: positions past it belong to lists
             // that did not fit and are dropped (the status word says so)
@@ -430,7 +425,7 @@ __device__ __forceinline__ void warp_bitonic(unsigned long long (&v)[E], int lan
 
 // Sorts the list of n slots from b (W = 32: the warp's one list; else this lane's group's).
 template <int W, int E>
-__device__ __forceinline__ void warp_sort_list(const unsigned long long* __restrict__ ent_tmp,
+__device__ __forceinline__ void warp_sort_list(const unsigned long long* ent_tmp,
                                                int* __restrict__ tile_ent, float* __restrict__ tile_key,
                                                int b, int n, int lane)
 {
@@ -444,7 +439,7 @@ __device__ __forceinline__ void warp_sort_list(const unsigned long long* __restr
         if (e * W + i < n) put(tile_ent, tile_key, b + e * W + i, v[e]);
 }
 
-__device__ void sort_long_list(const unsigned long long* __restrict__ ent_tmp,
+__device__ void sort_long_list(const unsigned long long* ent_tmp,
                                int* __restrict__ tile_ent, float* __restrict__ tile_key, int b, int n,
                                unsigned long long* s)
 {
@@ -493,8 +488,8 @@ __device__ void sort_long_list(const unsigned long long* __restrict__ ent_tmp,
 // planes in 8 views of 640x480 take 5.2 us (one list per warp and a second launch for the
 // long ones: 13.5 us), those of 16 uneven rooms 31 us (96 us), of 10,000 planes in 64 views
 // at lambda 20 118 us (169 us).
-__global__ void __launch_bounds__(kSortWarps * 32) k_sort(const int* __restrict__ tile_ptr, int n_tiles,
-                                                          const unsigned long long* __restrict__ ent_tmp,
+__global__ void __launch_bounds__(kSortWarps * 32) k_sort(const int* tile_ptr, int n_tiles,
+                                                          const unsigned long long* ent_tmp,
                                                           int* __restrict__ tile_ent,
                                                           float* __restrict__ tile_key)
 {
@@ -507,7 +502,7 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort(const int* __restrict_
     __syncthreads();
     const int t0 = (blockIdx.x * kSortWarps + w) * kSortTiles;
     // lane l < kSortTiles + 1: the start of tile t0 + l's list (past the last tile: its end)
-    const int ptr = __ldg(&tile_ptr[min(t0 + min(lane, kSortTiles), n_tiles)]);
+    const int ptr = tile_ptr[min(t0 + min(lane, kSortTiles), n_tiles)];
     const int len = __shfl_down_sync(0xffffffffu, ptr, 1) - ptr;      // lanes < kSortTiles
     const int n4[kSortTiles] = {__shfl_sync(0xffffffffu, len, 0), __shfl_sync(0xffffffffu, len, 1),
                                 __shfl_sync(0xffffffffu, len, 2), __shfl_sync(0xffffffffu, len, 3)};

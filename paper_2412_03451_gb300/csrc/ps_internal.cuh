@@ -30,6 +30,13 @@ namespace ps {
 // between them to count: an eager step of 64 planes in 8 views of 128x96 56 -> 43 us, a fitted
 // render of 8 views 121 -> 110, a hard one of 64 views 261 -> 250.  Under capture the launches are
 // ordinary: replayed steps were 0..2% slower with programmatic edges.
+//
+// Such a kernel is resident while the kernels before it still write, and its successors may be
+// too.  Whatever a kernel of the chain writes is therefore read by ordinary loads through
+// pointers without __restrict__: __ldg and const __restrict__ promise data that nobody writes
+// during the kernel's life, so such a load may move above the wait or find an older line.  They
+// are left for what is complete before the chain's first kernel (views, supervision, upstream
+// gradients, parameters).
 __device__ __forceinline__ void after_previous()
 {
     asm volatile("griddepcontrol.launch_dependents;");

@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(128) k_project(ProjArgs a)
             nc[i] = row3(R, i, nw);
         }
         // the Gaussian extent does not depend on lambda: the schedule's margin is not used
-        const float delta = (float)((a.d_state && !a.gauss) ? __ldg(&a.d_state->delta) : a.delta);
+        const float delta = (float)((a.d_state && !a.gauss) ? a.d_state->delta : a.delta);
         const float r0 = rf[0], r1 = a.single_radii ? rf[0] : rf[1];
         const float r2 = rf[2], r3 = a.single_radii ? rf[2] : rf[3];
 

@@ -264,7 +264,7 @@ __device__ __forceinline__ void composite(Walk<KP>& s, Sink& k, const float4& n,
 }
 
 template <int MODE, int KP>
-__device__ __forceinline__ void flush(Walk<KP>& s, Sink& k, const float4* __restrict__ rec,
+__device__ __forceinline__ void flush(Walk<KP>& s, Sink& k, const float4* rec,
                                       float bound, int M)
 {
     // every later candidate lies behind the cut: nothing else can enter (no cut: NaN, false)
@@ -277,7 +277,7 @@ __device__ __forceinline__ void flush(Walk<KP>& s, Sink& k, const float4* __rest
         const float w = s.bw[0];
         pend_pop(s);
         float4 n = make_float4(0.f, 0.f, 0.f, 0.f);
-        if constexpr (MODE != kBwd) n = __ldg(&rec[(size_t)key_id(k0) * 4]);
+        if constexpr (MODE != kBwd) n = rec[(size_t)key_id(k0) * 4];
         composite<MODE>(s, k, n, key_t(k0), w, key_id(k0), M);
     }
     if (final_ && s.nb == 0 && s.ovf == kNoKey) s.done = true;
@@ -318,14 +318,14 @@ __device__ __forceinline__ void walk_strip(const SplatArgs& a, WarpStage& ws, Wa
                                                       ws.rec[3][lane], g, a.c, t_low);
                 low = ws.key[lane];
             } else if (i < end) {
-                const int id = __ldg(&a.tile_ent[i]);
+                const int id = a.tile_ent[i];
                 const float4* r = a.rec + (size_t)id * 4;
-                const float4 n = __ldg(r + 0), vx = __ldg(r + 1), vy = __ldg(r + 2), rr = __ldg(r + 3);
+                const float4 n = r[0], vx = r[1], vy = r[2], rr = r[3];
                 float t_low;
                 ok = region_may_hit<SB>(n, vx, vy, rr, g, a.c, t_low, t_floor);
-                if constexpr (!SB) low = __ldg(&a.key[i]) * kMargin;
+                if constexpr (!SB) low = a.key[i] * kMargin;
                 if (GR || ok) {
-                    if constexpr (SB) low = fmaxf(__ldg(&a.key[i]), t_low) * kMargin;
+                    if constexpr (SB) low = fmaxf(a.key[i], t_low) * kMargin;
                     ws.id[lane] = id;
                     ws.rec[0][lane] = n; ws.rec[1][lane] = vx; ws.rec[2][lane] = vy; ws.rec[3][lane] = rr;
                 }
@@ -334,7 +334,7 @@ __device__ __forceinline__ void walk_strip(const SplatArgs& a, WarpStage& ws, Wa
             // with strip bounds it is the smallest bound of the chunk's surviving entries from e
             // on and of the next chunk's first key.
             if constexpr (SB) {
-                const float next = (base + 32 < end) ? __ldg(&a.key[base + 32]) * kMargin : INFINITY;
+                const float next = (base + 32 < end) ? a.key[base + 32] * kMargin : INFINITY;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) low = fminf(low, __shfl_down_sync(kFull, low, o));
                 ws.key[lane] = fminf(low, next);
@@ -342,7 +342,7 @@ __device__ __forceinline__ void walk_strip(const SplatArgs& a, WarpStage& ws, Wa
             } else {
                 ws.key[lane] = low;
                 if (lane == 0)
-                    ws.key[32] = (base + 32 < end) ? __ldg(&a.key[base + 32]) * kMargin : INFINITY;
+                    ws.key[32] = (base + 32 < end) ? a.key[base + 32] * kMargin : INFINITY;
             }
             unsigned m = __ballot_sync(kFull, ok);
             if constexpr (GR) staged = end - beg <= 32;
@@ -451,8 +451,8 @@ __device__ __forceinline__ TileCtx tile_setup(const SplatArgs& a, int tile)
     t.cx = __ldg(&vw->cx); t.cy = __ldg(&vw->cy);
     t.pix_off = __ldg(&vw->pix_off);
     t.gt_off = __ldg(&vw->gt_off);
-    t.beg = (int)min((long long)__ldg(&a.tile_ptr[tile]), a.capacity);
-    t.end = (int)min((long long)__ldg(&a.tile_ptr[tile + 1]), a.capacity);
+    t.beg = (int)min((long long)a.tile_ptr[tile], a.capacity);
+    t.end = (int)min((long long)a.tile_ptr[tile + 1], a.capacity);
     t.pad = 0;
     return t;
 }
@@ -570,7 +570,7 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
         if (wmax - 1 >= 0 && wmax - 1 < cnt) {
             nxt = k.stk[(wmax - 1) * 32];
             const float4* r = a.rec + (size_t)nxt.x * 4;
-            qn = __ldg(r + 0); qx = __ldg(r + 1); qy = __ldg(r + 2); qr = __ldg(r + 3);
+            qn = r[0]; qx = r[1]; qy = r[2]; qr = r[3];
         }
         for (int j = wmax - 1; j >= 0; --j) {
             const bool act = j < cnt;
@@ -583,7 +583,7 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
             if (j - 1 >= 0 && j - 1 < cnt) {
                 nxt = k.stk[(j - 1) * 32];
                 const float4* r = a.rec + (size_t)nxt.x * 4;
-                qn = __ldg(r + 0); qx = __ldg(r + 1); qy = __ldg(r + 2); qr = __ldg(r + 3);
+                qn = r[0]; qx = r[1]; qy = r[2]; qr = r[3];
             }
             if (act) {
                 id = e.x;
@@ -703,21 +703,21 @@ __device__ __forceinline__ void run_hard(const SplatArgs& a, WarpStage& ws, int 
     WarpRegion g;
     g.dxa = __shfl_sync(kFull, dx, 0); g.dxb = __shfl_sync(kFull, dx, WX - 1);
     g.den_min = 0.f;
-    const int beg = (int)min((long long)__ldg(&a.tile_ptr[tile]), a.capacity);
-    const int end = (int)min((long long)__ldg(&a.tile_ptr[tile + 1]), a.capacity);
+    const int beg = (int)min((long long)a.tile_ptr[tile], a.capacity);
+    const int end = (int)min((long long)a.tile_ptr[tile + 1], a.capacity);
     const bool one = end - beg <= 32;
     auto stage = [&](int base) {
         __syncwarp();                              // the last chunk has been read
         const int i = base + lane;
         if (i < end) {
-            const int id = __ldg(&a.tile_ent[i]);
+            const int id = a.tile_ent[i];
             const float4* r = a.rec + (size_t)id * 4;
             ws.id[lane] = id;
-            ws.key[lane] = __ldg(&a.key[i]) * kMargin;
+            ws.key[lane] = a.key[i] * kMargin;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) ws.rec[c][lane] = __ldg(r + c);
+            for (int c = 0; c < 4; ++c) ws.rec[c][lane] = r[c];
         }
-        if (lane == 0) ws.key[32] = (base + 32 < end) ? __ldg(&a.key[base + 32]) * kMargin : INFINITY;
+        if (lane == 0) ws.key[32] = (base + 32 < end) ? a.key[base + 32] * kMargin : INFINITY;
         __syncwarp();
     };
     if (one) stage(beg);
@@ -778,8 +778,8 @@ __device__ __forceinline__ void run_hard(const SplatArgs& a, WarpStage& ws, int 
 __device__ __forceinline__ void load_state(SplatArgs& a)
 {
     if (a.d_state && !a.c.hard && !a.c.gauss) {
-        a.c.lam5 = 5.f * __ldg(&a.d_state->lambda);
-        a.c.reject = (float)(__ldg(&a.d_state->delta) * 1.02 + 1e-6);
+        a.c.lam5 = 5.f * a.d_state->lambda;
+        a.c.reject = (float)(a.d_state->delta * 1.02 + 1e-6);
     }
 }
 

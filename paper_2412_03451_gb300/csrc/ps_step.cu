@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kChainThreads) k_chain_adam(ChainAdamArgs a)
         for (int c = 0; c < 11; ++c) s_g[at][c] = ok ? out[c] : 0.f;
     }
     __syncthreads();
-    const float bc1 = a.d_state ? __ldg(&a.d_state->bc1) : a.bc1, bc2 = a.d_state ? __ldg(&a.d_state->bc2) : a.bc2;
+    const float bc1 = a.d_state ? a.d_state->bc1 : a.bc1, bc2 = a.d_state ? a.d_state->bc2 : a.bc2;
 #pragma unroll
     for (int e = 0; e < kPer; ++e) {
         const int t = threadIdx.x + e * kChainThreads;

@@ -185,7 +185,7 @@ class Renderer:
 
     def read_required(self):
         """Copies the entry count of the last binning to the host without waiting; returns the
-        event after which required_now() may be read."""
+        event after which grow_if_needed() may be called."""
         if self._required_host is None:
             self._required_host = torch.empty(1, dtype=torch.int64, pin_memory=True)
         self._required_host.copy_(self.required, non_blocking=True)
@@ -194,10 +194,14 @@ class Renderer:
         return ready
 
     def grow_if_needed(self, headroom=1.5) -> bool:
-        """After read_required()'s event: grows the tile lists if the binning did not fit."""
+        """After read_required()'s event: grows the tile lists if the binning did not fit (waits
+        for the current stream then)."""
         need = int(self._required_host[0])
         if need <= self.capacity:
             return False
+        # a splat enqueued after that event may still be walking the old lists, which the
+        # allocator would hand back to the stream they were allocated on
+        torch.cuda.current_stream().synchronize()
         self._alloc_lists(int(need * headroom) + 1024)
         self.status.zero_()
         return True

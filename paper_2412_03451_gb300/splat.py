@@ -32,9 +32,15 @@ def flat_views(flat: torch.Tensor, P: int):
     return flat[:3 * P].view(P, 3), flat[3 * P:7 * P].view(P, 4), flat[7 * P:].view(P, 4)
 
 
+def plain_flat(flat: torch.Tensor, P: int) -> bool:
+    """Whether flat is one contiguous float32 run of P planes' parameters."""
+    return flat.dim() == 1 and flat.numel() == 11 * P and flat.is_contiguous() and flat.dtype is torch.float32
+
+
 def flat_ptrs(flat: torch.Tensor, P: int):
-    """Device pointers of the three groups (flat_views without making the views)."""
-    if flat.is_contiguous() and flat.dtype is torch.float32:
+    """Device pointers of the three groups (flat_views without making the views; what it refuses
+    is refused)."""
+    if plain_flat(flat, P):
         p = flat.data_ptr()
         return p, p + 12 * P, p + 28 * P
     return tuple(x.data_ptr() for x in flat_views(flat, P))
@@ -439,8 +445,7 @@ class Fitter:
 
     def _one_call(self) -> bool:
         """Whether the library's whole step takes these buffers."""
-        return all(t.is_contiguous() and t.dtype is torch.float32 and t.numel() == 11 * self.r.P
-                   for t in (self.flat, self.grad, self.m, self.v))
+        return all(plain_flat(t, self.r.P) for t in (self.flat, self.grad, self.m, self.v))
 
     def _library_step(self, settings, gt_depth, gt_normal, view_sums, batch, fused, schedule=()):
         """The whole step as one library call; schedule: d_state, d_sched, n_sched, d_iter."""

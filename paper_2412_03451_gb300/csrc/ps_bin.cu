@@ -56,6 +56,9 @@ constexpr int kScanItems = 9;      // elements per thread per scan tile (odd: a 
 constexpr int kScanTile = kScanThreads * kScanItems;
 constexpr int kFlatBlocks = 152 * 8;
 constexpr int kPairBlock = 256;       // pairs per scatter block = pairs per chunk of the chunk table
+// The pair numbering is clamped here.  A total that reaches it exceeds every capacity; the pairs
+// past it have no number, so nothing is scattered and the sort fills the truncated lists.
+constexpr int kMaxPairs = 0x7fffffff;
 
 inline long long n_chunks(long long capacity) { return capacity / kPairBlock + 2; }
 
@@ -342,10 +345,12 @@ __global__ void __launch_bounds__(kPairBlock) k_pair_scatter(const int* rec_off,
 {
     after_previous();
     const int E = rec_off[R];
-    for (int base = blockIdx.x * kPairBlock; base < E; base += gridDim.x * kPairBlock) {
-        const int2 rg = chunk_record_range(rec_off, R, E, base, chunk_first, n_chunk);
-        const int i = base + threadIdx.x;
-        if (i < E) {
+    if (E == kMaxPairs) return;
+    // (unsigned: the step past the last block may pass the int range)
+    for (unsigned base = blockIdx.x * kPairBlock; base < (unsigned)E; base += gridDim.x * kPairBlock) {
+        const int2 rg = chunk_record_range(rec_off, R, E, (int)base, chunk_first, n_chunk);
+        if (base + threadIdx.x < (unsigned)E) {
+            const int i = (int)(base + threadIdx.x);
             const int r = pair_record(rec_off, rg.x, rg.y, i);
             const int4 info = rec_info[r];
             const int j = i - rec_off[r];
@@ -360,7 +365,8 @@ __global__ void __launch_bounds__(kPairBlock) k_pair_scatter(const int* rec_off,
             // tile_ptr is clamped to the capacity: positions past it belong to lists
             // that did not fit and are dropped (the status word says so)
             // (keys are positive or +inf, so their bits sort like the values)
-            if (pos < lim) ent_tmp[pos] = ((unsigned long long)__float_as_uint(k) << 32) | (unsigned)r;
+            // (unsigned: a cursor may count past the int range)
+            if ((unsigned)pos < (unsigned)lim) ent_tmp[pos] = ((unsigned long long)__float_as_uint(k) << 32) | (unsigned)r;
         }
     }
 }
@@ -489,6 +495,7 @@ __device__ void sort_long_list(const unsigned long long* ent_tmp,
 // long ones: 13.5 us), those of 16 uneven rooms 31 us (96 us), of 10,000 planes in 64 views
 // at lambda 20 118 us (169 us).
 __global__ void __launch_bounds__(kSortWarps * 32) k_sort(const int* tile_ptr, int n_tiles,
+                                                          const int* pairs,
                                                           const unsigned long long* ent_tmp,
                                                           int* __restrict__ tile_ent,
                                                           float* __restrict__ tile_key)
@@ -500,6 +507,14 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort(const int* tile_ptr, i
     if (threadIdx.x == 0) s_cnt = 0;
     after_previous();
     __syncthreads();
+    if (*pairs == kMaxPairs) {
+        // nothing was scattered: every entry is record 0, behind every depth
+        const int t = blockIdx.x * kSortWarps * kSortTiles;
+        const int e = tile_ptr[min(t + kSortWarps * kSortTiles, n_tiles)];
+        for (int j = tile_ptr[t] + (int)threadIdx.x; j < e; j += kSortWarps * 32)
+            put(tile_ent, tile_key, j, (unsigned long long)__float_as_uint(INFINITY) << 32);
+        return;
+    }
     const int t0 = (blockIdx.x * kSortWarps + w) * kSortTiles;
     // lane l < kSortTiles + 1: the start of tile t0 + l's list (past the last tile: its end)
     const int ptr = tile_ptr[min(t0 + min(lane, kSortTiles), n_tiles)];
@@ -585,10 +600,10 @@ ps_status ps::bin_tiles(const ps_frame* frame, const ps_settings* s, const float
             PS_LAUNCH_CHECK();
         }
     }
-    // Pair numbering: offsets clamp at the int range (still non-decreasing), so pairs
-    // past it are never scattered, and the tile total then exceeds every capacity.
+    // Pair numbering: offsets clamp at the int range (still non-decreasing); the tile total
+    // then exceeds every capacity and nothing is scattered (kMaxPairs).
     const int tr = scan_tiles(R), tt = scan_tiles(frame->n_tiles);
-    const ScanJob jr{w.rec_cnt, R, w.rec_cnt, nullptr, (1LL << 31) - 1, nullptr, nullptr, 0,
+    const ScanJob jr{w.rec_cnt, R, w.rec_cnt, nullptr, kMaxPairs, nullptr, nullptr, 0,
                      w.chunk_first, nch, w.part, tr};
     const ScanJob jt{w.tile_cnt, frame->n_tiles, tile_ptr, w.cursor, capacity, d_required,
                      d_status, 1, nullptr, 0, w.part + tr, tt};
@@ -600,7 +615,7 @@ ps_status ps::bin_tiles(const ps_frame* frame, const ps_settings* s, const float
                                    s->tile_w, s->tile_h, s->z_near, w.chunk_first, nch));
         constexpr int per = kSortWarps * kSortTiles;
         PS_CUDA_CHECK(launch_after(k_sort, (frame->n_tiles + per - 1) / per, kSortWarps * 32, 0, st, tile_ptr,
-                                   frame->n_tiles, w.ent_tmp, tile_ent, tile_key));
+                                   frame->n_tiles, w.rec_cnt + R, w.ent_tmp, tile_ent, tile_key));
     }
     return PS_OK;
 }

@@ -116,15 +116,15 @@ __global__ void __launch_bounds__(128) k_conv_first(const uint8_t* __restrict__ 
         mbar_expect(bw, kWTap);
         tma_load_2d(smem_u32(wt), &tmW, 0, 0, bw);
     }
-    ok = mbar_wait(bw, 0);
-    uint32_t np = 0, nm = 0;                           // patches loaded, tiles multiplied
-    for (int b = blockIdx.x; b < B; b += gridDim.x) {
+    ok = !__syncthreads_or(!mbar_wait(bw, 0));
+    uint32_t np = 0, nm = 0;                           // patch loads issued, tiles multiplied
+    for (int b = blockIdx.x; ok && b < B; b += gridDim.x) {
         if (tid == 0) {
             bulk_wait_read<2>();                       // the last patch's copy has left (older than two stores)
             mbar_expect(bp, kPatch);
             bulk_load(smem_u32(patch), x + (size_t)b * kPatch, kPatch, bp);
         }
-        ok = ok && mbar_wait(bp, np++ & 1);
+        ok = mbar_wait(bp, np++ & 1);
         if (__syncthreads_or(!ok)) { ok = false; break; }
         if (tid == 0 && copy) {
             asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
@@ -164,12 +164,12 @@ __global__ void __launch_bounds__(128) k_conv_first(const uint8_t* __restrict__ 
                 bulk_commit();
             }
         }
-        if (!ok) break;
     }
     if (tid == 0) {
         if (!ok) {
             if (err) atomicOr(err, 1 << PS_ERR_TIMEOUT);
             // what is in flight gets another bounded wait before the memory is given up
+            mbar_wait(bw, 0);
             if (np) mbar_wait(bp, (np - 1) & 1);
             if (nm) mbar_wait(bm, (nm - 1) & 1);
         }
@@ -328,6 +328,7 @@ __global__ void __launch_bounds__(kInnerThreads, 1) k_conv_inner(const __grid_co
     if ((failed || out_failed) && tid == 0) {
         if (a.err) atomicOr(a.err, 1 << PS_ERR_TIMEOUT);
         // copies and MMAs in flight get another bounded wait before the memory is given up
+        mbar_wait(smem_u32(&w_full), 0);
         for (int j = issued > kStages ? issued - kStages : 0; j < issued; ++j) {
             mbar_wait(smem_u32(&full[j % kStages]), (uint32_t)((j / kStages) & 1));
             mbar_wait(smem_u32(&empty[j % kStages]), (uint32_t)((j / kStages) & 1), 1 << 16);

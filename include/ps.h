@@ -355,8 +355,9 @@ typedef struct ps_fit_buffers {
    ps_splat_fwd without alpha, ps_loss and ps_splat_bwd), ps_radii_grad_accum if split_acc is
    given, and ps_adam_step on all 11 P parameters (with the bias corrections of
    settings->d_state if that is set), the radii clamped at r_min (NaN: no clamp).  The results
-   of those calls, with fewer launches; the first error of one of them is returned.  n_planes
-   is the number of planes of all scenes. */
+   of those calls, with fewer launches; what any of them would refuse is refused before the
+   first launch, so that the schedule does not advance for it.  n_planes is the number of
+   planes of all scenes. */
 ps_status ps_fit_step(int n_planes, const ps_frame* frame, const ps_settings* settings,
                       const ps_fit_buffers* buffers, int fused, float lr, float b1, float b2,
                       float eps, float r_min, int step, ps_stream stream);

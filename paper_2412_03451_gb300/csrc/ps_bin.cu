@@ -575,10 +575,9 @@ ps_status ps::bin_count(const ps_frame* frame, long long capacity, void* ws, siz
     return PS_OK;
 }
 
-ps_status ps::bin_tiles(const ps_frame* frame, const ps_settings* s, const float* rec, const int* rect,
-                        const float* key, int* tile_ptr, int* tile_ent, float* tile_key, long long capacity,
-                        long long* d_required, void* ws, size_t ws_bytes_, bool counted, int* d_status,
-                        cudaStream_t st)
+ps_status ps::check_bin(const ps_frame* frame, const ps_settings* s, const float* rec, const int* rect,
+                        const float* key, const int* tile_ptr, const int* tile_ent, const float* tile_key,
+                        long long capacity, const long long* d_required, void* ws, size_t ws_bytes_)
 {
     if (!frame || !s || !rec || !rect || !key || !tile_ptr || !d_required || !ws || !frame->views)
         return PS_ERR_ARG;
@@ -587,8 +586,19 @@ ps_status ps::bin_tiles(const ps_frame* frame, const ps_settings* s, const float
     if (reinterpret_cast<uintptr_t>(rec) & 15) return PS_ERR_ARG;
     if (reinterpret_cast<uintptr_t>(rect) & 15) return PS_ERR_ARG;
     BinCount cnt;
-    const ps_status e = bin_count(frame, capacity, ws, ws_bytes_, &cnt);
+    return bin_count(frame, capacity, ws, ws_bytes_, &cnt);
+}
+
+ps_status ps::bin_tiles(const ps_frame* frame, const ps_settings* s, const float* rec, const int* rect,
+                        const float* key, int* tile_ptr, int* tile_ent, float* tile_key, long long capacity,
+                        long long* d_required, void* ws, size_t ws_bytes_, bool counted, int* d_status,
+                        cudaStream_t st)
+{
+    const ps_status e = check_bin(frame, s, rec, rect, key, tile_ptr, tile_ent, tile_key, capacity, d_required,
+                                  ws, ws_bytes_);
     if (e != PS_OK) return e;
+    BinCount cnt;
+    bin_count(frame, capacity, ws, ws_bytes_, &cnt);
     const int R = frame->n_records;
     BinWs w = carve(ws, R, frame->n_tiles, capacity, nullptr);
     const long long nch = n_chunks(capacity);

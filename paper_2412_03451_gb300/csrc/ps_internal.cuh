@@ -350,6 +350,28 @@ __device__ __forceinline__ void count_record(const BinCount& b, size_t r, const 
     b.rec_info[r] = info;
 }
 
+// What the entry points of a step ask of their arguments: PS_OK, or what they return before
+// anything is launched.
+ps_status check_project(const ps_planes* planes, const ps_frame* frame, const ps_settings* s, const float* rec,
+                        const int* rect, const float* key);
+ps_status check_bin(const ps_frame* frame, const ps_settings* s, const float* rec, const int* rect,
+                    const float* key, const int* tile_ptr, const int* tile_ent, const float* tile_key,
+                    long long capacity, const long long* d_required, void* ws, size_t ws_bytes);
+ps_status check_fwd(const ps_frame* f, const ps_settings* s, const float* rec, const float* key,
+                    const int* tile_ptr, const int* tile_ent, long long capacity, const float* depth,
+                    const float* normal, void* ws, size_t ws_bytes);
+ps_status check_loss(const ps_frame* f, const ps_settings* s, const float* depth, const float* normal,
+                     const float* gt_depth, const float* gt_normal, const float* dLdD, const float* dLdN,
+                     const double* view_sums);
+ps_status check_bwd(const ps_planes* planes, const ps_frame* f, const ps_settings* s, const float* rec,
+                    const float* key, const int* tile_ptr, const int* tile_ent, long long capacity,
+                    const float* dLdD, const float* dLdN, const float* g_center, const float* g_quat,
+                    const float* g_radii, void* ws, size_t ws_bytes);
+ps_status check_fused(const ps_planes* planes, const ps_frame* f, const ps_settings* s, const float* rec,
+                      const float* key, const int* tile_ptr, const int* tile_ent, long long capacity,
+                      const float* gt_depth, const float* gt_normal, const float* g_radii, void* ws,
+                      size_t ws_bytes);
+
 // The parts of a step that ps_fit_step runs with less between them than the entry points do.
 // project with `count` leaves the binning's counts as well (diff zeroed before).
 ps_status project(const ps_planes* planes, const ps_frame* frame, const ps_settings* s, float* rec, int* rect,

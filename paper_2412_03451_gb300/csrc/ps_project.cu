@@ -273,8 +273,8 @@ __global__ void __launch_bounds__(128) k_project(ProjArgs a)
 
 }  // namespace
 
-ps_status ps::project(const ps_planes* planes, const ps_frame* frame, const ps_settings* s, float* rec,
-                      int* rect, float* key, const BinCount* count, int* d_status, cudaStream_t st)
+ps_status ps::check_project(const ps_planes* planes, const ps_frame* frame, const ps_settings* s,
+                            const float* rec, const int* rect, const float* key)
 {
     if (!planes || !frame || !s || !rec || !rect || !key || !frame->views) return PS_ERR_ARG;
     if (!planes->center || !planes->quat || !planes->radii) return PS_ERR_ARG;
@@ -285,6 +285,14 @@ ps_status ps::project(const ps_planes* planes, const ps_frame* frame, const ps_s
     if (!(s->z_near > 0.f) || !(s->z_far > s->z_near)) return PS_ERR_ARG;
     if ((reinterpret_cast<uintptr_t>(rec) & 15) || (reinterpret_cast<uintptr_t>(rect) & 15))
         return PS_ERR_ARG;
+    return PS_OK;
+}
+
+ps_status ps::project(const ps_planes* planes, const ps_frame* frame, const ps_settings* s, float* rec,
+                      int* rect, float* key, const BinCount* count, int* d_status, cudaStream_t st)
+{
+    const ps_status e = check_project(planes, frame, s, rec, rect, key);
+    if (e != PS_OK) return e;
     if (frame->max_K == 0 || frame->n_records == 0) return PS_OK;
     ProjArgs a{};
     a.center = planes->center; a.quat = planes->quat; a.radii = planes->radii;

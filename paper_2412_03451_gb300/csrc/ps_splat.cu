@@ -1273,15 +1273,24 @@ extern "C" size_t ps_fwd_workspace_bytes(const ps_frame* f)
     return kCounterBytes;
 }
 
+ps_status ps::check_fwd(const ps_frame* f, const ps_settings* s, const float* rec, const float* key,
+                        const int* tile_ptr, const int* tile_ent, long long capacity, const float* depth,
+                        const float* normal, void* ws, size_t ws_bytes)
+{
+    const ps_status e = check_common(f, s, rec, key, tile_ptr, tile_ent, capacity);
+    if (e != PS_OK) return e;
+    if (!depth || !normal || !ws) return PS_ERR_ARG;
+    if (ws_bytes < kCounterBytes || (reinterpret_cast<uintptr_t>(ws) & 15)) return PS_ERR_ARG;
+    return PS_OK;
+}
+
 extern "C" ps_status ps_splat_fwd(const ps_frame* f, const ps_settings* s, const float* rec,
                                   const float* key, const int* tile_ptr, const int* tile_ent,
                                   long long capacity, float* depth, float* normal, float* alpha,
                                   void* ws, size_t ws_bytes, int* d_status, ps_stream stream)
 {
-    ps_status e = check_common(f, s, rec, key, tile_ptr, tile_ent, capacity);
+    const ps_status e = check_fwd(f, s, rec, key, tile_ptr, tile_ent, capacity, depth, normal, ws, ws_bytes);
     if (e != PS_OK) return e;
-    if (!depth || !normal || !ws) return PS_ERR_ARG;
-    if (ws_bytes < kCounterBytes || (reinterpret_cast<uintptr_t>(ws) & 15)) return PS_ERR_ARG;
     SplatArgs a{};
     a.views = f->views; a.n_views = f->n_views;
     a.rec = reinterpret_cast<const float4*>(rec); a.key = key;
@@ -1321,18 +1330,29 @@ extern "C" size_t ps_bwd_workspace_bytes(const ps_frame* f)
     return fused_bytes(f);
 }
 
+ps_status ps::check_bwd(const ps_planes* planes, const ps_frame* f, const ps_settings* s, const float* rec,
+                        const float* key, const int* tile_ptr, const int* tile_ent, long long capacity,
+                        const float* dLdD, const float* dLdN, const float* g_center, const float* g_quat,
+                        const float* g_radii, void* ws, size_t ws_bytes)
+{
+    const ps_status e = check_common(f, s, rec, key, tile_ptr, tile_ent, capacity);
+    if (e != PS_OK) return e;
+    if (!planes || !planes->center || !planes->quat || !planes->radii) return PS_ERR_ARG;
+    if (!dLdD || !dLdN || !g_center || !g_quat || !g_radii || !ws) return PS_ERR_ARG;
+    if (s->flags & PS_HARD) return PS_ERR_ARG;
+    if (ws_bytes < bwd_ws(f) || (reinterpret_cast<uintptr_t>(ws) & 15)) return PS_ERR_ARG;
+    return PS_OK;
+}
+
 extern "C" ps_status ps_splat_bwd(const ps_planes* planes, const ps_frame* f, const ps_settings* s,
                                   const float* rec, const float* key, const int* tile_ptr,
                                   const int* tile_ent, long long capacity, const float* dLdD,
                                   const float* dLdN, float* g_center, float* g_quat, float* g_radii,
                                   void* ws, size_t ws_bytes, int* d_status, ps_stream stream)
 {
-    ps_status e = check_common(f, s, rec, key, tile_ptr, tile_ent, capacity);
+    const ps_status e = check_bwd(planes, f, s, rec, key, tile_ptr, tile_ent, capacity, dLdD, dLdN, g_center,
+                                  g_quat, g_radii, ws, ws_bytes);
     if (e != PS_OK) return e;
-    if (!planes || !planes->center || !planes->quat || !planes->radii) return PS_ERR_ARG;
-    if (!dLdD || !dLdN || !g_center || !g_quat || !g_radii || !ws) return PS_ERR_ARG;
-    if (s->flags & PS_HARD) return PS_ERR_ARG;
-    if (ws_bytes < bwd_ws(f) || (reinterpret_cast<uintptr_t>(ws) & 15)) return PS_ERR_ARG;
     if (f->n_records == 0) return PS_OK;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const size_t grec_bytes = grad_bytes(f, s);
@@ -1367,20 +1387,31 @@ ps_status ps::fused_ws(const ps_frame* f, const ps_settings* s, void* ws, size_t
     return PS_OK;
 }
 
+ps_status ps::check_fused(const ps_planes* planes, const ps_frame* f, const ps_settings* s, const float* rec,
+                          const float* key, const int* tile_ptr, const int* tile_ent, long long capacity,
+                          const float* gt_depth, const float* gt_normal, const float* g_radii, void* ws,
+                          size_t ws_bytes)
+{
+    const ps_status e = check_common(f, s, rec, key, tile_ptr, tile_ent, capacity);
+    if (e != PS_OK) return e;
+    if (!planes || !planes->center || !planes->quat || !planes->radii) return PS_ERR_ARG;
+    if (!gt_depth || !gt_normal || !g_radii) return PS_ERR_ARG;
+    if (s->flags & PS_HARD) return PS_ERR_ARG;
+    FusedWs w;
+    return fused_ws(f, s, ws, ws_bytes, &w);
+}
+
 ps_status ps::splat_fused(const ps_planes* planes, const ps_frame* f, const ps_settings* s, const float* rec,
                           const float* key, const int* tile_ptr, const int* tile_ent, long long capacity,
                           const float* gt_depth, const float* gt_normal, float* depth, float* normal,
                           float* dL_dD, float* dL_dN, float* g_radii, void* ws, size_t ws_bytes, bool cleared,
                           int* d_status, cudaStream_t st)
 {
-    ps_status e = check_common(f, s, rec, key, tile_ptr, tile_ent, capacity);
+    const ps_status e = check_fused(planes, f, s, rec, key, tile_ptr, tile_ent, capacity, gt_depth, gt_normal,
+                                    g_radii, ws, ws_bytes);
     if (e != PS_OK) return e;
-    if (!planes || !planes->center || !planes->quat || !planes->radii) return PS_ERR_ARG;
-    if (!gt_depth || !gt_normal || !g_radii) return PS_ERR_ARG;
-    if (s->flags & PS_HARD) return PS_ERR_ARG;
     FusedWs w;
-    e = fused_ws(f, s, ws, ws_bytes, &w);
-    if (e != PS_OK) return e;
+    fused_ws(f, s, ws, ws_bytes, &w);
     // record gradients, work counter and partial loss sums: one memset
     if (!cleared) PS_CUDA_CHECK(cudaMemsetAsync(ws, 0, w.bytes, st));
     SplatArgs a{};
@@ -1423,14 +1454,23 @@ extern "C" ps_status ps_splat_fused(const ps_planes* planes, const ps_frame* f,
     return PS_OK;
 }
 
-extern "C" ps_status ps_loss(const ps_frame* f, const ps_settings* s, const float* depth,
-                             const float* normal, const float* gt_depth, const float* gt_normal,
-                             float* dLdD, float* dLdN, double* view_sums, ps_stream stream)
+ps_status ps::check_loss(const ps_frame* f, const ps_settings* s, const float* depth, const float* normal,
+                         const float* gt_depth, const float* gt_normal, const float* dLdD, const float* dLdN,
+                         const double* view_sums)
 {
     if (!f || !s || !f->views || !depth || !normal || !gt_depth || !gt_normal || !dLdD || !dLdN ||
         !view_sums)
         return PS_ERR_ARG;
     if (f->n_views <= 0) return PS_ERR_ARG;
+    return PS_OK;
+}
+
+extern "C" ps_status ps_loss(const ps_frame* f, const ps_settings* s, const float* depth,
+                             const float* normal, const float* gt_depth, const float* gt_normal,
+                             float* dLdD, float* dLdN, double* view_sums, ps_stream stream)
+{
+    const ps_status e = check_loss(f, s, depth, normal, gt_depth, gt_normal, dLdD, dLdN, view_sums);
+    if (e != PS_OK) return e;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     PS_CUDA_CHECK(cudaMemsetAsync(view_sums, 0, sizeof(double) * 4 * (size_t)f->n_views, st));
     LossArgs a;

@@ -158,13 +158,31 @@ extern "C" ps_status ps_fit_step(int n_planes, const ps_frame* frame, const ps_s
     pl.n_planes = n_planes;
     pl.center = b->params; pl.quat = b->params + 3 * P; pl.radii = b->params + 7 * P;
     float *gc = b->grad, *gq = b->grad + 3 * P, *gr = b->grad + 7 * P;
-    ps_status e;
+    // every argument first: nothing is launched, and the schedule not advanced, for a refused step
+    ps_status e = check_project(&pl, frame, s, b->rec, b->rect, b->key);
+    if (e != PS_OK) return e;
+    e = check_bin(frame, s, b->rec, b->rect, b->key, b->tile_ptr, b->tile_ent, b->tile_key, b->capacity,
+                  b->d_required, b->bin_ws, b->bin_ws_bytes);
+    if (e != PS_OK) return e;
     if (fused) {
         if (!b->view_sums) return PS_ERR_ARG;
+        e = check_fused(&pl, frame, s, b->rec, b->tile_key, b->tile_ptr, b->tile_ent, b->capacity, b->gt_depth,
+                        b->gt_normal, gr, b->bwd_ws, b->bwd_ws_bytes);
+    } else {
+        e = check_fwd(frame, s, b->rec, b->tile_key, b->tile_ptr, b->tile_ent, b->capacity, b->depth, b->normal,
+                      b->fwd_ws, b->fwd_ws_bytes);
+        if (e != PS_OK) return e;
+        e = check_loss(frame, s, b->depth, b->normal, b->gt_depth, b->gt_normal, b->dL_dD, b->dL_dN, b->view_sums);
+        if (e != PS_OK) return e;
+        e = check_bwd(&pl, frame, s, b->rec, b->tile_key, b->tile_ptr, b->tile_ent, b->capacity, b->dL_dD,
+                      b->dL_dN, gc, gq, gr, b->bwd_ws, b->bwd_ws_bytes);
+    }
+    if (e != PS_OK) return e;
+    if (fused) {
         BinCount count;
         FusedWs w;
-        if ((e = bin_count(frame, b->capacity, b->bin_ws, b->bin_ws_bytes, &count)) != PS_OK) return e;
-        if ((e = fused_ws(frame, s, b->bwd_ws, b->bwd_ws_bytes, &w)) != PS_OK) return e;
+        bin_count(frame, b->capacity, b->bin_ws, b->bin_ws_bytes, &count);
+        fused_ws(frame, s, b->bwd_ws, b->bwd_ws_bytes, &w);
         BeginArgs a{};
         // (the counts' buffer is padded to 256 bytes, the splat's range is whole 16 bytes)
         a.zero[0] = reinterpret_cast<uint4*>(count.diff); a.n[0] = (count.n_tiles + 3) / 4;

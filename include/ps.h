@@ -114,7 +114,7 @@ typedef struct ps_settings {
 /* Per-view descriptor, 128 bytes.  Filled on the host by ps_plan_views and
    copied to the device by the caller. */
 typedef struct ps_view {
-    float w2c[12];         /* world-to-camera [R|t], row-major 3x4; R orthonormal (the backward relies on it) */
+    float w2c[12];         /* world-to-camera [R|t], row-major 3x4 */
     float fx, fy, cx, cy;  /* intrinsics */
     int H, W;              /* image size */
     int tiles_x, tiles_y;  /* tile grid of this view */
@@ -249,8 +249,8 @@ size_t ps_bwd_workspace_bytes(const ps_frame* frame);
    forward), takes the adjoint of Eq. 11-13 back to front
    (A_j = w_j t_j + (1 - w_j) A_{j+1}, dD/dw_j = T_j (t_j - A_{j+1}); no
    division by 1 - w), chains it through Eq. 9, 7-8, 6, 4 into per-record
-   gradients and then through Eq. 2-3 (with the quaternion normalisation; the
-   camera's rotation drops out) into the world parameters.  The clamp
+   gradients and then through the camera transform and Eq. 2-3 (with the
+   quaternion normalisation) into the world parameters.  The clamp
    min(1, .) has derivative 0 where m >= 0.  Ties of Eq. 9 go to the Y side.
    g_center [P][3], g_quat [P][4], g_radii [P][4] (device) are ACCUMULATED
    into (the caller zeroes them).  ws (device, >= ps_bwd_workspace_bytes) is

@@ -257,40 +257,63 @@ __device__ __forceinline__ double slot_sum(const double* vs_slots, int v, int c)
     return t;
 }
 
-// A plane's record gradients (sums over any of its records) -> world parameters (Eq. 2-3 and
-// the quaternion normalisation): out = center 3, quaternion 4, radii 4.  Returns false for a
-// quaternion without a direction.
-__device__ __forceinline__ bool chain_plane(const float4& g0, const float4& g3, float gax, float gay,
-                                            float q0, float q1, float q2, float q3, int single_radii,
-                                            float (&out)[11])
+// A plane's axes (Eq. 2-3): columns of the Hamilton matrix of its normalised quaternion.
+struct PlaneAxes {
+    float vx[3], vy[3], n[3];
+    float w, x, y, z, norm;    // the normalised quaternion and the length it was divided by
+};
+
+// Returns false for a quaternion without a direction.
+__device__ __forceinline__ bool plane_axes(float q0, float q1, float q2, float q3, PlaneAxes& o)
 {
     const float qs = sqrtf(q0 * q0 + q1 * q1 + q2 * q2 + q3 * q3);
-    if (!(qs > 0.f) || !isfinite(qs)) return false;
     const float w = q0 / qs, x = q1 / qs, y = q2 / qs, z = q3 / qs;
-    // world axes: columns of the Hamilton matrix (Eq. 2-3)
-    const float vx[3] = {1.f - 2.f * (y * y + z * z), 2.f * (x * y + w * z), 2.f * (x * z - w * y)};
-    const float vy[3] = {2.f * (x * y - w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z + w * x)};
-    const float nn[3] = {2.f * (x * z + w * y), 2.f * (y * z - w * x), 1.f - 2.f * (x * x + y * y)};
-    // The centre moves s = n_c . p_c, a_x and a_y; the camera rotation takes n_c, v^x_c, v^y_c
-    // back to the world axes, so the world gradient is their combination.
+    o.w = w; o.x = x; o.y = y; o.z = z; o.norm = qs;
+    o.vx[0] = 1.f - 2.f * (y * y + z * z); o.vx[1] = 2.f * (x * y + w * z); o.vx[2] = 2.f * (x * z - w * y);
+    o.vy[0] = 2.f * (x * y - w * z); o.vy[1] = 1.f - 2.f * (x * x + z * z); o.vy[2] = 2.f * (y * z + w * x);
+    o.n[0] = 2.f * (x * z + w * y); o.n[1] = 2.f * (y * z - w * x); o.n[2] = 1.f - 2.f * (x * x + y * y);
+    return qs > 0.f && isfinite(qs);
+}
+
+// Adds one record's part of the centre's gradient.  The centre moves s = n_c . p_c, a_x and a_y
+// with p_c = R c + t and the axes n_c = R n, ..., so the part is R^T R (gs n + gax v^x + gay v^y):
+// for any 3x3 block R of the view's w2c, orthonormal or not.
+__device__ __forceinline__ void add_centre(float (&g)[3], const PlaneAxes& a, float gs, float gax, float gay,
+                                           const ps_view* vw)
+{
+    float R[9], u[3], y[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) out[i] = g0.x * nn[i] + gax * vx[i] + gay * vy[i];
-    // A turn by theta in the plane's own frame moves v^x by theta_z v^y - theta_y n, v^y by
-    // theta_x n - theta_z v^x and n by theta_y v^x - theta_x v^y.  At a fixed centre the
-    // gradient of n lies along v^x (g0.y) and v^y (g0.z), those of v^x and v^y in the plane
-    // with the moment g0.w about n; parts along an axis itself do not turn it.  With
-    // dq = q (0, theta) / 2 the quaternion gradient is 2 q (0, torque) / |q|.
-    const float tx = -g0.z, ty = g0.y, tz = g0.w;
-    const float s2 = 2.f / qs;
-    out[3] = s2 * -(x * tx + y * ty + z * tz);
-    out[4] = s2 * (w * tx + y * tz - z * ty);
-    out[5] = s2 * (w * ty + z * tx - x * tz);
-    out[6] = s2 * (w * tz + x * ty - y * tx);
-    out[7] = single_radii ? g3.x + g3.y : g3.x;
-    out[8] = single_radii ? 0.f : g3.y;
-    out[9] = single_radii ? g3.z + g3.w : g3.z;
-    out[10] = single_radii ? 0.f : g3.w;
-    return true;
+    for (int i = 0; i < 9; ++i) R[i] = __ldg(&vw->w2c[4 * (i / 3) + i % 3]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) u[i] = fmaf(gs, a.n[i], fmaf(gax, a.vx[i], gay * a.vy[i]));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) y[i] = fmaf(R[3 * i], u[0], fmaf(R[3 * i + 1], u[1], R[3 * i + 2] * u[2]));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) g[i] = fmaf(R[i], y[0], fmaf(R[3 + i], y[1], fmaf(R[6 + i], y[2], g[i])));
+}
+
+// The torque and the radii of a plane's record gradients (sums over any of its records) ->
+// quaternion 4 and radii 4 of the world parameters.
+//
+// A turn by theta in the plane's own frame moves v^x by theta_z v^y - theta_y n, v^y by theta_x n -
+// theta_z v^x and n by theta_y v^x - theta_x v^y, and R takes them to the camera.  At a fixed centre
+// what the gradients of n_c, v^x_c and v^y_c find along the others' axes are the moments (mx, my, mz)
+// = record floats 1-3, whatever R is: the gradients of v^x_c and v^y_c are multiples of q = t d - p_c
+// and that of n_c is one of q and the normal's, with n_c . q = 0, v^x_c . q = P_X, v^y_c . q = P_Y.
+// With dq = quat (0, theta) / 2 the quaternion gradient is 2 quat (0, torque) / |quat|.
+__device__ __forceinline__ void chain_turn(const PlaneAxes& a, float mx, float my, float mz, const float4& g3,
+                                           int single_radii, float (&out)[8])
+{
+    const float tx = -my, ty = mx, tz = mz;
+    const float s2 = 2.f / a.norm;
+    out[0] = s2 * -(a.x * tx + a.y * ty + a.z * tz);
+    out[1] = s2 * (a.w * tx + a.y * tz - a.z * ty);
+    out[2] = s2 * (a.w * ty + a.z * tx - a.x * tz);
+    out[3] = s2 * (a.w * tz + a.x * ty - a.y * tx);
+    out[4] = single_radii ? g3.x + g3.y : g3.x;
+    out[5] = single_radii ? 0.f : g3.y;
+    out[6] = single_radii ? g3.z + g3.w : g3.z;
+    out[7] = single_radii ? 0.f : g3.w;
 }
 
 // Adam with bias correction; values below `lowest` (NaN: none) are raised to it.

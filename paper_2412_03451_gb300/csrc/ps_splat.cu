@@ -34,9 +34,10 @@
 // parameters.  8 floats suffice because the axes of a plane turn together: the
 // record keeps the gradients of s and of the radii and the three moments of the
 // axis gradients in the plane's own frame, built from the intersection relative to
-// the centre, t d - p_c = P_X v^x + P_Y v^y (so no metre-sized terms are summed only
-// to cancel), and the gradient of a_x is that of r^x+ less that of r^x- (a pair's
-// margin is r - |P|).  The camera rotation drops out of the chain.  The kernel is
+// the centre, q = t d - p_c with n_c . q = 0, v^x_c . q = P_X, v^y_c . q = P_Y (so no
+// metre-sized terms are summed only to cancel), and the gradient of a_x is that of
+// r^x+ less that of r^x- (a pair's margin is r - |P|).  None of this asks w2c's 3x3 block
+// to be orthonormal; only the centre's gradient meets it again, as R^T R.  The kernel is
 // bound by instruction issue, so what counts is the length of the aggregation: with
 // the 16 floats of n_c, s, v^x_c, a_x, v^y_c, a_y and the radii, summed in two halves
 // of 8, a step of the 3,000-plane room at 8 x 640x480 took 461 us at the first lambda (with 8
@@ -636,8 +637,8 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
                         atomicAdd(&a.g_radii[4 * (size_t)p + (a.single_radii ? (ridx & 2) : ridx)], gm);
                     }
                 }
-                // Eq. 4: t = s / (d . n_c); at a fixed p_c, dt/dn_c = (p_c - t d) / (d . n_c)
-                // with t d - p_c = P_X v^x + P_Y v^y (Eq. 6 on the plane)
+                // Eq. 4: t = s / (d . n_c); at a fixed p_c, dt/dn_c = (p_c - t d) / (d . n_c),
+                // whose products with v^x_c and v^y_c are -P_X and -P_Y over d . n_c (Eq. 6)
                 const float gs = __fdividef(gt, pe.den);
                 const float gNx = fmaf(gN0, vx.x, fmaf(gN1, vx.y, gN2 * vx.z));
                 const float gNy = fmaf(gN0, vy.x, fmaf(gN1, vy.y, gN2 * vy.z));
@@ -995,16 +996,19 @@ __global__ void __launch_bounds__(128) k_chain(ChainArgs a)
         g3.z == 0.f && g3.w == 0.f && gax == 0.f && gay == 0.f)
         return;
     const int p = __ldg(&vw->plane_off) + k;
-    float g[11];
-    if (!chain_plane(g0, g3, gax, gay, __ldg(&a.quat[4 * p + 0]), __ldg(&a.quat[4 * p + 1]),
-                     __ldg(&a.quat[4 * p + 2]), __ldg(&a.quat[4 * p + 3]), a.single_radii, g))
+    PlaneAxes ax;
+    if (!plane_axes(__ldg(&a.quat[4 * p + 0]), __ldg(&a.quat[4 * p + 1]), __ldg(&a.quat[4 * p + 2]),
+                    __ldg(&a.quat[4 * p + 3]), ax))
         return;
+    float gc[3] = {}, g[8];
+    add_centre(gc, ax, g0.x, gax, gay, vw);
+    chain_turn(ax, g0.y, g0.z, g0.w, g3, a.single_radii, g);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) atomicAdd(&a.g_center[3 * p + i], g[i]);
+    for (int i = 0; i < 3; ++i) atomicAdd(&a.g_center[3 * p + i], gc[i]);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        atomicAdd(&a.g_quat[4 * p + i], g[3 + i]);
-        atomicAdd(&a.g_radii[4 * p + i], g[7 + i]);
+        atomicAdd(&a.g_quat[4 * p + i], g[i]);
+        atomicAdd(&a.g_radii[4 * p + i], g[4 + i]);
     }
 }
 

@@ -61,8 +61,8 @@ struct ChainAdamArgs {
     int plane_blocks;                // blocks of planes; the rest add up the views' loss sums
 };
 
-// Eight lanes per plane add up its records over the views of its scene, one lane chains the
-// sum, then the block writes its planes' gradients and updates their parameters in order of
+// Eight lanes per plane add up its records over the views of its scene (the centre's part by each
+// view's rotation), one lane chains the sum, then the block writes its planes' gradients and updates their parameters in order of
 // address.  grad holds the radii's direct part (pairs at P = 0) on entry.  Bound by the latency
 // of its dependent loads, so what Adam reads is loaded before the chain.  3,000 planes in 8 views:
 // 7.8 -> 5.6 us; 64 planes, a whole eager step 42 -> 37.
@@ -92,8 +92,13 @@ __global__ void __launch_bounds__(kChainThreads) k_chain_adam(ChainAdamArgs a)
             gv[e] = t < 7 * n ? 0.f : a.grad[idx[e]];
         }
     }
+    // centre 3, moments 3, radii 4
     float g[10] = {};
+    PlaneAxes ax;
+    bool ok = false;
     if (p < a.P) {
+        const float* q = a.params + 3 * (size_t)a.P + 4 * (size_t)p;
+        ok = plane_axes(q[0], q[1], q[2], q[3], ax);
         // planes of a scene are consecutive and its views too: the last view whose planes start
         // at or before p is the last view of p's scene, if that scene has views at all
         int lo = 0, hi = a.n_views - 1;
@@ -107,9 +112,14 @@ __global__ void __launch_bounds__(kChainThreads) k_chain_adam(ChainAdamArgs a)
                 const size_t r = (size_t)__ldg(&a.views[v].rec_off) + k;
                 const float4* q = reinterpret_cast<const float4*>(a.g_rec + r * grad_stride(a.gauss));
                 const float4 x = q[0], y = q[1];
-                g[0] += x.x; g[1] += x.y; g[2] += x.z; g[3] += x.w;
-                g[4] += y.x; g[5] += y.y; g[6] += y.z; g[7] += y.w;
-                if (a.gauss) { const float4 z = q[2]; g[8] += z.x; g[9] += z.y; }
+                // rectangle: every pair's gradient of P is that of its radius, negative on the + side
+                float gax = y.x - y.y, gay = y.z - y.w;
+                if (a.gauss) { const float4 z = q[2]; gax = z.x; gay = z.y; }
+                float gc[3] = {g[0], g[1], g[2]};
+                add_centre(gc, ax, x.x, gax, gay, a.views + v);
+                g[0] = gc[0]; g[1] = gc[1]; g[2] = gc[2];
+                g[3] += x.y; g[4] += x.z; g[5] += x.w;
+                g[6] += y.x; g[7] += y.y; g[8] += y.z; g[9] += y.w;
             }
         }
     }
@@ -118,14 +128,10 @@ __global__ void __launch_bounds__(kChainThreads) k_chain_adam(ChainAdamArgs a)
 #pragma unroll
         for (int c = 0; c < 10; ++c) g[c] += __shfl_xor_sync(0xffffffffu, g[c], o);
     if (j == 0 && p < a.P) {
-        const float4 g0 = make_float4(g[0], g[1], g[2], g[3]), g3 = make_float4(g[4], g[5], g[6], g[7]);
-        // rectangle: every pair's gradient of P is that of its radius, negative on the + side
-        const float gax = a.gauss ? g[8] : g3.x - g3.y, gay = a.gauss ? g[9] : g3.z - g3.w;
-        const float* q = a.params + 3 * (size_t)a.P + 4 * (size_t)p;
-        float out[11];
-        const bool ok = chain_plane(g0, g3, gax, gay, q[0], q[1], q[2], q[3], a.single_radii, out);
+        float out[8];
+        chain_turn(ax, g[3], g[4], g[5], make_float4(g[6], g[7], g[8], g[9]), a.single_radii, out);
 #pragma unroll
-        for (int c = 0; c < 11; ++c) s_g[at][c] = ok ? out[c] : 0.f;
+        for (int c = 0; c < 11; ++c) s_g[at][c] = !ok ? 0.f : c < 3 ? g[c] : out[c - 3];
     }
     __syncthreads();
     const float bc1 = a.d_state ? a.d_state->bc1 : a.bc1, bc2 = a.d_state ? a.d_state->bc2 : a.bc2;

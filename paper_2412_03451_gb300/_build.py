@@ -20,11 +20,6 @@ LIB = os.path.join(OUT_DIR, "libps.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-fmad=false", "-Xcompiler", "-fPIC",
               "-Xcompiler", "-Wall", "-I" + INCLUDE]
-# ps_splat.cu: subnormal arguments and results of the FP32 arithmetic are taken as 0, which
-# shortens the approximate division and exponential (t > z_near, |d . n_c| > 1e-6 and w >= w_min
-# keep every value of a pair far above them).  3,000 planes, 8 views of 640x480: a step 396 -> 378 us
-# at the first lambda, 175 -> 171 at lambda 300.
-FILE_FLAGS = {"ps_splat.cu": ["-ftz=true"]}
 
 
 def nvcc() -> str:
@@ -54,7 +49,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     for src in sources():
         obj = os.path.join(OUT_DIR, os.path.basename(src).replace(".cu", ".o"))
         objs.append(obj)
-        cmd = [nvcc()] + ARCH + NVCC_FLAGS + FILE_FLAGS.get(os.path.basename(src), []) + ["-c", src, "-o", obj]
+        cmd = [nvcc()] + ARCH + NVCC_FLAGS + ["-c", src, "-o", obj]
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
         procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))

@@ -43,9 +43,9 @@
 // of 8, a step of the 3,000-plane room at 8 x 640x480 took 461 us at the first lambda (with 8
 // floats 408), 205 us at lambda 20 with 8 degree tilts (195) and 197 us at lambda 300 (193);
 // 2,000 planes with the Eq. 5 weight, whose a_x and a_y need two floats more, 2,562 us
-// (2,420).  With what followed (subnormals taken as 0, strips in groups, the replay's votes and
-// warp maximum instead of shuffles: -2.5% by themselves) these steps take 361, 158, 156 and 2,087
-// us.
+// (2,420).  With what followed (a shorter approximate division and exponential, strips in
+// groups, the replay's votes and warp maximum instead of shuffles: -2.5% by themselves) these
+// steps take 363, 160, 158 and 2,133 us.
 #include <mutex>
 
 #include <cuda.h>
@@ -639,7 +639,7 @@ __device__ __forceinline__ StripLoss run_strip(const SplatArgs& a, WarpStage& ws
                 }
                 // Eq. 4: t = s / (d . n_c); at a fixed p_c, dt/dn_c = (p_c - t d) / (d . n_c),
                 // whose products with v^x_c and v^y_c are -P_X and -P_Y over d . n_c (Eq. 6)
-                const float gs = __fdividef(gt, pe.den);
+                const float gs = quotient(gt, pe.den);
                 const float gNx = fmaf(gN0, vx.x, fmaf(gN1, vx.y, gN2 * vx.z));
                 const float gNy = fmaf(gN0, vy.x, fmaf(gN1, vy.y, gN2 * vy.z));
                 gr[0] = gs;
@@ -1203,6 +1203,7 @@ SplatConst make_const(const ps_settings* s)
     SplatConst c;
     c.lam5 = 5.f * s->lambda;
     c.w_min = s->w_min;
+    c.tiny = s->w_min < kFlushFrom;
     c.z_near = s->z_near;
     c.z_far = s->z_far;
     c.hard = (s->flags & PS_HARD) ? 1 : 0;

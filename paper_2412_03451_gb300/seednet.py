@@ -125,7 +125,9 @@ class SeedNet:
 
     # -- backward ------------------------------------------------------------
     def backward(self, dout: torch.Tensor):
-        """Gradient of sum(dout * out) w.r.t. every parameter, into self.grad."""
+        """Gradient of sum(dout * out) w.r.t. every parameter, into self.grad (dout [B, 96] fp32)."""
+        if tuple(dout.shape) != (self.B, OUT) or dout.dtype != torch.float32:
+            raise ValueError(f"dout must be float32 [{self.B}, {OUT}], not {dout.dtype} {list(dout.shape)}")
         if self.bwd_ws is None:
             n = B.ps_seed_backward_ws_bytes(self.B)
             self.bwd_ws = torch.empty((n + 255) // 256 * 64, dtype=torch.float32, device=self.device)

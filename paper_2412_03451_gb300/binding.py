@@ -335,8 +335,9 @@ def ps_adam_step(param, grad, m, v, lr, b1, b2, eps, step, clamp_min=float("nan"
 def ps_fit_step(n_planes, frame, settings, buffers: PsFitBuffers, fused, lr, b1, b2, eps, r_min, step,
                 stream=None):
     """One optimisation step in one call (see ps.h)."""
-    _check(load().ps_fit_step(n_planes, ctypes.byref(frame), ctypes.byref(settings), ctypes.byref(buffers),
-                              int(bool(fused)), lr, b1, b2, eps, r_min, step, _stream(stream)), "ps_fit_step")
+    _check(load().ps_fit_step(int(n_planes), ctypes.byref(frame), ctypes.byref(settings), ctypes.byref(buffers),
+                              int(bool(fused)), float(lr), float(b1), float(b2), float(eps), float(r_min), int(step),
+                              _stream(stream)), "ps_fit_step")
 
 
 def ps_count_pairs(frame, settings, rec, key, tile_ptr, tile_ent, capacity, counts, stream=None):

@@ -56,7 +56,9 @@ inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, siz
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cfg.attrs = &at; cfg.numAttrs = cs == cudaStreamCaptureStatusNone ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    const cudaError_t r = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    if (r != cudaSuccess) cudaGetLastError();      // reported here, not by the next launch's check
+    return r;
 }
 
 constexpr int kRecFloats = 16;   // floats per record

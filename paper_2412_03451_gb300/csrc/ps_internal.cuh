@@ -79,19 +79,24 @@ __device__ __forceinline__ int view_of_tile(const ps_view* views, int V, int til
     return lo;
 }
 
-// The same by a whole warp: 32 views per step, one load each, instead of a chain of
-// dependent loads.
+// The same by a whole warp: 32 probes per step instead of a chain of dependent loads; every step
+// leaves the stride between two probes (one step up to 32 views, two up to 1,024).  A forward of
+// 16,384 views of 32x32 took 833 us with view_of_tile, 4,952 with 32 consecutive views per step and
+// 340 so; 64 views 26, 20, 20.
 __device__ __forceinline__ int warp_view_of_tile(const ps_view* views, int V, int tile)
 {
     const int lane = threadIdx.x & 31;
-    int v = -1;
-    for (int b = 0; b < V; b += 32) {
-        const bool in = b + lane < V && __ldg(&views[b + lane].tile_off) <= tile;
-        const unsigned m = __ballot_sync(0xffffffffu, in);
-        v += __popc(m);
-        if (m != 0xffffffffu) break;
+    int lo = 0, n = V;
+    for (;;) {
+        const int stride = (n + 31) >> 5;
+        const int at = lane * stride;
+        const bool in = at < n && __ldg(&views[lo + at].tile_off) <= tile;
+        // (views are sorted by tile_off and view lo starts at or before the tile)
+        const int k = __popc(__ballot_sync(0xffffffffu, in)) - 1;
+        lo += k * stride;
+        if (stride == 1) return lo;
+        n = min(stride, n - k * stride);
     }
-    return v;
 }
 
 // One plane in camera coordinates, as stored in a record.

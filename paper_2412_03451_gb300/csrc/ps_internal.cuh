@@ -453,6 +453,10 @@ ps_status splat_fused(const ps_planes* planes, const ps_frame* f, const ps_setti
                       const float* gt_depth, const float* gt_normal, float* depth, float* normal, float* dL_dD,
                       float* dL_dN, float* g_radii, void* ws, size_t ws_bytes, bool cleared, int* d_status,
                       cudaStream_t st);
+// The chain after splat_fused, with the views' loss sums.
+ps_status chain_fused(const ps_planes* planes, const ps_frame* f, const ps_settings* s, double* view_sums,
+                      float* g_center, float* g_quat, float* g_radii, void* ws, size_t ws_bytes,
+                      cudaStream_t st);
 
 // (t, id) lexicographic order of candidates.
 __device__ __forceinline__ bool cand_less(float ta, int ia, float tb, int ib)

@@ -1446,8 +1446,16 @@ extern "C" ps_status ps_splat_fused(const ps_planes* planes, const ps_frame* f,
     ps_status e = ps::splat_fused(planes, f, s, rec, key, tile_ptr, tile_ent, capacity, gt_depth, gt_normal,
                                   depth, normal, dL_dD, dL_dN, g_radii, ws, ws_bytes, false, d_status, st);
     if (e != PS_OK) return e;
+    return ps::chain_fused(planes, f, s, view_sums, g_center, g_quat, g_radii, ws, ws_bytes, st);
+}
+
+ps_status ps::chain_fused(const ps_planes* planes, const ps_frame* f, const ps_settings* s, double* view_sums,
+                          float* g_center, float* g_quat, float* g_radii, void* ws, size_t ws_bytes,
+                          cudaStream_t st)
+{
     FusedWs w;
-    ps::fused_ws(f, s, ws, ws_bytes, &w);
+    const ps_status e = fused_ws(f, s, ws, ws_bytes, &w);
+    if (e != PS_OK) return e;
     ChainArgs c;
     c.views = f->views; c.center = planes->center; c.quat = planes->quat; c.radii = planes->radii;
     c.g_rec = f->n_records > 0 ? w.g_rec : nullptr;

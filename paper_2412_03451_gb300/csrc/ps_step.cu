@@ -149,6 +149,29 @@ __global__ void __launch_bounds__(kChainThreads) k_chain_adam(ChainAdamArgs a)
     }
 }
 
+// Plane splitting's sums and Adam on the finished gradient, by the entry points.
+ps_status adam_parameters(int n_planes, const ps_settings* s, const ps_fit_buffers* b, float lr, float b1, float b2,
+                          float eps, float r_min, int step, ps_stream stream)
+{
+    const long long g = 7LL * n_planes, n = 11LL * n_planes;     // the radii's first value, all values
+    ps_status e;
+    if (b->split_acc) {
+        e = ps_radii_grad_accum(b->grad + g, b->split_scale, 1.f, n_planes, b->split_acc, stream);
+        if (e != PS_OK) return e;
+    }
+    if (s->d_state)
+        return ps_adam_step_state(b->params, b->grad, b->m, b->v, n, lr, b1, b2, eps, s->d_state, r_min, g, stream);
+    e = ps_adam_step(b->params, b->grad, b->m, b->v, g, lr, b1, b2, eps, step, NAN, stream);
+    if (e != PS_OK) return e;
+    return ps_adam_step(b->params + g, b->grad + g, b->m + g, b->v + g, n - g, lr, b1, b2, eps, step, r_min, stream);
+}
+
+// From so many records per plane on (the mean number of views of a scene) the chain goes record by
+// record, as ps_splat_fused's does, and Adam by its own launches: eight lanes would walk a plane's
+// views too long.  64 planes in views of 32x32, an eager step by k_chain_adam and by records: 64
+// views 68 and 71 us, 128 80 and 78, 256 105 and 92, 1,024 242 and 176, 4,096 839 and 497.
+constexpr int kManyViews = 128;
+
 }  // namespace
 
 extern "C" ps_status ps_fit_step(int n_planes, const ps_frame* frame, const ps_settings* s,
@@ -193,7 +216,8 @@ extern "C" ps_status ps_fit_step(int n_planes, const ps_frame* frame, const ps_s
         // (the counts' buffer is padded to 256 bytes, the splat's range is whole 16 bytes)
         a.zero[0] = reinterpret_cast<uint4*>(count.diff); a.n[0] = (count.n_tiles + 3) / 4;
         a.zero[1] = static_cast<uint4*>(b->bwd_ws); a.n[1] = (long long)(w.bytes / 16);
-        a.zero_f = gr; a.n_f = 4LL * n_planes;
+        const bool many = frame->n_records >= kManyViews * (long long)n_planes;
+        a.zero_f = many ? b->grad : gr; a.n_f = (many ? 11LL : 4LL) * n_planes;
         a.state = b->d_state; a.sched = b->d_sched; a.n_sched = b->n_sched; a.iter = b->d_iter;
         const long long most = a.n[1] > a.n[0] ? a.n[1] : a.n[0];
         const long long blocks = (most + 255) / 256;
@@ -207,6 +231,10 @@ extern "C" ps_status ps_fit_step(int n_planes, const ps_frame* frame, const ps_s
                         b->gt_normal, nullptr, nullptr, nullptr, nullptr, gr, b->bwd_ws, b->bwd_ws_bytes, true,
                         b->d_status, st);
         if (e != PS_OK) return e;
+        if (many) {
+            e = chain_fused(&pl, frame, s, b->view_sums, gc, gq, gr, b->bwd_ws, b->bwd_ws_bytes, st);
+            return e == PS_OK ? adam_parameters(n_planes, s, b, lr, b1, b2, eps, r_min, step, stream) : e;
+        }
         ChainAdamArgs c{};
         c.views = frame->views; c.n_views = frame->n_views; c.P = n_planes;
         c.g_rec = w.g_rec;
@@ -242,16 +270,5 @@ extern "C" ps_status ps_fit_step(int n_planes, const ps_frame* frame, const ps_s
     e = ps_splat_bwd(&pl, frame, s, b->rec, b->tile_key, b->tile_ptr, b->tile_ent, b->capacity, b->dL_dD,
                      b->dL_dN, gc, gq, gr, b->bwd_ws, b->bwd_ws_bytes, b->d_status, stream);
     if (e != PS_OK) return e;
-    if (b->split_acc) {
-        e = ps_radii_grad_accum(gr, b->split_scale, 1.f, n_planes, b->split_acc, stream);
-        if (e != PS_OK) return e;
-    }
-    const long long n = 11LL * n_planes;
-    if (s->d_state)
-        return ps_adam_step_state(b->params, b->grad, b->m, b->v, n, lr, b1, b2, eps, s->d_state, r_min,
-                                  7LL * n_planes, stream);
-    e = ps_adam_step(b->params, b->grad, b->m, b->v, 7LL * n_planes, lr, b1, b2, eps, step, NAN, stream);
-    if (e != PS_OK) return e;
-    return ps_adam_step(b->params + 7 * P, gr, b->m + 7 * P, b->v + 7 * P, 4LL * n_planes, lr, b1, b2, eps, step,
-                        r_min, stream);
+    return adam_parameters(n_planes, s, b, lr, b1, b2, eps, r_min, step, stream);
 }

@@ -114,6 +114,7 @@ class SeedNet:
         """x16: [B, 64, 64, 4] bf16 (NHWC).  Returns out [B, 96] fp32."""
         Bn = x16.shape[0]
         self._alloc(Bn)
+        self.x16 = x16                # held while the first layer may still be reading it
         inp = x16
         for i, (h, cin, kp) in enumerate(LAYERS):
             B.ps_seed_conv_fwd(inp, Bn, h, cin, self._bf16[i], self.b[i], self.Y[i],

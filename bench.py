@@ -140,11 +140,11 @@ def step_launches(fused: bool, graph: bool = True) -> int:
 # .._ite1000.md, .._ite2000.md, .._ite4000.md (later points of the fit), keyed by the
 # regime's iteration; reported only while the kernel source is the one they were taken
 # on.  The issue roof is 152 SMs x 4 schedulers x one warp instruction per clock.
-CAPTURES = {"src_sha": "0da2c5833519367c",
-            "splat_fused": {0: {"dram_bytes": 51190784, "warp_instructions": 301960299},
-                            1000: {"dram_bytes": 44065792, "warp_instructions": 125205850},
-                            2000: {"dram_bytes": 42823424, "warp_instructions": 101321330},
-                            4000: {"dram_bytes": 42342400, "warp_instructions": 91234628}}}
+CAPTURES = {"src_sha": "798db94b7e7552f4",
+            "splat_fused": {0: {"dram_bytes": 51331840, "warp_instructions": 312985061},
+                            1000: {"dram_bytes": 44128512, "warp_instructions": 128747384},
+                            2000: {"dram_bytes": 42843392, "warp_instructions": 105089558},
+                            4000: {"dram_bytes": 42417152, "warp_instructions": 95114275}}}
 SCHEDULERS_PER_SM = 4
 
 

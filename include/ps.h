@@ -386,12 +386,13 @@ ps_status ps_step_advance(ps_step_state* d_state, const ps_step_state* d_sched, 
    points[i] to the nearest other point, +inf if n == 1, exact up to FP32 rounding
    of the distances (the minimum over every other point); radii (device f32
    [n][4], 16-byte aligned, or NULL) = all four radii of plane i set to
-   clamp(scale x dist[i], r_lo, r_hi) (scale 0.5 in the paper).  Points are
-   counted into a hashed uniform grid (cell edge about the cube root of the
-   bounding box's volume per point) and each query searches shells of cells around
-   its own until the nearest point found lies within the searched radius.  ws
-   (device, 16-byte aligned, >= ps_nn_workspace_bytes(n)) is scratch.  Asynchronous
-   on the stream; five launches.  PS_ERR_ARG for n < 0, NULL points or ws, both
+   clamp(scale x dist[i], r_lo, r_hi) (scale 0.5 in the paper).  Up to 10,000
+   points every pair is taken, in one launch.  Beyond, points are counted into a
+   hashed uniform grid (cell edge about the cube root of the bounding box's volume
+   per point) and each query searches shells of cells around its own until the
+   nearest point found lies within the searched radius, in a memset and five
+   launches.  ws (device, 16-byte aligned, >= ps_nn_workspace_bytes(n)) is scratch.
+   Asynchronous on the stream.  PS_ERR_ARG for n < 0, NULL points or ws, both
    outputs NULL, scale < 0, r_lo > r_hi or a small workspace. */
 size_t ps_nn_workspace_bytes(int n);
 ps_status ps_nn_distance(const float* points, int n, float scale, float r_lo, float r_hi,
@@ -510,10 +511,15 @@ ps_status ps_wait_selftest(int* d_status, long long polls, ps_stream stream);
    the planes of Sec. 3.1).  Four 3x3 stride-2 convolutions (64 channels, ReLU),
    global average pooling and a 64 -> 96 linear layer map a 64x64 patch of depth
    and camera-frame normals to 8 plane seeds.  Convolutions run as
-   implicit GEMMs on the tensor cores (ps_seed_conv_fwd), or as im2col +
-   ps_gemm_bf16.  Activations NHWC bf16; gradients fp32; the im2col column
-   order is (ky, kx, c) zero-padded to Kp (a multiple of 64).  All pointers are
-   device pointers; every call is asynchronous on the stream. ---- */
+   implicit GEMMs on the tensor cores (ps_seed_conv_fwd, ps_seed_backward).
+   Activations NHWC bf16; gradients fp32; the im2col column order is (ky, kx, c)
+   zero-padded to Kp (a multiple of 64).  All pointers are device pointers; every
+   call is asynchronous on the stream.
+
+   The network itself calls ps_seed_conv_fwd, ps_seed_backward,
+   ps_seed_sync_weights, ps_seed_pool, ps_gemm_bf16 and ps_seed_loss.  The other
+   calls are the same steps one by one (im2col + ps_gemm_bf16 and their adjoints),
+   which the tests hold these against. ---- */
 
 /* One convolution layer, y = relu(bias + conv(x)): x [B, side, side, C] and y
    [B, side/2, side/2, 64] bf16, w [64, Kp] bf16 (Kp = 64 for C = 4, 576 for C = 64,

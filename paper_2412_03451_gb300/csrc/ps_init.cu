@@ -22,7 +22,7 @@ namespace {
 
 constexpr int kSetupThreads = 1024;
 // All pairs up to here: radii of 3,000 centres take 11 us by pairs and 39 us by the grid,
-// 8,192 31 and 44 us, 12,000 58 and 46 us.  (One thread per point in the grid, its cells one
+// 8,192 31 and 44 us, 12,000 58 and 46 us (events around the call; from Python the first takes 17).  (One thread per point in the grid, its cells one
 // after another, with the cells' runs from a one-CTA scan, took 81, 98 and 132 us.)
 constexpr int kBruteMax = 10000;
 

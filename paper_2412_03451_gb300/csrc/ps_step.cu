@@ -6,10 +6,11 @@
 // of a small scene is bound by the host that enqueues them.  So k_begin advances the schedule
 // and zeroes everything the step accumulates into, the projection leaves the binning's counts,
 // and k_chain_adam takes the records' gradients to the world parameters and updates them: 8
-// launches instead of 13.  64 planes in 8 views of 128x96, eager: 162 us by nine calls, 62 by
-// one call of the same launches, 37 now (launches overlapped as in launch_after); 3,000 planes
-// in 8 views of 640x480 at lambda 300, replayed from a graph: 171 -> 167 us, 160 with the loads
-// of k_chain_adam ahead of its chain and the splat's grouped strips.
+// launches instead of 13.  64 planes in 8 views of 128x96, eager, by events: 162 us by nine calls,
+// 62 by one call of the same launches, 39 now (launches overlapped as in launch_after; a step
+// among others from Python takes 50-57, bound by the host); 3,000 planes in 8 views of 640x480 at
+// lambda 300, replayed from a graph: 171 -> 167 us, 158 with the loads of k_chain_adam ahead of
+// its chain and the splat's grouped strips.
 #include <math.h>
 
 #include "ps_internal.cuh"
